@@ -4,9 +4,9 @@
 // structure factors S(k), S(k, t) (isotropic: exp(i k.r) averaged over the directions of k is
 // sin(kr)/(kr)).
 //
-// Every output element is one thread block's fixed-order sum: threads stride over the
-// summation domain in a fixed pattern and combine in a fixed shared-memory tree, so results
-// are reproducible bit for bit.  No kernel allocates memory; outputs are caller-owned device
+// Every output element is a fixed-order sum of one thread block or one or two clusters of
+// blocks: threads stride over the summation domain in a fixed pattern and combine in a fixed
+// tree, so results are reproducible bit for bit.  No kernel allocates memory; outputs are caller-owned device
 // arrays.  All arithmetic is FP64.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -34,6 +34,29 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double (*sh)[kThreads
   }
 #pragma unroll
   for (int q = 0; q < NV; ++q) v[q] = sh[q][0];
+}
+
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_blocks() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the double at the same shared-memory location in block `rank` of the cluster
+__device__ __forceinline__ double cluster_load(const double* p, unsigned rank) {
+  unsigned a, b;
+  double v;
+  a = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(b) : "memory");
+  return v;
 }
 
 __device__ __forceinline__ void centre(const double* __restrict__ f, int N, double c[3]) {
@@ -118,76 +141,307 @@ __global__ void __launch_bounds__(kThreads) k_rouse_corr(const double* __restric
   if (threadIdx.x == 0) c[(size_t)p * nlag + lag] = norig > 0 ? v[0] / norig : 0.0;
 }
 
-__device__ __forceinline__ double sinc_kr(double k, double r2) {
-  const double x = k * sqrt(r2);
-  return x == 0.0 ? 1.0 : sin(x) / x;
-}
+// ---------------------------------------------------------------------------------------
+// structure factors and hydrodynamic radius
+//
+// These sums are bound by the FP64 pipe (2 fused multiply-adds per clock and SM: a warp's
+// instruction holds it for 16 clocks), so a pair costs what its FP64 operations cost and
+// index arithmetic, conversions by integer operations and table lookups in shared memory are
+// nearly free beside them.  Measured at T = 1000, N = 128 (before: one block per output, sqrt,
+// sine and division per pair and wave number): S(k) at 16 wave numbers 144.0 -> 6.5 ms, S(k, t) at
+// 4 wave numbers and 101 lags 29.1 -> 11.4 ms (83 % of the FP64 pipe's cycles), <1/R_H> 70.4 ->
+// 0.86 ms.  A pair takes its distance once for a group of wave numbers (14
+// operations: difference, square, 1/r, r) and 14 operations per wave number:
+//   sum of sin(k r)/(k r) = (1/k) sum of sin(k r) (1/r),
+// the sine from a table of 1024 angles and short polynomials.
+//
+// Every output is the sum of one cluster of blocks, or of two: each thread walks its pairs in a
+// fixed order, each block adds its threads in a fixed tree, and block 0 of the cluster adds the
+// blocks in rank order through distributed shared memory.  Two clusters add their sums to the
+// zeroed output atomically (0 + a + b in either order is the same number).  So results are
+// reproducible and no scratch memory is needed.
+// ---------------------------------------------------------------------------------------
 
-// one block per k: pairs i < j of every frame (the sum is symmetric; the N diagonal terms
-// are 1 each); the threads walk all ordered pairs and skip i >= j
-__global__ void __launch_bounds__(kThreads) k_static_sk(const double* __restrict__ traj, int T, int N,
-                                                        const double* __restrict__ ks, double* __restrict__ S) {
-  __shared__ double sh[1][kThreads];
-  const double k = ks[blockIdx.x];
-  const long long nn = (long long)N * N;
-  const long long total = nn * T;
-  double v[1] = {0};
-  for (long long u = threadIdx.x; u < total; u += kThreads) {
-    const int t = (int)(u / nn);
-    const int r = (int)(u - (long long)t * nn);
-    const int i = r / N, j = r - (r / N) * N;
-    if (i >= j) continue;
-    const double* f = traj + (size_t)t * N * 3;
-    const double dx = f[3 * i] - f[3 * j], dy = f[3 * i + 1] - f[3 * j + 1], dz = f[3 * i + 2] - f[3 * j + 2];
-    v[0] += sinc_kr(k, dx * dx + dy * dy + dz * dz);
+// sin and cos of 2 pi n / 1024 for n = 0 .. 511 (n + 512: the negatives)
+constexpr int kAngles = 1024;
+struct SinTab {
+  double2 a[kAngles / 2];  // (sin, cos)
+};
+
+// Fill the table with a block of at least 48 threads: 32 coarse and 16 fine angles by
+// sincospi, the products by angle addition (four operations per entry instead of a sincospi).
+// Ends with a barrier.
+__device__ __forceinline__ void fill_sin_table(SinTab* tab, double2* seed /* 48 */) {
+  const int t = threadIdx.x;
+  if (t < 48) {
+    double s, c;
+    sincospi(t < 32 ? (double)t / 32.0 : (double)(t - 32) / 512.0, &s, &c);
+    seed[t] = make_double2(s, c);
   }
-  block_sum<1>(v, sh);
-  if (threadIdx.x == 0) S[blockIdx.x] = ((double)N * T + 2.0 * v[0]) / ((double)N * T);
+  __syncthreads();
+  for (int n = t; n < kAngles / 2; n += blockDim.x) {
+    const double2 A = seed[n >> 4], B = seed[32 + (n & 15)];
+    tab->a[n] = make_double2(fma(A.x, B.y, A.y * B.x), fma(A.y, B.y, -(A.x * B.x)));
+  }
+  __syncthreads();
 }
 
-// one block per (k, lag): all ordered pairs (i, j) at the origins t0 = 0, s, 2s, ...
+// sin(2 pi p / 1024) for |p| < 2^31: p = n + f with n the nearest integer (the sum with
+// 1.5 2^52 leaves n in the low mantissa bits; f is exact), sin(n) cos(f) + cos(n) sin(f) with
+// the Taylor series of sin and cos - 1 in f (|angle| <= pi/1024: truncation below 2e-18).
+__device__ __forceinline__ double sin_turns(double p, const SinTab* __restrict__ tab) {
+  constexpr double kMagic = 6755399441055744.0;  // 1.5 2^52
+  constexpr double u = 2.0 * M_PI / kAngles;
+  const double t = p + kMagic;
+  const int n = __double2loint(t);
+  const double f = p - (t - kMagic);
+  const double2 e = tab->a[n & (kAngles / 2 - 1)];
+  const double z = f * f;
+  const double sf = f * fma(z, fma(z, u * u * u * u * u / 120.0, -(u * u * u) / 6.0), u);
+  const double cf = z * fma(z, u * u * u * u / 24.0, -(u * u) / 2.0);
+  const double v = e.x + fma(e.x, cf, e.y * sf);
+  return __hiloint2double(__double2hiint(v) ^ (int)(((unsigned)n << 22) & 0x80000000u), __double2loint(v));
+}
+
+// 1/sqrt(x) for x in [2^-100, 2^100) (rsqrt_range): the single-precision reciprocal square root of x
+// truncated to single precision (rounding and truncation by integer operations: |e| < 1e-6
+// below) and one third-order step y (1 + e/2 + 3 e^2/8), e = 1 - x y^2 (next term below 4e-19).
+__device__ __forceinline__ double rsqrt_pos(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned bits = ((unsigned)(hi - (896 << 20)) << 3) | ((unsigned)__double2loint(x) >> 29);
+  const unsigned yb = __float_as_uint(rsqrtf(__uint_as_float(bits)));
+  const double y = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+constexpr int kRangeLo = (1023 - 100) << 20, kRangeHi = (1023 + 100) << 20;  // high words of the range
+__device__ __forceinline__ bool rsqrt_range(double x) {  // also false for NaN and negative x
+  return (unsigned)(__double2hiint(x) - kRangeLo) < (unsigned)(kRangeHi - kRangeLo);
+}
+
+constexpr int kKGroup = 4;           // most wave numbers of one pass over the pairs
+constexpr double kFastArg = 1.0e6;   // largest k r of the table path
+
+// sin(k r)/(k r) as k times the sum needs it: sin(k r)/r, general arguments
+__device__ __noinline__ double sinc_general(double k, double r2) {
+  const double x = k * sqrt(r2);
+  return x == 0.0 ? k : sin(x) / x * k;
+}
+
+// Wave numbers g0 .. g0 + KG - 1 (the last group repeats the last one) and the squared distances
+// [2^-100, r2_end) that take the table path for all of them, as a span of high words: compared
+// by integer operations (a comparison in FP64 would cost as much as any other operation).
+template <int KG>
+struct WaveNumbers {
+  double k[KG], kt[KG];
+  unsigned span;
+  __device__ __forceinline__ WaveNumbers(const double* __restrict__ ks, int nk, int g0) {
+    double kmax = 0.0;
+#pragma unroll
+    for (int g = 0; g < KG; ++g) {
+      k[g] = ks[g0 + g < nk ? g0 + g : nk - 1];
+      kt[g] = k[g] * (kAngles / (2.0 * M_PI));
+      kmax = fabs(k[g]) > 0.0 ? fmax(kmax, fabs(k[g])) : INFINITY;  // k = 0 and NaN: the general path
+    }
+    const double rmax = kFastArg / kmax;
+    const int end = __double2hiint(rmax * rmax);
+    span = end <= kRangeLo ? 0u : (unsigned)((end < kRangeHi ? end : kRangeHi) - kRangeLo);
+  }
+};
+
+// acc[g] += sin(k_g r)/r of one pair at squared distance r2 (k_g where k_g r = 0)
+template <int KG>
+__device__ __forceinline__ void add_pair(double r2, const WaveNumbers<KG>& w, const SinTab* __restrict__ tab,
+                                         double (&acc)[KG]) {
+  if ((unsigned)(__double2hiint(r2) - kRangeLo) < w.span) {
+    const double y = rsqrt_pos(r2);
+    const double s = r2 * y;
+    const double r = fma(0.5 * y, fma(-s, s, r2), s);
+#pragma unroll
+    for (int g = 0; g < KG; ++g) acc[g] = fma(sin_turns(w.kt[g] * r, tab), y, acc[g]);
+  } else {
+#pragma unroll
+    for (int g = 0; g < KG; ++g) acc[g] += sinc_general(w.k[g], r2);
+  }
+}
+
+// sum of v over the threads of every block of the cluster, in a fixed order; the result in
+// thread 0 of block 0.  Every thread of every block calls it once; no block returns before
+// block 0 has read its sums.
+template <int NV>
+__device__ __forceinline__ void cluster_sum(double (&v)[NV], double* warp_sums /* NV x 32 */, double* block_sums /* NV */) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+    if (lane == 0) warp_sums[q * 32 + warp] = v[q];
+  }
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      double s = lane < nw ? warp_sums[q * 32 + lane] : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+      if (lane == 0) block_sums[q] = s;
+    }
+  }
+  cluster_barrier();
+  if (cluster_rank() == 0 && threadIdx.x == 0) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      v[q] = 0.0;
+      for (unsigned b = 0; b < cluster_blocks(); ++b) v[q] += cluster_load(block_sums + q, b);
+    }
+  }
+  cluster_barrier();
+}
+
+// The pairs i < j of a frame as q = 0 .. N (N - 1)/2 - 1: j = i + d mod N with d = q / N + 1
+// and i = q mod N (the last d of an even N has N/2 of them), so that consecutive q read
+// consecutive beads.
+__device__ __forceinline__ double pair_r2(const double* __restrict__ f, int N, unsigned q) {
+  const unsigned d = q / (unsigned)N + 1, i = q % (unsigned)N;
+  const unsigned j = i + d < (unsigned)N ? i + d : i + d - (unsigned)N;
+  const double dx = f[3 * i] - f[3 * j], dy = f[3 * i + 1] - f[3 * j + 1], dz = f[3 * i + 2] - f[3 * j + 2];
+  return fma(dx, dx, fma(dy, dy, dz * dz));
+}
+
+// Walk the pairs of all frames, thread by thread of the two clusters `half` = 0, 1: f(r2) for each.
+template <class F>
+__device__ __forceinline__ void walk_pairs(const double* __restrict__ traj, int T, int N, unsigned half, F&& f) {
+  const unsigned np = (unsigned)N * (unsigned)(N - 1) / 2;
+  const unsigned nt = 2 * cluster_blocks() * blockDim.x;
+  unsigned q = (half * cluster_blocks() + cluster_rank()) * blockDim.x + threadIdx.x;
+  const double* fr = traj;
+  for (int t = 0; t < T; ++t, fr += 3 * (size_t)N) {
+    for (; q < np; q += nt) f(pair_r2(fr, N, q));
+    q -= np;  // the walk goes on in the next frame where it would have
+  }
+}
+
+// Two clusters per group of KG wave numbers; S zeroed
+template <int KG>
+__global__ void __launch_bounds__(kThreads) k_static_sk(const double* __restrict__ traj, int T, int N,
+                                                        const double* __restrict__ ks, int nk, double* __restrict__ S) {
+  __shared__ SinTab tab;
+  __shared__ double2 seed[48];
+  __shared__ double ws[KG * 32], bs[KG];
+  fill_sin_table(&tab, seed);
+  const unsigned half = blockIdx.x / cluster_blocks() & 1;
+  const int g0 = (int)(blockIdx.x / cluster_blocks() / 2) * KG;
+  const WaveNumbers<KG> w(ks, nk, g0);
+  double acc[KG] = {};
+  walk_pairs(traj, T, N, half, [&](double r2) { add_pair<KG>(r2, w, &tab, acc); });
+  cluster_sum<KG>(acc, ws, bs);
+  if (cluster_rank() == 0 && threadIdx.x == 0) {
+#pragma unroll
+    for (int g = 0; g < KG; ++g)
+      if (g0 + g < nk) {
+        // the N diagonal terms of every frame and each pair twice, over N T
+        const double pairs = w.k[g] == 0.0 ? 0.25 * (double)N * (N - 1) * T : acc[g] / w.k[g];
+        atomicAdd(S + g0 + g, (half ? 0.0 : 1.0) + 2.0 * pairs / ((double)N * T));
+      }
+  }
+}
+
+// One cluster per lag (blockIdx.y) and group of KG wave numbers: all ordered pairs (i, j) at the
+// origins t0 = 0, s, 2s, ...
+template <int KG>
 __global__ void __launch_bounds__(kThreads) k_dynamic_sk(const double* __restrict__ traj, int T, int N,
-                                                         const double* __restrict__ ks, int stride,
+                                                         const double* __restrict__ ks, int nk, int stride,
                                                          double* __restrict__ S, int nlag) {
-  __shared__ double sh[1][kThreads];
-  const double k = ks[blockIdx.x];
+  __shared__ SinTab tab;
+  __shared__ double2 seed[48];
+  __shared__ double ws[KG * 32], bs[KG];
+  fill_sin_table(&tab, seed);
+  const int g0 = (int)(blockIdx.x / cluster_blocks()) * KG;
   const int lag = blockIdx.y;
   const int norig = T - lag > 0 ? (T - lag + stride - 1) / stride : 0;
-  const long long nn = (long long)N * N;
-  const long long total = nn * norig;
-  double v[1] = {0};
-  for (long long u = threadIdx.x; u < total; u += kThreads) {
-    const int o = (int)(u / nn);
-    const int r = (int)(u - (long long)o * nn);
-    const int i = r / N, j = r - (r / N) * N;
-    const int t0 = o * stride;
-    const double* fa = traj + (size_t)t0 * N * 3;
-    const double* fb = traj + (size_t)(t0 + lag) * N * 3;
-    const double dx = fb[3 * i] - fa[3 * j], dy = fb[3 * i + 1] - fa[3 * j + 1], dz = fb[3 * i + 2] - fa[3 * j + 2];
-    v[0] += sinc_kr(k, dx * dx + dy * dy + dz * dz);
+  const WaveNumbers<KG> w(ks, nk, g0);
+  double acc[KG] = {};
+  const unsigned nn = (unsigned)N * (unsigned)N, nt = cluster_blocks() * blockDim.x;
+  unsigned q = cluster_rank() * blockDim.x + threadIdx.x;
+  const double* fa = traj;
+  const double* fb = traj + (size_t)lag * N * 3;
+  for (int o = 0; o < norig; ++o, fa += 3 * (size_t)N * stride, fb += 3 * (size_t)N * stride) {
+    for (; q < nn; q += nt) {
+      const unsigned i = q / (unsigned)N, j = q % (unsigned)N;
+      const double dx = fb[3 * i] - fa[3 * j], dy = fb[3 * i + 1] - fa[3 * j + 1], dz = fb[3 * i + 2] - fa[3 * j + 2];
+      add_pair<KG>(fma(dx, dx, fma(dy, dy, dz * dz)), w, &tab, acc);
+    }
+    q -= nn;
   }
-  block_sum<1>(v, sh);
-  if (threadIdx.x == 0) S[(size_t)blockIdx.x * nlag + lag] = norig > 0 ? v[0] / ((double)N * norig) : 0.0;
+  cluster_sum<KG>(acc, ws, bs);
+  if (cluster_rank() == 0 && threadIdx.x == 0) {
+#pragma unroll
+    for (int g = 0; g < KG; ++g)
+      if (g0 + g < nk) {
+        const double pairs = w.k[g] == 0.0 ? (double)nn * norig : acc[g] / w.k[g];
+        S[(size_t)(g0 + g) * nlag + lag] = norig > 0 ? pairs / ((double)N * norig) : 0.0;
+      }
+  }
 }
 
-// one block: 1/r_ij over the pairs i < j of every frame
-__global__ void __launch_bounds__(kThreads) k_inverse_radius(const double* __restrict__ traj, int T, int N,
-                                                             double* __restrict__ out) {
-  __shared__ double sh[1][kThreads];
-  const long long nn = (long long)N * N;
-  const long long total = nn * T;
-  double v[1] = {0};
-  for (long long u = threadIdx.x; u < total; u += kThreads) {
-    const int t = (int)(u / nn);
-    const int r = (int)(u - (long long)t * nn);
-    const int i = r / N, j = r - (r / N) * N;
-    if (i >= j) continue;
-    const double* f = traj + (size_t)t * N * 3;
-    const double dx = f[3 * i] - f[3 * j], dy = f[3 * i + 1] - f[3 * j + 1], dz = f[3 * i + 2] - f[3 * j + 2];
-    v[0] += 1.0 / sqrt(dx * dx + dy * dy + dz * dz);
+// two clusters: 1/r_ij over the pairs i < j of every frame; out zeroed
+__global__ void __launch_bounds__(2 * kThreads) k_inverse_radius(const double* __restrict__ traj, int T, int N,
+                                                                 double* __restrict__ out) {
+  __shared__ double ws[32], bs[1];
+  double acc[1] = {0.0};
+  walk_pairs(traj, T, N, blockIdx.x / cluster_blocks(),
+             [&](double r2) { acc[0] += rsqrt_range(r2) ? rsqrt_pos(r2) : 1.0 / sqrt(r2); });
+  cluster_sum<1>(acc, ws, bs);
+  if (cluster_rank() == 0 && threadIdx.x == 0) atomicAdd(out, 2.0 * acc[0] / ((double)N * N * T));
+}
+
+// Dynamic shared memory that keeps a second block off the SM: a cluster's blocks are otherwise
+// placed two or three to an SM while other SMs idle, and these kernels fill an SM's FP64 pipe
+// with one block.
+constexpr size_t kOnePerSM = 116 * 1024;
+// Clusters of each size that fit the chip at one block per SM (cudaOccupancyMaxActiveClusters on a
+// GB300: 152 SMs, whose groups do not hold a whole number of larger clusters)
+struct ClusterFit {
+  int size, fit;
+};
+constexpr ClusterFit kClusterFit[] = {{16, 7}, {10, 13}, {9, 15}, {6, 23}, {4, 36}};
+template <class K>
+bool allow_shared(K* kernel, size_t bytes) {
+  if (bytes <= 40 * 1024) return true;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
+}
+
+// a launch of `grid` blocks in clusters of cs along x
+template <class... A, class... B>
+int launch_cluster(void (*kernel)(A...), dim3 grid, int threads, int cs, size_t smem, cudaStream_t s, B... args) {
+  if (!allow_shared(kernel, smem)) return LB_ERR_CUDA;
+  if (cs > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return LB_ERR_CUDA;
   }
-  block_sum<1>(v, sh);
-  if (threadIdx.x == 0) out[0] = 2.0 * v[0] / ((double)N * N * T);
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = dim3(threads);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&lc, kernel, (A)args...);
+  return e == cudaSuccess ? LB_OK : (e == cudaErrorMemoryAllocation ? LB_ERR_OOM : LB_ERR_CUDA);
+}
+
+// Blocks per cluster for `items` pairs per cluster, at most `most`: no more than leave each thread
+// eight pairs.
+int cluster_for(unsigned long long items, int threads, int most) {
+  const unsigned long long by_work = items / (8ull * threads);
+  return by_work < 1 ? 1 : (by_work < (unsigned long long)most ? (int)by_work : most);
 }
 
 int launch_status() {
@@ -220,23 +474,52 @@ int lb_analysis_rouse_correlation(const double* X, int T, int P, int max_lag, do
 
 int lb_analysis_static_sk(const double* traj, int T, int N, const double* k, int nk, double* S, void* stream) {
   if (!traj || !k || !S || T < 1 || N < 1 || nk < 1) return LB_ERR_ARG;
-  k_static_sk<<<nk, kThreads, 0, (cudaStream_t)stream>>>(traj, T, N, k, S);
-  return launch_status();
+  // A group of KG wave numbers runs on two clusters and a pair costs 1 + KG units there (its
+  // distance, and each sine): the KG and cluster size with the shortest time, all clusters in one
+  // wave where possible.  16 wave numbers: groups of 3 on 12 clusters of 10 (6.8 ms at T = 1000,
+  // N = 128; groups of 2 on 16 clusters of 8, two waves, 11.5 ms; one block per wave number 144 ms).
+  int kg = 1, cs = 1;
+  double best = 1e30;
+  for (int g = 1; g <= kKGroup; ++g)
+    for (const ClusterFit& f : kClusterFit) {
+      const int clusters = 2 * ((nk + g - 1) / g), waves = (clusters + f.fit - 1) / f.fit;
+      const double t = (double)waves * (1 + g) / f.size;
+      if (t < best) {
+        best = t;
+        kg = g;
+        cs = f.size;
+      }
+    }
+  cs = cluster_for((unsigned long long)N * (N - 1) / 4 * T, kThreads, cs);
+  const size_t apart = cs > 1 ? kOnePerSM : 0;
+  const dim3 grid((nk + kg - 1) / kg * 2 * cs);
+  const cudaStream_t s = (cudaStream_t)stream;
+  if (cudaMemsetAsync(S, 0, nk * sizeof(double), s) != cudaSuccess) return launch_status();
+  if (kg == 1) return launch_cluster(k_static_sk<1>, grid, kThreads, cs, apart, s, traj, T, N, k, nk, S);
+  if (kg == 2) return launch_cluster(k_static_sk<2>, grid, kThreads, cs, apart, s, traj, T, N, k, nk, S);
+  if (kg == 3) return launch_cluster(k_static_sk<3>, grid, kThreads, cs, apart, s, traj, T, N, k, nk, S);
+  return launch_cluster(k_static_sk<kKGroup>, grid, kThreads, cs, apart, s, traj, T, N, k, nk, S);
 }
 
 int lb_analysis_inverse_radius(const double* traj, int T, int N, double* out, void* stream) {
   if (!traj || !out || T < 1 || N < 2) return LB_ERR_ARG;
-  k_inverse_radius<<<1, kThreads, 0, (cudaStream_t)stream>>>(traj, T, N, out);
-  return launch_status();
+  const int cs = cluster_for((unsigned long long)N * (N - 1) / 4 * T, 2 * kThreads, 16);
+  const cudaStream_t s = (cudaStream_t)stream;
+  if (cudaMemsetAsync(out, 0, sizeof(double), s) != cudaSuccess) return launch_status();
+  return launch_cluster(k_inverse_radius, dim3(2 * cs), 2 * kThreads, cs, 0, s, traj, T, N, out);
 }
 
 int lb_analysis_dynamic_sk(const double* traj, int T, int N, const double* k, int nk, int max_lag,
                            int origin_stride, double* S, void* stream) {
   if (!traj || !k || !S || T < 1 || N < 1 || nk < 1 || max_lag < 0 || max_lag > 65535 || origin_stride < 1)
     return LB_ERR_ARG;
-  k_dynamic_sk<<<dim3(nk, max_lag + 1), kThreads, 0, (cudaStream_t)stream>>>(traj, T, N, k, origin_stride, S,
-                                                                               max_lag + 1);
-  return launch_status();
+  const int cs = cluster_for((unsigned long long)N * N * ((T + origin_stride - 1) / origin_stride), kThreads, 8);
+  const dim3 grid((nk + kKGroup - 1) / kKGroup * cs, max_lag + 1);
+  const cudaStream_t s = (cudaStream_t)stream;
+  if (nk == 1) return launch_cluster(k_dynamic_sk<1>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
+  if (nk == 2) return launch_cluster(k_dynamic_sk<2>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
+  if (nk == 3) return launch_cluster(k_dynamic_sk<3>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
+  return launch_cluster(k_dynamic_sk<kKGroup>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
 }
 
 }  // extern "C"
