@@ -59,6 +59,23 @@ __device__ __forceinline__ double cluster_load(const double* p, unsigned rank) {
   return v;
 }
 
+// two neighbouring doubles (16-byte aligned) in the shared memory of block `rank`; four such loads
+// in flight together
+struct RemotePair {
+  unsigned at;  // shared::cluster address
+  __device__ __forceinline__ RemotePair(const double* p, unsigned rank) {
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  }
+};
+__device__ __forceinline__ void cluster_load4(const RemotePair (&p)[4], double2 (&v)[4]) {
+  asm volatile(
+      "ld.shared::cluster.v2.f64 {%0, %1}, [%8];\n\tld.shared::cluster.v2.f64 {%2, %3}, [%9];\n\t"
+      "ld.shared::cluster.v2.f64 {%4, %5}, [%10];\n\tld.shared::cluster.v2.f64 {%6, %7}, [%11];"
+      : "=d"(v[0].x), "=d"(v[0].y), "=d"(v[1].x), "=d"(v[1].y), "=d"(v[2].x), "=d"(v[2].y), "=d"(v[3].x), "=d"(v[3].y)
+      : "r"(p[0].at), "r"(p[1].at), "r"(p[2].at), "r"(p[3].at)
+      : "memory");
+}
+
 __device__ __forceinline__ void centre(const double* __restrict__ f, int N, double c[3]) {
   double s0 = 0, s1 = 0, s2 = 0;
   for (int n = 0; n < N; ++n) {
@@ -71,7 +88,124 @@ __device__ __forceinline__ void centre(const double* __restrict__ f, int N, doub
   c[2] = s2 / N;
 }
 
-// one block per lag: origins t0 strided over the threads
+// g1, g2, g3 of one origin pair: frames a and b with centres ca, cb
+__device__ __forceinline__ void add_displacements(const double* ca, const double* cb, const double* a0,
+                                                  const double* b0, const double* a1, const double* b1, double v[3]) {
+  double dcm[3], s3 = 0;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    dcm[q] = cb[q] - ca[q];
+    s3 += dcm[q] * dcm[q];
+  }
+  v[2] += s3;
+  double s1 = 0, s2 = 0;
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const double *fa = w ? a1 : a0, *fb = w ? b1 : b0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const double d = fb[q] - fa[q];
+      s1 += d * d;
+      const double dr = d - dcm[q];
+      s2 += dr * dr;
+    }
+  }
+  v[0] += s1;
+  v[1] += s2;
+}
+
+__device__ __forceinline__ void write_msd(const double v[3], int norig, int lag, int nlag, double* out) {
+  const bool any = norig > 0;
+  out[lag] = any ? v[0] / (2.0 * norig) : 0.0;
+  out[nlag + lag] = any ? v[1] / (2.0 * norig) : 0.0;
+  out[2 * nlag + lag] = any ? v[2] / norig : 0.0;
+}
+
+// The whole run staged in shared memory (kMsdFrames frames at most): a cluster of blocks forms the
+// centres of mass once, a warp per frame, each block a share of the frames, and every block
+// takes the full series of the centre and the two inner beads (9 doubles per frame) from its
+// peers through distributed shared memory.  Then the cluster's lags, one after the other per
+// block, origins strided over the threads.  At T = 1000, N = 128, 501 lags 115 us
+// (k_msd below, two centres of N beads for every lag and origin with frame-strided reads: 1233 us;
+// 19 clusters instead of the 15 that fit at a time: 184 us).
+constexpr int kMsdFrames = 3000;
+constexpr int kMsdCluster = 8;
+constexpr int kMsdThreads = 512;
+__global__ void __launch_bounds__(kMsdThreads) k_msd_staged(const double* __restrict__ traj, int T, int N, int i0, int i1,
+                                                         double* __restrict__ out, int nlag, int nclusters) {
+  extern __shared__ __align__(16) double series[];  // [T][9]: centre, bead i0, bead i1
+  __shared__ double ws[3][kMsdThreads / 32];
+  const int rank = (int)cluster_rank(), G = (int)cluster_blocks();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = ((T + G - 1) / G + 1) & ~1;  // frames of a block, an even number
+  const int f0 = rank * per < T ? rank * per : T, f1 = f0 + per < T ? f0 + per : T;
+  for (int t = f0 + warp; t < f1; t += kMsdThreads / 32) {
+    const double* f = traj + (size_t)t * N * 3;
+    double s[3] = {0, 0, 0};  // s[j]: elements lane + 32 j + 96 m, component (lane + 2 j) mod 3
+    for (int e = lane; e < 3 * N; e += 96) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (e + 32 * j < 3 * N) s[j] += f[e + 32 * j];
+    }
+    double c[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int j = (2 * q + lane) % 3;  // (lane + 2 j) mod 3 = q for j = 2 (q - lane) = 2 q + lane mod 3
+      c[q] = j == 0 ? s[0] : (j == 1 ? s[1] : s[2]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) c[q] += __shfl_xor_sync(0xffffffffu, c[q], o);
+    }
+    if (lane < 9) {
+      const int q = lane % 3;
+      series[9 * t + lane] = lane < 3 ? (q == 0 ? c[0] : (q == 1 ? c[1] : c[2])) / N : f[3 * (lane < 6 ? i0 : i1) + q];
+    }
+  }
+  cluster_barrier();
+  // pairs of doubles, a block's share a whole number of them (`per` is even)
+  const int npair = (9 * T + 1) / 2;
+  for (int e0 = threadIdx.x; e0 < npair; e0 += 4 * kMsdThreads) {
+    const int last = npair - 1;
+    const int e[4] = {e0, min(e0 + kMsdThreads, last), min(e0 + 2 * kMsdThreads, last), min(e0 + 3 * kMsdThreads, last)};
+    int owner[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) owner[j] = 2 * e[j] / 9 / per;
+    const RemotePair from[4] = {{series + 2 * e[0], (unsigned)owner[0]}, {series + 2 * e[1], (unsigned)owner[1]},
+                                {series + 2 * e[2], (unsigned)owner[2]}, {series + 2 * e[3], (unsigned)owner[3]}};
+    double2 v[4];
+    cluster_load4(from, v);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (owner[j] != rank) reinterpret_cast<double2*>(series)[e[j]] = v[j];
+  }
+  cluster_barrier();  // every share has been read; also the block's barrier
+  for (int lag = (int)(blockIdx.x / G) + nclusters * rank; lag < nlag; lag += nclusters * G) {
+    const int norig = T - lag;
+    double v[3] = {0, 0, 0};
+    for (int t0 = threadIdx.x; t0 < norig; t0 += kMsdThreads) {
+      const double *a = series + 9 * t0, *b = a + 9 * lag;
+      add_displacements(a, b, a + 3, b + 3, a + 6, b + 6, v);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+      if (lane == 0) ws[q][warp] = v[q];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        v[q] = 0.0;
+        for (int w = 0; w < kMsdThreads / 32; ++w) v[q] += ws[q][w];
+      }
+      write_msd(v, norig, lag, nlag, out);
+    }
+    __syncthreads();
+  }
+}
+
+// Longer runs: one block per lag, origins t0 strided over the threads, the centres of both frames
+// formed by each thread
 __global__ void __launch_bounds__(kThreads) k_msd(const double* __restrict__ traj, int T, int N, int i0, int i1,
                                                   double* __restrict__ out, int nlag) {
   __shared__ double sh[3][kThreads];
@@ -84,37 +218,59 @@ __global__ void __launch_bounds__(kThreads) k_msd(const double* __restrict__ tra
     double ca[3], cb[3];
     centre(fa, N, ca);
     centre(fb, N, cb);
-    double dcm[3], s3 = 0;
-    for (int q = 0; q < 3; ++q) {
-      dcm[q] = cb[q] - ca[q];
-      s3 += dcm[q] * dcm[q];
-    }
-    v[2] += s3;
-    for (int w = 0; w < 2; ++w) {
-      const int i = w ? i1 : i0;
-      double s1 = 0, s2 = 0;
-      for (int q = 0; q < 3; ++q) {
-        const double d = fb[3 * i + q] - fa[3 * i + q];
-        s1 += d * d;
-        const double dr = d - dcm[q];
-        s2 += dr * dr;
-      }
-      v[0] += s1;
-      v[1] += s2;
-    }
+    add_displacements(ca, cb, fa + 3 * i0, fb + 3 * i0, fa + 3 * i1, fb + 3 * i1, v);
   }
   block_sum<3>(v, sh);
-  if (threadIdx.x == 0) {
-    const bool any = norig > 0;
-    out[lag] = any ? v[0] / (2.0 * norig) : 0.0;
-    out[nlag + lag] = any ? v[1] / (2.0 * norig) : 0.0;
-    out[2 * nlag + lag] = any ? v[2] / norig : 0.0;
-  }
+  if (threadIdx.x == 0) write_msd(v, norig, lag, nlag, out);
 }
 
-// one block per frame; threads over (p, component); the sum over n in bead order
-__global__ void __launch_bounds__(kThreads) k_rouse_modes(const double* __restrict__ traj, int N, int P,
+// Rouse modes: X_p(t) = (1/N) sum_n r_n(t) cos(p pi (n - 1/2)/N).  The angles are multiples of
+// pi/2N, p (2n - 1) of them, so a table of 4N cosines holds every factor (one cospi each).  66 us
+// at T = 1000, N = 128; one cospi per term took 3045 us.  The terms n and N + 1 - n
+// have the same factor up to (-1)^p: even modes take the sums of the two beads, odd modes the
+// differences, which halves the FP64 operations.  A block takes kRouseFrames frames, a thread
+// a mode p of one frame after the other, its three components sharing the factor.
+constexpr int kRouseFrames = 4;
+__global__ void __launch_bounds__(kThreads) k_rouse_modes(const double* __restrict__ traj, int T, int N, int P,
                                                           double* __restrict__ X) {
+  extern __shared__ __align__(16) double rsm[];
+  const int H = (N + 1) / 2;  // pairs (n, N + 1 - n), the middle bead of an odd N last
+  double* tab = rsm;          // 4N cosines of m pi / 2N
+  double* sd = tab + 4 * N;   // [frame][parity][n][3]: sums and differences
+  const int t0 = blockIdx.x * kRouseFrames, nf = T - t0 < kRouseFrames ? T - t0 : kRouseFrames;
+  for (int m = threadIdx.x; m < 4 * N; m += kThreads) tab[m] = cospi((double)m / (2.0 * (double)N));
+  for (int e = threadIdx.x; e < nf * 3 * H; e += kThreads) {
+    const int f = e / (3 * H), r = e - f * 3 * H, n = r / 3, q = r - 3 * n;
+    const double* fr = traj + (size_t)(t0 + f) * N * 3;
+    const double lo = fr[r], hi = fr[3 * (N - 1 - n) + q];
+    const bool mid = 2 * n + 1 == N;
+    sd[(2 * f) * 3 * H + r] = mid ? lo : lo + hi;
+    sd[(2 * f + 1) * 3 * H + r] = mid ? 0.0 : lo - hi;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nf * P; e += kThreads) {
+    const int f = e / P, p = e - f * P + 1;
+    const double* v = sd + (2 * f + (p & 1)) * 3 * H;
+    double s0 = 0, s1 = 0, s2 = 0;
+    int m = p;  // p (2n - 1) mod 4N
+    for (int n = 0; n < H; ++n) {
+      const double c = tab[m];
+      s0 = fma(v[3 * n], c, s0);
+      s1 = fma(v[3 * n + 1], c, s1);
+      s2 = fma(v[3 * n + 2], c, s2);
+      m += 2 * p;
+      if (m >= 4 * N) m -= 4 * N;
+    }
+    double* x = X + ((size_t)(t0 + f) * P + (p - 1)) * 3;
+    x[0] = s0 / N;
+    x[1] = s1 / N;
+    x[2] = s2 / N;
+  }
+}
+// Longer chains (the table and the frames exceed shared memory): one block per frame, one cospi per
+// term
+__global__ void __launch_bounds__(kThreads) k_rouse_modes_long(const double* __restrict__ traj, int N, int P,
+                                                               double* __restrict__ X) {
   const int t = blockIdx.x;
   const double* f = traj + (size_t)t * N * 3;
   for (int e = threadIdx.x; e < 3 * P; e += kThreads) {
@@ -125,7 +281,49 @@ __global__ void __launch_bounds__(kThreads) k_rouse_modes(const double* __restri
   }
 }
 
-// one block per (p, lag)
+// Correlation of mode p at kCorrLags lags from its series X_p(t) staged in shared memory (three
+// component planes; kCorrFrames frames at most): a warp's lanes take 32 consecutive lags, so that
+// they read consecutive words and share X_p(t0), and the block's 8 warps an eighth of the origins
+// each, added in warp order.  FP64-bound: three multiply-adds per origin and lag, 282 us at T = 1000,
+// P = 127, 501 lags (227 us of FP64 pipe; a block per (p, lag) with strided reads 642 us).
+constexpr int kCorrLags = 64;
+constexpr int kCorrFrames = 9000;
+__global__ void __launch_bounds__(kThreads) k_rouse_corr_staged(const double* __restrict__ X, int T, int P,
+                                                                double* __restrict__ c, int nlag) {
+  extern __shared__ __align__(16) double csm[];  // [3][T]
+  __shared__ double part[kThreads / 32][32];
+  const int p = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int e = threadIdx.x; e < 3 * T; e += kThreads) {
+    const int t = e / 3, q = e - 3 * t;
+    csm[q * T + t] = X[((size_t)t * P + p) * 3 + q];
+  }
+  __syncthreads();
+  const int l1 = (int)(blockIdx.y + 1) * kCorrLags < nlag ? (int)(blockIdx.y + 1) * kCorrLags : nlag;
+  for (int l0 = blockIdx.y * kCorrLags; l0 < l1; l0 += 32) {
+    const int lag = l0 + lane;
+    const int longest = T - l0;  // origins of the smallest lag; a lane beyond its own adds nothing
+    const int a = warp * longest / (kThreads / 32), b = (warp + 1) * longest / (kThreads / 32);
+    const int own = T - lag < b ? T - lag : b;
+    double s = 0.0;
+    for (int t0 = a; t0 < own; ++t0) {
+      const double* x = csm + t0;
+      s = fma(x[0], x[lag], s);
+      s = fma(x[T], x[T + lag], s);
+      s = fma(x[2 * T], x[2 * T + lag], s);
+    }
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && lag < l1) {
+      s = 0.0;
+#pragma unroll
+      for (int w = 0; w < kThreads / 32; ++w) s += part[w][lane];
+      c[(size_t)p * nlag + lag] = T - lag > 0 ? s / (T - lag) : 0.0;
+    }
+    __syncthreads();
+  }
+}
+
+// Longer runs: one block per (p, lag)
 __global__ void __launch_bounds__(kThreads) k_rouse_corr(const double* __restrict__ X, int T, int P,
                                                          double* __restrict__ c, int nlag) {
   __shared__ double sh[1][kThreads];
@@ -395,6 +593,7 @@ __global__ void __launch_bounds__(2 * kThreads) k_inverse_radius(const double* _
   if (cluster_rank() == 0 && threadIdx.x == 0) atomicAdd(out, 2.0 * acc[0] / ((double)N * N * T));
 }
 
+constexpr size_t kMaxShared = 227 * 1024;  // dynamic and static shared memory of a block
 // Dynamic shared memory that keeps a second block off the SM: a cluster's blocks are otherwise
 // placed two or three to an SM while other SMs idle, and these kernels fill an SM's FP64 pipe
 // with one block.
@@ -456,18 +655,40 @@ extern "C" {
 
 int lb_analysis_msd(const double* traj, int T, int N, int max_lag, int i0, int i1, double* out, void* stream) {
   if (!traj || !out || T < 1 || N < 1 || max_lag < 0 || i0 < 0 || i1 < 0 || i0 >= N || i1 >= N) return LB_ERR_ARG;
+  if (T <= kMsdFrames) {
+    // as many clusters as fit the chip with one block per SM (15 of 8), no more than the lags need
+    int nc = (max_lag + kMsdCluster) / kMsdCluster;
+    nc = nc < 15 ? nc : 15;
+    size_t smem = ((size_t)T * 9 + 1) * sizeof(double);
+    smem = smem < kOnePerSM ? kOnePerSM : smem;
+    return launch_cluster(k_msd_staged, dim3(nc * kMsdCluster), kMsdThreads, kMsdCluster, smem,
+                          (cudaStream_t)stream, traj, T, N, i0, i1, out, max_lag + 1, nc);
+  }
   k_msd<<<max_lag + 1, kThreads, 0, (cudaStream_t)stream>>>(traj, T, N, i0, i1, out, max_lag + 1);
   return launch_status();
 }
 
 int lb_analysis_rouse_modes(const double* traj, int T, int N, int P, double* X, void* stream) {
   if (!traj || !X || T < 1 || N < 2 || P < 1 || P > N - 1) return LB_ERR_ARG;
-  k_rouse_modes<<<T, kThreads, 0, (cudaStream_t)stream>>>(traj, N, P, X);
+  const size_t smem = (4 * (size_t)N + kRouseFrames * 6 * ((size_t)N + 1) / 2) * sizeof(double);
+  if (smem > kMaxShared) {
+    k_rouse_modes_long<<<T, kThreads, 0, (cudaStream_t)stream>>>(traj, N, P, X);
+    return launch_status();
+  }
+  if (!allow_shared(k_rouse_modes, smem)) return LB_ERR_CUDA;
+  k_rouse_modes<<<(T + kRouseFrames - 1) / kRouseFrames, kThreads, smem, (cudaStream_t)stream>>>(traj, T, N, P, X);
   return launch_status();
 }
 
 int lb_analysis_rouse_correlation(const double* X, int T, int P, int max_lag, double* c, void* stream) {
   if (!X || !c || T < 1 || P < 1 || max_lag < 0 || max_lag > 65535) return LB_ERR_ARG;
+  if (T <= kCorrFrames) {
+    const size_t smem = 3 * (size_t)T * sizeof(double);
+    if (!allow_shared(k_rouse_corr_staged, smem)) return LB_ERR_CUDA;
+    k_rouse_corr_staged<<<dim3(P, (max_lag + kCorrLags) / kCorrLags), kThreads, smem, (cudaStream_t)stream>>>(
+        X, T, P, c, max_lag + 1);
+    return launch_status();
+  }
   k_rouse_corr<<<dim3(P, max_lag + 1), kThreads, 0, (cudaStream_t)stream>>>(X, T, P, c, max_lag + 1);
   return launch_status();
 }
