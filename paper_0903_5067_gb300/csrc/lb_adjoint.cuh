@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(256) k_adj_lb(const S* __restrict__ state, con
     // a_k += ag_k sqrt(rho) g_k:  d/drho = ag_k g_k / (2 sqrt(rho))
     R acc = R(0);
     fluid_noise<R>(step, node, P.rk, P.ncalls > 1, NoiseScale<R>(R(1)),
-                   [&](int j, R g) { acc += P.ag[4 + j] * g * ab[4 + j]; });
+                   [&](int j, R g) { acc += P.ag[4 + j] * g * ab[4 + j]; }, P.tab);
     mb[0] += acc * R(0.5) / sqrt(rho);
   }
   // nbar_ps,i = sum_k e_k(c_i) mb_k, pushed to r - e_i

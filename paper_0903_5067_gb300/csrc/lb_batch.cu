@@ -39,14 +39,6 @@ struct ReplicaK {
 __global__ void k_set_step(uint32_t* d_step, uint32_t v) { *d_step = v; }
 __global__ void k_add_step(uint32_t* d_step, uint32_t v) { *d_step += v; }
 
-// n / d for n < 2^24 and 2 <= d <= 256 by one multiply-high with m = ceil(2^32 / d): with
-// e = m d - 2^32 < d, n m / 2^32 = n / d + n e / (d 2^32) and n e < 2^32 keeps the error below
-// the distance of n / d to the next integer (checked exhaustively for every d and n in range).
-__host__ __device__ __forceinline__ unsigned magic_of(unsigned d) {
-  return (unsigned)((0x100000000ull + d - 1) / d);
-}
-__device__ __forceinline__ unsigned div_magic(unsigned n, unsigned m) { return __umulhi(n, m); }
-
 // Per-replica fields of the batched LB kernel; the shared fluid parameters and up to
 // kBatchGroup replicas travel in the kernel's parameter block (constant bank), so the
 // collision's coefficients stay instruction operands as in the single-box kernel.
@@ -268,7 +260,7 @@ class BatchT final : public Batch {
   }
 
   BatchT(const std::vector<Config>& cfgs, const std::vector<std::vector<double>>& x0) : x0_(x0) {
-    for (const Config& c : cfgs) eng_.emplace_back(new EngineT<S, R, DEV>(c));
+    for (const Config& c : cfgs) eng_.emplace_back(new EngineT<S, R, DEV>(c, /*own_tables=*/false));
     size_t off = 0;
     for (auto& e : eng_) {
       off = align_up(off, 256);
@@ -284,6 +276,9 @@ class BatchT final : public Batch {
     off = align_up(off, 256);
     counters_off_ = off;
     off += 2 * (cfgs.size() / kBatchGroup + 1) * sizeof(unsigned long long);
+    off = align_up(off, 256);
+    noise_off_ = off;
+    if (sizeof(R) == 8) off += noise_table_bytes();
     off = align_up(off, 256);
     table_off_ = off;
     off += cfgs.size() * sizeof(ReplicaK<S, R>);
@@ -301,7 +296,10 @@ class BatchT final : public Batch {
 
   void bind(void* base) override {
     base_ = static_cast<unsigned char*>(base);
-    for (size_t r = 0; r < eng_.size(); ++r) eng_[r]->bind(base_ + offs_[r]);
+    for (size_t r = 0; r < eng_.size(); ++r) {
+      eng_[r]->bind(base_ + offs_[r]);
+      if (sizeof(R) == 8) eng_[r]->set_noise_tables(base_ + noise_off_);  // one for all replicas
+    }
     d_reps_ = reinterpret_cast<ReplicaK<S, R>*>(base_ + table_off_);
     flags_[0] = reinterpret_cast<unsigned*>(base_ + flags_off_);
     flags_[1] = flags_[0] + max_segs_;
@@ -310,6 +308,7 @@ class BatchT final : public Batch {
   }
 
   void initialise(cudaStream_t s) override {
+    if (sizeof(R) == 8) launch_fill_noise_tables(base_ + noise_off_, s);
     for (size_t r = 0; r < eng_.size(); ++r)
       eng_[r]->initialise(x0_[r].empty() ? nullptr : x0_[r].data(), nullptr, s);
     smem_ = 0;
@@ -564,7 +563,7 @@ class BatchT final : public Batch {
   std::vector<BatchLB<S, R>> groups_;
   std::vector<std::vector<double>> x0_;
   std::vector<size_t> offs_;
-  size_t table_off_ = 0, step_off_ = 0, flags_off_ = 0, counters_off_ = 0, bytes_ = 0, smem_ = 0;
+  size_t noise_off_ = 0, table_off_ = 0, step_off_ = 0, flags_off_ = 0, counters_off_ = 0, bytes_ = 0, smem_ = 0;
   unsigned long long* counters_ = nullptr;
   size_t max_segs_ = 0;
   unsigned* flags_[2] = {nullptr, nullptr};  // node marks by slot

@@ -120,7 +120,7 @@ struct FluidK {
   unsigned long long* nonpos;  // counter of non-positive densities met by the noise
   int pdl;         // launch chaining of the LB kernel: bit 0 waits for the previous grid before
                    // reading, bit 1 waits for it before completing (see k_lb_step)
-  int angle_tab;   // double precision: the LB kernel's Box-Muller angles from per-block tables
+  NoiseTab tab;    // double precision: the noise's radii and angles
   // null, or a device counter the step kernels add their step argument to (graph replays of a
   // fixed sequence of launches at other step numbers)
   const uint32_t* d_step;
@@ -418,8 +418,7 @@ __host__ __device__ __forceinline__ void pops_from_w2scaled(const R a[Q], R n[Q]
 // i * pl + node for population i).
 template <class R, bool DEV, bool NOISE>
 __device__ __forceinline__ void lb_collide(const R* n, R out[Q], const FluidK<R>& P, const RoundKeys& rk,
-                                           unsigned long long* nonpos, const uint32_t step, const unsigned node,
-                                           const AngleTab* tab = nullptr) {
+                                           unsigned long long* nonpos, const uint32_t step, const unsigned node) {
   // moments 0..9 (the kinetic modes relax to zero and are not needed)
   R m[10];
   moments_0_9<R>(n, m);
@@ -451,7 +450,7 @@ __device__ __forceinline__ void lb_collide(const R* n, R out[Q], const FluidK<R>
   if (NOISE) {
     if (!(rho > R(0))) atomicAdd(nonpos, 1ull);
     fluid_noise<R>(step, node, rk, P.ncalls > 1, NoiseScale<R>(rho),
-                   [&](int j, R g) { a[4 + j] += P.wag[4 + j] * g; }, tab);
+                   [&](int j, R g) { a[4 + j] += P.wag[4 + j] * g; }, P.tab);
   }
 
   if (P.body_on) {
@@ -576,9 +575,9 @@ __device__ __forceinline__ void lb_collide_pair(const f2 n[Q], f2 out[Q], const 
                    [&](int j, f2 g) { a[4 + j] = fma2(f2(P.wag[4 + j]), g, a[4 + j]); });
     } else {
       fluid_noise<float>(step, node, rk, P.ncalls > 1, NoiseScale<float>(rho.v.x),
-                         [&](int j, float g) { a[4 + j].v.x = fmaf(P.wag[4 + j], g, a[4 + j].v.x); });
+                         [&](int j, float g) { a[4 + j].v.x = fmaf(P.wag[4 + j], g, a[4 + j].v.x); }, P.tab);
       fluid_noise<float>(step, node + 1, rk, P.ncalls > 1, NoiseScale<float>(rho.v.y),
-                         [&](int j, float g) { a[4 + j].v.y = fmaf(P.wag[4 + j], g, a[4 + j].v.y); });
+                         [&](int j, float g) { a[4 + j].v.y = fmaf(P.wag[4 + j], g, a[4 + j].v.y); }, P.tab);
     }
   }
 
@@ -603,10 +602,9 @@ __device__ __forceinline__ void lb_collide_pair(const f2 n[Q], f2 out[Q], const 
 template <class S, class R, bool DEV, bool NOISE, class I>
 __device__ __forceinline__ void lb_collide_store(const R* n, S* __restrict__ dst, const FluidK<R>& P, const I pl,
                                                  const RoundKeys& rk, unsigned long long* nonpos,
-                                                 const uint32_t step, const unsigned node,
-                                                 const AngleTab* tab = nullptr) {
+                                                 const uint32_t step, const unsigned node) {
   R out[Q];
-  lb_collide<R, DEV, NOISE>(n, out, P, rk, nonpos, step, node, tab);
+  lb_collide<R, DEV, NOISE>(n, out, P, rk, nonpos, step, node);
 #pragma unroll
   for (int i = 0; i < Q; ++i) st<S, R>(dst + ((I)i * pl + (I)node), out[i]);
 }
@@ -659,36 +657,31 @@ __device__ __forceinline__ void stage_corrections(const R* __restrict__ corr, un
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// One LB tile: pull-stream + collide for the (blockDim.x x blockDim.y) nodes at (tx, ty, z)
-// (Sec. II B, Eq. 3).  Every thread loads its 19 populations and its mark word together; a
-// node marked by the previous deferred step then stages that step's corrections at its pull
-// sources (in shared memory, 19 x blockDim.x x blockDim.y values) and adds them to what it
-// pulled, and one copy of the collision follows.  (Branching on the mark before the loads put
-// an L2 round trip in front of every warp's loads, 1.4 us per launch at L = 128 with no node
-// marked; with two inlined copies of the update, a warp holding marked and unmarked nodes
-// ran both: 67.8 against 64.0 us with 1.5 % of the nodes marked.)
+// One node: pull-stream + collide (Sec. II B, Eq. 3).  Every thread loads its 19 populations and
+// its mark word together; a node marked by the previous deferred step then stages that step's
+// corrections at its pull sources (in shared memory at stage[i * T], T threads per block) and
+// adds them to what it pulled, and one copy of the collision follows.  (Branching on the mark
+// before the loads put an L2 round trip in front of every warp's loads, 1.4 us per launch at
+// L = 128 with no node marked; with two inlined copies of the update, a warp holding marked and
+// unmarked nodes ran both: 67.8 against 64.0 us with 1.5 % of the nodes marked.)
 // CORR = false (a box without a chain): no correction code at all (the dead correction path
 // alone cost 0.5 us per chained launch at L = 128).
 template <class S, class R, bool DEV, bool NOISE, class I, bool CORR>
-__device__ __forceinline__ void lb_tile(const S* __restrict__ src, S* __restrict__ dst, const FluidK<R>& P,
-                                        const PendK<R>& Pd, const uint32_t step, unsigned tx, unsigned ty,
-                                        unsigned z, R* stage, const AngleTab* tab) {
+__device__ __forceinline__ void lb_node(const S* __restrict__ src, S* __restrict__ dst, const FluidK<R>& P,
+                                        const PendK<R>& Pd, const uint32_t step, unsigned x, unsigned y, unsigned z,
+                                        R* stage, unsigned T) {
   const unsigned L = P.L;
-  const unsigned x = tx * blockDim.x + threadIdx.x;
-  const unsigned y = ty * blockDim.y + threadIdx.y;
-  if (x >= L || y >= L) return;
   const unsigned node = x + L * (y + L * z);
   const unsigned mw = CORR && Pd.have_prev ? Pd.prev_mask[Pd.seg0 + (node >> kSegShift)] : 0u;
   const I pl = (I)P.plane;
   R n[Q];
   lb_pull<S, R, I>(src, L, pl, x, y, z, n);
   if (CORR && ((mw >> (node & 31u)) & 1u)) {
-    const unsigned T = blockDim.x * blockDim.y, tid = threadIdx.x + blockDim.x * threadIdx.y;
-    stage_corrections<R>(Pd.prev_dense, Pd.plane, L, x, y, z, stage + tid, T);
+    stage_corrections<R>(Pd.prev_dense, Pd.plane, L, x, y, z, stage, T);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) n[i] += stage[tid + i * T];
+    for (int i = 0; i < Q; ++i) n[i] += stage[i * T];
   }
-  lb_collide_store<S, R, DEV, NOISE, I>(n, dst, P, pl, P.rk, P.nonpos, step, node, tab);
+  lb_collide_store<S, R, DEV, NOISE, I>(n, dst, P, pl, P.rk, P.nonpos, step, node);
 }
 
 // Collide the pulled populations n0, n1 of the nodes (node, node + 1) and store the pairs
@@ -743,36 +736,30 @@ __device__ __forceinline__ void lb_pull2(const S* __restrict__ src, const unsign
   }
 }
 
-// One LB tile with two nodes per thread along x (L even): the 2 blockDim.x x blockDim.y nodes
-// at x = 2 (tx blockDim.x + threadIdx.x) + {0, 1}, y = ty blockDim.y + threadIdx.y, z.  The
-// same update as lb_tile, node by node, with the 19 post-collision pairs written by
-// two-element stores.  Marked nodes stage their corrections one node after the other into
-// stage[tid + i * T], the same 19 T values as lb_tile.
+// Two nodes (x0, y, z) and (x0 + 1, y, z), x0 even, L even: the same update as lb_node, node by
+// node, with the 19 post-collision pairs written by two-element stores.  Marked nodes stage their
+// corrections one node after the other into the same 19 T values.
 template <class S, class R, bool DEV, bool NOISE, class I, bool CORR>
-__device__ __forceinline__ void lb_tile2(const S* __restrict__ src, S* __restrict__ dst, const FluidK<R>& P,
-                                         const PendK<R>& Pd, const uint32_t step, unsigned tx, unsigned ty,
-                                         unsigned z, R* stage) {
+__device__ __forceinline__ void lb_nodes2(const S* __restrict__ src, S* __restrict__ dst, const FluidK<R>& P,
+                                          const PendK<R>& Pd, const uint32_t step, unsigned x0, unsigned y,
+                                          unsigned z, R* stage, unsigned T) {
   const unsigned L = P.L;
-  const unsigned x0 = 2 * (tx * blockDim.x + threadIdx.x);
-  const unsigned y = ty * blockDim.y + threadIdx.y;
-  if (x0 >= L || y >= L) return;
   const unsigned node = x0 + L * (y + L * z);
   const unsigned mw = CORR && Pd.have_prev ? Pd.prev_mask[Pd.seg0 + (node >> kSegShift)] >> (node & 31u) : 0u;
   const I pl = (I)P.plane;
   R n0[Q], n1[Q];
   lb_pull2<S, R, I>(src, L, pl, x0, y, z, n0, n1);
   if (CORR && (mw & 3u)) {
-    const unsigned T = blockDim.x * blockDim.y, tid = threadIdx.x + blockDim.x * threadIdx.y;
 #pragma unroll 1
     for (unsigned j = 0; j < 2; ++j) {
       if (!((mw >> j) & 1u)) continue;
-      stage_corrections<R>(Pd.prev_dense, Pd.plane, L, x0 + j, y, z, stage + tid, T);
+      stage_corrections<R>(Pd.prev_dense, Pd.plane, L, x0 + j, y, z, stage, T);
       if (j == 0) {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) n0[i] += stage[tid + i * T];
+        for (int i = 0; i < Q; ++i) n0[i] += stage[i * T];
       } else {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) n1[i] += stage[tid + i * T];
+        for (int i = 0; i < Q; ++i) n1[i] += stage[i * T];
       }
     }
   }
@@ -802,7 +789,7 @@ struct LbMinBlocks {
   static constexpr int value = sizeof(R) == 4 ? (PAIR ? 4 : 6) : 1;
 };
 
-// PAIR: two nodes per thread along x (lb_tile2, L even), else one (lb_tile).
+// PAIR: two nodes per thread along x (lb_nodes2, L even), else one (lb_node).
 template <class S, class R, bool DEV, bool NOISE, class I, bool CORR, bool PAIR>
 __global__ void __launch_bounds__(256, LbMinBlocks<R, PAIR>::value) k_lb_step(const S* __restrict__ src, S* __restrict__ dst,
                                                   const FluidK<R> P, const PendK<R> Pd, const uint32_t step) {
@@ -815,21 +802,50 @@ __global__ void __launch_bounds__(256, LbMinBlocks<R, PAIR>::value) k_lb_step(co
   if (P.pdl & 1) grid_dependency_wait();
   allow_dependent_launch();
   const uint32_t k = launch_step(P, step);
-  const AngleTab* tab = nullptr;
-  if constexpr (sizeof(R) == 8) {
-    __shared__ AngleTab s_tab;
-    if (P.angle_tab) {  // before any thread leaves: every thread reaches the barrier
-      fill_angle_tables(&s_tab, threadIdx.x + blockDim.x * threadIdx.y);
-      __syncthreads();
-      tab = &s_tab;
-    }
+  const unsigned T = blockDim.x * blockDim.y;
+  R* const stage = reinterpret_cast<R*>(lsm) + (threadIdx.x + blockDim.x * threadIdx.y);
+  const unsigned xt = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+  if constexpr (PAIR) {
+    if (2 * xt < P.L && y < P.L)
+      lb_nodes2<S, R, DEV, NOISE, I, CORR>(src, dst, P, Pd, k, 2 * xt, y, blockIdx.z, stage, T);
+  } else {
+    if (xt < P.L && y < P.L) lb_node<S, R, DEV, NOISE, I, CORR>(src, dst, P, Pd, k, xt, y, blockIdx.z, stage, T);
   }
-  if constexpr (PAIR)
-    lb_tile2<S, R, DEV, NOISE, I, CORR>(src, dst, P, Pd, k, blockIdx.x, blockIdx.y, blockIdx.z,
-                                        reinterpret_cast<R*>(lsm));
-  else
-    lb_tile<S, R, DEV, NOISE, I, CORR>(src, dst, P, Pd, k, blockIdx.x, blockIdx.y, blockIdx.z,
-                                       reinterpret_cast<R*>(lsm), tab);
+}
+
+// n / d for n < 2^24 and 2 <= d <= 256 by one multiply-high with m = ceil(2^32 / d): with
+// e = m d - 2^32 < d, n m / 2^32 = n / d + n e / (d 2^32) and n e < 2^32 keeps the error below
+// the distance of n / d to the next integer (checked exhaustively for every d and n in range).
+__host__ __device__ __forceinline__ unsigned magic_of(unsigned d) {
+  return (unsigned)((0x100000000ull + d - 1) / d);
+}
+__device__ __forceinline__ unsigned div_magic(unsigned n, unsigned m) { return __umulhi(n, m); }
+
+// The same launch over consecutive nodes (4 <= L <= 256), one block of threads after the other, with
+// one more block that waits, for the FP64 kernel.  That kernel is bound by the FP64 pipe (2
+// multiply-adds per clock and SM), which an instruction holds for 16 clocks whatever its lanes do:
+// no lane may idle, and a small box must reach every SM.  With the noise's radii and angles read
+// from tables, L = 72: 163 us per step (580 with a logarithm and a square root per pair; 2.3
+// GLUPS); L = 16, alone under ncu: 46 us (32 blocks of 256 threads with half the lanes idle) to
+// the bead kernel's shadow.
+template <class S, class R, bool DEV, bool NOISE, bool CORR>
+__global__ void __launch_bounds__(256) k_lb_linear(const S* __restrict__ src, S* __restrict__ dst, const FluidK<R> P,
+                                                   const PendK<R> Pd, const uint32_t step, const unsigned nnodes,
+                                                   const unsigned mag_L) {
+  extern __shared__ __align__(16) unsigned char lsm[];
+  const unsigned node = blockIdx.x * blockDim.x + threadIdx.x;
+  if (P.pdl & 1) grid_dependency_wait();
+  allow_dependent_launch();
+  if ((P.pdl & 2) && blockIdx.x == gridDim.x - 1) {  // the waiting block
+    grid_dependency_wait();
+    return;
+  }
+  if (node >= nnodes) return;
+  const uint32_t k = launch_step(P, step);
+  const unsigned row = div_magic(node, mag_L), x = node - row * P.L;
+  const unsigned z = div_magic(row, mag_L), y = row - z * P.L;
+  lb_node<S, R, DEV, NOISE, unsigned, CORR>(src, dst, P, Pd, k, x, y, z, reinterpret_cast<R*>(lsm) + threadIdx.x,
+                                            blockDim.x);
 }
 
 // ---------------------------------------------------------------------------------------

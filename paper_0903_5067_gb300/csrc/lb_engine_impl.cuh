@@ -14,10 +14,23 @@ namespace gblb {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// the noise tables of the FP64 kernels (NoiseTab) in one region: radii, then angles
+inline size_t noise_table_bytes() { return kRadii * sizeof(double) + kAngles * sizeof(double2); }
+inline NoiseTab noise_tables_at(void* base) {
+  double* radius = static_cast<double*>(base);
+  return NoiseTab{radius, reinterpret_cast<const double2*>(radius + kRadii)};
+}
+inline void launch_fill_noise_tables(void* base, cudaStream_t s) {
+  double* radius = static_cast<double*>(base);
+  fill_noise_tables<<<1216, 256, 0, s>>>(radius, reinterpret_cast<double2*>(radius + kRadii));
+  cuda_check(cudaGetLastError(), "noise tables");
+}
+
 template <class S, class R, bool DEV>
 class EngineT final : public Engine {
  public:
-  explicit EngineT(const Config& c) : cfg_(c) {
+  // own_tables: the FP64 noise tables are part of this engine's workspace (else set_noise_tables)
+  explicit EngineT(const Config& c, bool own_tables = true) : cfg_(c), own_tables_(own_tables && sizeof(R) == 8) {
     L_ = c.L;
     nnodes_ = (unsigned long long)L_ * L_ * L_;
     plane_ = align_up(nnodes_, 64);
@@ -33,19 +46,19 @@ class EngineT final : public Engine {
   void bind(void* base) override { layout(static_cast<unsigned char*>(base)); }
 
   void set_config(const Config& c) override { cfg_ = c; }
+  void set_noise_tables(void* base) { noise_tab_ = base; }
 
   void initialise(const double* x0, const double* v0, cudaStream_t s) override {
     snap_valid_ = false;
     {
-      dim3 blk, grd;
-      lb_launch_shape(blk, grd, pair_nodes());
-      const size_t sb = lb_stage_bytes(blk);
-      if (sb > 48 * 1024)  // FP64: staged corrections of a 256-thread tile
+      const LbLaunch q = lb_launch(false);
+      if (q.stage_bytes > 48 * 1024)  // FP64: staged corrections of a 256-thread tile
         for (int v = 0; v < 8; ++v)
           cuda_check(cudaFuncSetAttribute(lb_kernel(v & 1, (v >> 1) & 1, v >> 2, pair_nodes()),
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb),
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q.stage_bytes),
                      "LB kernel shared memory");
     }
+    if (own_tables_) launch_fill_noise_tables(noise_tab_, s);
     if (bead_smem() > 48 * 1024)
       cuda_check(cudaFuncSetAttribute(k_bead_step<S, R, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)bead_smem()),
@@ -751,15 +764,12 @@ class EngineT final : public Engine {
     FluidK<R> P = P0;
     const bool chained = ev0 == nullptr;
     P.pdl = chained ? (N_ > 0 ? 2 : 1) : 0;
-    P.angle_tab = sizeof(R) == 8 ? 1 : 0;
-    dim3 blk, grd;
-    lb_launch_shape(blk, grd, pair_nodes());
+    const LbLaunch q = lb_launch((P.pdl & 2) != 0);
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof(lc));
-    if (P.pdl & 2) grd.z += 1;  // the plane of waiting blocks
-    lc.gridDim = grd;
-    lc.blockDim = blk;
-    lc.dynamicSmemBytes = Pd.have_prev ? lb_stage_bytes(blk) : 0;  // staged corrections
+    lc.gridDim = q.grd;
+    lc.blockDim = q.blk;
+    lc.dynamicSmemBytes = Pd.have_prev ? q.stage_bytes : 0;  // staged corrections
     lc.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -767,8 +777,15 @@ class EngineT final : public Engine {
     lc.attrs = at;
     lc.numAttrs = chained ? 1 : 0;
     if (ev0) cudaEventRecord(ev0, s);
-    cuda_check(cudaLaunchKernelEx(&lc, lb_kernel(P.ncalls > 0, narrow_offsets(), N_ > 0, pair_nodes()), A, Bo, P, Pd, k),
-               "LB kernel");
+    if constexpr (sizeof(R) == 8) {
+      if (q.linear)
+        cuda_check(cudaLaunchKernelEx(&lc, lb_linear_kernel(P.ncalls > 0, N_ > 0), A, Bo, P, Pd, k, (unsigned)nnodes_,
+                                      magic_of((unsigned)L_)),
+                   "LB kernel");
+    }
+    if (!q.linear)
+      cuda_check(cudaLaunchKernelEx(&lc, lb_kernel(P.ncalls > 0, narrow_offsets(), N_ > 0, pair_nodes()), A, Bo, P, Pd, k),
+                 "LB kernel");
     if (ev1) cudaEventRecord(ev1, s);
     cuda_check(cudaGetLastError(), "LB kernel");
   }
@@ -855,6 +872,35 @@ class EngineT final : public Engine {
   // nodes per thread do not reduce)
   bool pair_nodes() const { return (L_ & 1) == 0 && sizeof(R) == 4; }
 
+  using LbLinear = void (*)(const S*, S*, const FluidK<R>, const PendK<R>, const uint32_t, const unsigned, const unsigned);
+  static LbLinear lb_linear_kernel(bool noise, bool corr) {
+    if (corr) return noise ? k_lb_linear<S, R, DEV, true, true> : k_lb_linear<S, R, DEV, false, true>;
+    return noise ? k_lb_linear<S, R, DEV, true, false> : k_lb_linear<S, R, DEV, false, false>;
+  }
+
+  // How the LB kernel covers the box: in FP64 consecutive nodes (k_lb_linear; its division needs
+  // L <= 256), in blocks of 256, halved down to one warp while there are fewer than two blocks per
+  // SM; else rows (lb_launch_shape).
+  struct LbLaunch {
+    bool linear;
+    dim3 blk, grd;
+    size_t stage_bytes;  // staged corrections of marked nodes: 19 values per thread
+  };
+  LbLaunch lb_launch(bool waiting) const {
+    LbLaunch q;
+    q.linear = sizeof(R) == 8 && L_ <= 256;
+    if (q.linear) {
+      unsigned t = 256;
+      while (t > 32 && (nnodes_ + t - 1) / t < 2 * 152) t /= 2;
+      q.blk = dim3(t);
+      q.grd = dim3((unsigned)((nnodes_ + t - 1) / t) + (waiting ? 1 : 0));
+    } else {
+      lb_launch_shape(q.blk, q.grd, pair_nodes());
+      if (waiting) q.grd.z += 1;  // the plane of waiting blocks
+    }
+    q.stage_bytes = (size_t)Q * q.blk.x * q.blk.y * sizeof(R);
+    return q;
+  }
   // threads along x cover a row of L nodes (L/2 threads with two nodes each), up to 256 per
   // block; the rest of the 256 threads take further rows
   void lb_launch_shape(dim3& blk, dim3& grd, bool pair) const {
@@ -865,8 +911,6 @@ class EngineT final : public Engine {
     blk = dim3(bx, by, 1);
     grd = dim3((row + bx - 1) / bx, ((unsigned)L_ + by - 1) / by, (unsigned)L_);
   }
-  // staged corrections of marked nodes: 19 values per thread of a tile
-  size_t lb_stage_bytes(const dim3& blk) const { return (size_t)Q * blk.x * blk.y * sizeof(R); }
 
   size_t bead_smem() const {
     // phase 5: up to kGroupHashMax entries a node table (4 x H ints, H >= 2 x entries), entry
@@ -938,6 +982,7 @@ class EngineT final : public Engine {
     P.body_on = (body[0] != 0 || body[1] != 0 || body[2] != 0) ? 1 : 0;
     for (int q = 0; q < 3; ++q) P.body_dJ[q] = (R)(body[q] * c.h * c.h / c.a);
     P.nonpos = nonpos_;
+    if (noise_tab_) P.tab = noise_tables_at(noise_tab_);
     return P;
   }
 
@@ -1061,10 +1106,13 @@ class EngineT final : public Engine {
     acc_ = reinterpret_cast<double*>(take(4 * sizeof(double)));
     obs_ = reinterpret_cast<double*>(take(kNObs * sizeof(double)));
     parts_ = reinterpret_cast<double*>(take(4 * (size_t)nparts_ * sizeof(double)));
+    if (own_tables_) noise_tab_ = take(noise_table_bytes());
     bytes_ = align_up(off, 256);
   }
 
   Config cfg_;
+  bool own_tables_ = false;
+  void* noise_tab_ = nullptr;
   int L_ = 0, N_ = 0, cap_ = 8, nparts_ = 0, nsub_ = 1;
   unsigned long long nnodes_ = 0, plane_ = 0;
   size_t bytes_ = 0;

@@ -182,46 +182,37 @@ __device__ __forceinline__ void fluid_pair(uint32_t w, const NoiseScale<float>& 
   g0 = r * approx_cos(th);
   if (SECOND) g1 = r * approx_sin(th);
 }
-// Double precision.  The angle theta = pi j / 2048, j = 2 k_a + 1 - 2048 (odd, |j| < 2048),
-// takes 2048 values; with `tab` (two tables of (cos, sin) filled by fill_angle_tables) its
-// cosine and sine come from j = 64 a + b (a = j >> 6 in [-32, 31], b = j & 63) by the angle
-// addition formulas, four operations instead of sincospi; without, from sincospi.
-struct AngleTab {
-  double2 a[64];  // (cos, sin)(pi a / 32), a = -32 .. 31 at index a + 32
-  double2 b[64];  // (cos, sin)(pi b / 2048), b = 0 .. 63
+// Double precision: every factor of a pair is one of 2^21 radii and one of 2048 angles, so both are
+// read from tables in global memory (fill_noise_tables) instead of computed: the radius table
+// (16 MiB) stays in the L2 cache, the angle table (32 KiB) in the L1 cache.  A logarithm and a
+// square root cost about 40 FP64 instructions, each of which holds an SM's FP64 pipe for 16
+// clocks; a lookup costs one load.
+struct NoiseTab {
+  const double* radius;  // sqrt(-2 ln u0), u0 = (k + 1/2) 2^-21, k < 2^21
+  const double2* angle;  // (cos, sin)(2 pi (u1 - 1/2)), u1 = (k + 1/2) 2^-11, k < 2048
 };
-// fill the tables with the block's threads 0..127 (the caller synchronises the block)
-__device__ __forceinline__ void fill_angle_tables(AngleTab* t, unsigned tid) {
-  double s, c;
-  if (tid < 64) {
-    sincospi((double)((int)tid - 32) / 32.0, &s, &c);
-    t->a[tid] = make_double2(c, s);
-  } else if (tid < 128) {
-    sincospi((double)(tid - 64) / 2048.0, &s, &c);
-    t->b[tid - 64] = make_double2(c, s);
+constexpr unsigned kRadii = 1u << 21, kAngles = 1u << 11;
+__global__ inline void fill_noise_tables(double* radius, double2* angle) {
+  for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < kRadii; k += gridDim.x * blockDim.x) {
+    radius[k] = sqrt(-2.0 * log(((double)k + 0.5) * 0x1p-21));
+    if (k < kAngles) {
+      double s, c;
+      sincospi(2.0 * (((double)k + 0.5) * 0x1p-11) - 1.0, &s, &c);
+      angle[k] = make_double2(c, s);
+    }
   }
 }
 template <bool SECOND>
 __device__ __forceinline__ void fluid_pair(uint32_t w, const NoiseScale<double>& ns, double& g0, double& g1,
-                                           const AngleTab* tab = nullptr) {
-  const double u0 = ((double)(w >> 11) + 0.5) * 0x1p-21;
-  const double r = ns.sr * sqrt(-2.0 * log(u0));
-  double s, c;
-  if (tab) {
-    const int j = 2 * (int)(w & 0x7ffu) + 1 - 2048;
-    const double2 A = tab->a[(j >> 6) + 32], B = tab->b[j & 63];
-    c = fma(A.x, B.x, -(A.y * B.y));
-    s = fma(A.y, B.x, A.x * B.y);
-  } else {
-    const double u1 = ((double)(w & 0x7ffu) + 0.5) * 0x1p-11;
-    sincospi(2.0 * u1 - 1.0, &s, &c);
-  }
-  g0 = r * c;
-  if (SECOND) g1 = r * s;
+                                           const NoiseTab& tab) {
+  const double r = ns.sr * __ldg(tab.radius + (w >> 11));
+  const double2 cs = __ldg(tab.angle + (w & 0x7ffu));
+  g0 = r * cs.x;
+  if (SECOND) g1 = r * cs.y;
 }
 
 template <int P, bool SECOND = true, class R, class Emit>
-__device__ __forceinline__ void fluid_pair_emit(uint32_t w, const NoiseScale<R>& ns, Emit& emit, const AngleTab* tab) {
+__device__ __forceinline__ void fluid_pair_emit(uint32_t w, const NoiseScale<R>& ns, Emit& emit, const NoiseTab& tab) {
   R g0, g1;
   if constexpr (sizeof(R) == 8)
     fluid_pair<SECOND>(w, ns, g0, g1, tab);
@@ -232,11 +223,11 @@ __device__ __forceinline__ void fluid_pair_emit(uint32_t w, const NoiseScale<R>&
 }
 
 // The Gaussians of one node, times sqrt(rho), handed out as emit(j, g_j) for mode 4 + j:
-// j = 0..5 (stress modes) always, j = 6..14 (kinetic modes) when `kinetic`.  tab: the angle
-// tables of the double-precision pairs (null: sincospi; ignored in single precision).
+// j = 0..5 (stress modes) always, j = 6..14 (kinetic modes) when `kinetic`.  tab: the tables of
+// the double-precision pairs (ignored in single precision).
 template <class R, class Emit>
 __device__ __forceinline__ void fluid_noise(uint32_t step, uint32_t node, const RoundKeys& rk, bool kinetic,
-                                            const NoiseScale<R>& ns, Emit emit, const AngleTab* tab = nullptr) {
+                                            const NoiseScale<R>& ns, Emit emit, const NoiseTab& tab) {
   U4 w = philox4x32_10_rk(U4{step, node, 0u, 0u}, rk);
   fluid_pair_emit<0>(w.x, ns, emit, tab);
   fluid_pair_emit<1>(w.y, ns, emit, tab);
