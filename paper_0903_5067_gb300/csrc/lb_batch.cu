@@ -17,6 +17,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <memory>
 #include <vector>
 
@@ -146,9 +147,17 @@ template <class S, class R, bool DEV, bool NOISE, bool PERSIST>
 __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_batch_lb(const __grid_constant__ BatchLB<S, R> B, int parity,
                                                    const uint32_t* __restrict__ d_step, uint32_t j) {
   extern __shared__ __align__(16) unsigned char dsm[];  // staged corrections, 19 x T
+  // every grid releases the next at once, and one more block than there are tiles (!PERSIST), or
+  // every block at its end, waits for the grid before: the bead kernel of this step or the previous
+  // group's LB kernel, so that this grid's completion stands for all before it
+  allow_dependent_launch();
   const uint32_t step = *d_step + j;
   if (!PERSIST) {
     const unsigned long long tile = blockIdx.x;
+    if (tile == B.total_tiles) {
+      grid_dependency_wait();
+      return;
+    }
     int lo = 0, hi = B.nrep - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
@@ -175,36 +184,47 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_batch_lb(const 
     __syncthreads();
     cur = s_next;
   }
+  grid_dependency_wait();
 }
 
-// One 256-thread block per replica's chain: in FP32 at most 80 registers per thread, which
-// leaves room on its SM for four 256-thread LB blocks.  Block 0 also zeroes the tile
-// counters the next step's LB launches will use.
+// One cluster of G 256-thread blocks per replica's chain (a chain that needs the sorted grouping runs
+// on its first block): in FP32 at most 80 registers per thread, which leaves room on its SM for
+// four 256-thread LB blocks.  Block 0 also zeroes the tile counters the next step's LB launches
+// will use.
 template <class S, class R, bool DEV>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_batch_bead(const ReplicaK<S, R>* __restrict__ reps, int parity,
                                                      const uint32_t* __restrict__ d_step, uint32_t j,
-                                                     unsigned long long* __restrict__ counters, int ngroups) {
+                                                     unsigned long long* __restrict__ counters, int ngroups, int G) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ FluidK<R> sP;
   __shared__ ChainK<R> sC;
-  allow_dependent_launch();
-  if (blockIdx.x == 0)
-    for (int g = threadIdx.x; g < ngroups; g += blockDim.x) counters[2 * g + (parity ^ 1)] = 0ull;
-  const ReplicaK<S, R>& rp = reps[blockIdx.x];
-  if (!rp.has_chain) return;
-  {
+  const ReplicaK<S, R>& rp = reps[blockIdx.x / (unsigned)G];
+  const int rank = (int)(blockIdx.x % (unsigned)G);
+  const bool sorted = 8 * rp.C.N * rp.C.nsub > kGroupMax;
+  const bool idle = !rp.has_chain || (sorted && rank > 0);
+  if (!idle) {
     const unsigned* a = reinterpret_cast<const unsigned*>(&rp.P);
     unsigned* b = reinterpret_cast<unsigned*>(&sP);
     for (unsigned w = threadIdx.x; w < sizeof(FluidK<R>) / 4; w += blockDim.x) b[w] = a[w];
     const unsigned* c = reinterpret_cast<const unsigned*>(&rp.C);
     unsigned* d = reinterpret_cast<unsigned*>(&sC);
     for (unsigned w = threadIdx.x; w < sizeof(ChainK<R>) / 4; w += blockDim.x) d[w] = c[w];
+    __syncthreads();
   }
-  __syncthreads();
   const uint32_t step = *d_step + j;
+  if (blockIdx.x == 0 || idle || sorted) {
+    grid_dependency_wait();
+    if (blockIdx.x == 0)  // the previous step's LB kernels have finished with these
+      for (int g = threadIdx.x; g < ngroups; g += blockDim.x) counters[2 * g + (parity ^ 1)] = 0ull;
+    if (idle || sorted) allow_dependent_launch();
+    if (idle) return;
+  }
   PendK<R> Pd = rp.pd[parity];
   Pd.have_prev = 1;  // an empty list after a flush
-  bead_step_block<S, R, DEV>(rp.pop[parity], sP, sC, Pd, step, smem);
+  if (sorted)
+    bead_step_sorted<S, R, DEV>(rp.pop[parity], sP, sC, Pd, step, smem);
+  else
+    bead_step_block<S, R, DEV, true>(rp.pop[parity], sP, sC, Pd, step, smem, rank, G);
 }
 
 // zero the counts of one pending slot of every replica (after the flush applied it)
@@ -214,8 +234,8 @@ __global__ void k_batch_clear(const ReplicaK<S, R>* __restrict__ reps, int nrep,
     if (reps[r].has_chain) *reps[r].pd[slot].cur_count = 0;
 }
 
-// B[i][node] += dn_i for the pending list of `slot` of every replica, into buffer `buf`, and
-// those entries of the dense correction field back to zero
+// B[i][node] += the dense field's corrections at the nodes of the pending list of `slot` of every
+// replica, into buffer `buf`, and those entries of the field back to zero
 template <class S, class R>
 __global__ void __launch_bounds__(256) k_batch_apply(const ReplicaK<S, R>* __restrict__ reps, int buf, int slot) {
   const ReplicaK<S, R>& rp = reps[blockIdx.z];
@@ -225,9 +245,10 @@ __global__ void __launch_bounds__(256) k_batch_apply(const ReplicaK<S, R>* __res
   if (u >= *pd.cur_count) return;
   const int i = blockIdx.y;
   const int4 q = pd.cur_pos[u];
+  if (q.x < 0) return;
   const unsigned long long off = (unsigned long long)i * rp.P.plane + (unsigned)q.x;
   S* p = rp.pop[buf] + off;
-  st<S, R>(p, ld<S, R>(p) + pd.cur_dn[i * pd.cap + u]);
+  st<S, R>(p, ld<S, R>(p) + pd.cur_dense[off]);
   pd.cur_dense[off] = R(0);
   if (i == 0) clear_marks(pd.cur_mask, pd.seg0, (int)rp.P.L, q.y, q.z, q.w);
 }
@@ -308,12 +329,14 @@ class BatchT final : public Batch {
   }
 
   void initialise(cudaStream_t s) override {
+    bead_g_ = bead_cluster();
     if (sizeof(R) == 8) launch_fill_noise_tables(base_ + noise_off_, s);
     for (size_t r = 0; r < eng_.size(); ++r)
       eng_[r]->initialise(x0_[r].empty() ? nullptr : x0_[r].data(), nullptr, s);
     smem_ = 0;
     for (auto& e : eng_)
-      if (e->chain_length() > 0 && e->bead_smem_bytes() > smem_) smem_ = e->bead_smem_bytes();
+      if (e->chain_length() > 0 && e->bead_smem_bytes(e->sorted_beads() ? 1 : bead_g_) > smem_)
+        smem_ = e->bead_smem_bytes(e->sorted_beads() ? 1 : bead_g_);
     if (smem_ > 48 * 1024)
       cuda_check(cudaFuncSetAttribute(k_batch_bead<S, R, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem_),
@@ -355,7 +378,7 @@ class BatchT final : public Batch {
       if (!graph_exec_) build_graph(s);
       for (; done + kGraph <= n; done += kGraph) cuda_check(cudaGraphLaunch(graph_exec_, s), "graph launch");
     }
-    for (int64_t j = done; j < n; ++j) launch_step(s, (uint32_t)(j - done), /*advance=*/false);
+    for (int64_t j = done; j < n; ++j) launch_step(s, (uint32_t)(j - done), j > done);
     if (done < n) {
       k_add_step<<<1, 1, 0, s>>>(d_step_, (uint32_t)(n - done));
       cuda_check(cudaGetLastError(), "advance step");
@@ -381,9 +404,9 @@ class BatchT final : public Batch {
         set_shape(t, b);
         upload_table(s);
         k_set_step<<<1, 1, 0, s>>>(d_step_, 0);
-        for (int w = 0; w < 2; ++w) launch_step(s, 0, true);
+        for (int w = 0; w < 2; ++w) launch_step(s, (uint32_t)w, w > 0);
         cuda_check(cudaEventRecord(e0, s), "event");
-        for (int w = 0; w < 6; ++w) launch_step(s, 0, true);
+        for (int w = 2; w < 8; ++w) launch_step(s, (uint32_t)w, w > 2);
         flush(s);
         cuda_check(cudaEventRecord(e1, s), "event");
         cuda_check(cudaEventSynchronize(e1), "event sync");
@@ -407,6 +430,21 @@ class BatchT final : public Batch {
 
  private:
   static constexpr int kGraph = 16;
+  // Blocks per replica's chain.  More shorten the bead kernel, which sets the step of small boxes,
+  // while the bead kernels have the chip to themselves, a block per SM (8 replicas of L = 15,
+  // N = 32, two substeps: 27.6, 18.8, 15.5 and 12.9 us per step on 1, 2, 4 and 8 blocks; 64 of them:
+  // 32.5, 23.3, 23.8 and 31.2); where the LB kernel sets the step they only take its place (64
+  // replicas, 5.2 M nodes: 131.6, 132.2 and 134.6 us on 1, 2 and 4).
+  int bead_cluster() const {
+    unsigned long long nodes = 0;
+    int longest = 1;
+    for (auto& e : eng_) {
+      nodes += e->nodes();
+      longest = std::max(longest, e->chain_length());
+    }
+    if (nodes > 2000000ull) return 1;
+    return std::max(1, std::min({8, (longest + 3) / 4, 152 / (int)eng_.size()}));
+  }
 
   void ensure_streams() {
     if (cap_) return;
@@ -461,7 +499,6 @@ class BatchT final : public Batch {
         pd.cur_dense = eng_[r]->pending_dense(jj);
         pd.plane = eng_[r]->plane();
         pd.cur_pos = eng_[r]->pending_pos(jj);
-        pd.cur_dn = eng_[r]->pending_dn(jj);
         pd.cur_count = eng_[r]->pending_count(jj);
         pd.cur_mask = flags_[jj];
         pd.mark = 1;
@@ -511,21 +548,40 @@ class BatchT final : public Batch {
     table_threads_ = threads_;
   }
 
-  // one lockstep step; kernels read step = *d_step + j (advance: bump the counter after).
-  // The bead kernel releases the first LB launch at its start; the next step's bead kernel,
-  // an ordinary launch, waits for both.  The force corrections stay pending (see k_batch_lb).
-  void launch_step(cudaStream_t s, uint32_t j, bool advance) {
+  // one lockstep step; kernels read step = *d_step + j.
+  // Launches are chained by programmatic stream serialization: the bead kernel (chained: it follows
+  // a step's LB kernel, not one that writes the counter, which it reads before it waits) waits for
+  // the previous step's last LB kernel, then releases the first LB kernel of its step, which runs
+  // beside it and completes only after it (see k_batch_lb).  The force corrections stay pending.
+  void launch_step(cudaStream_t s, uint32_t j, bool chained) {
     const int par = eng_[0]->parity();
     const int R_ = (int)eng_.size();
-    k_batch_bead<S, R, DEV><<<R_, 256, smem_, s>>>(d_reps_, par, d_step_, j, counters_, (int)groups_.size());
-    cuda_check(cudaGetLastError(), "batch bead");
+    {
+      cudaLaunchConfig_t lc;
+      memset(&lc, 0, sizeof(lc));
+      lc.gridDim = dim3((unsigned)(R_ * bead_g_));
+      lc.blockDim = dim3(256);
+      lc.dynamicSmemBytes = smem_;
+      lc.stream = s;
+      cudaLaunchAttribute at[2];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)bead_g_;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      at[1].val.programmaticStreamSerializationAllowed = 1;
+      lc.attrs = at;
+      lc.numAttrs = chained ? 2 : 1;
+      cuda_check(cudaLaunchKernelEx(&lc, k_batch_bead<S, R, DEV>, (const ReplicaK<S, R>*)d_reps_, par,
+                                    (const uint32_t*)d_step_, j, counters_, (int)groups_.size(), bead_g_),
+                 "batch bead");
+    }
     int dev = 0, sms = 0;
     cuda_check(cudaGetDevice(&dev), "device");
     cuda_check(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-    bool first = true;
     for (const BatchLB<S, R>& G : groups_) {
-      unsigned grid = (unsigned)G.total_tiles;
-      if (bps_ > 0 && (unsigned long long)sms * bps_ < G.total_tiles) grid = (unsigned)(sms * bps_);
+      unsigned grid = (unsigned)G.total_tiles + 1;  // one block that waits
+      if (bps_ > 0) grid = (unsigned)std::min<unsigned long long>((unsigned long long)sms * bps_, G.total_tiles);
       cudaLaunchConfig_t lc;
       memset(&lc, 0, sizeof(lc));
       lc.gridDim = dim3(grid);
@@ -536,12 +592,10 @@ class BatchT final : public Batch {
       at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
       at[0].val.programmaticStreamSerializationAllowed = 1;
       lc.attrs = at;
-      lc.numAttrs = first ? 1 : 0;
+      lc.numAttrs = 1;
       cuda_check(cudaLaunchKernelEx(&lc, lb_kernel(noise_, bps_ > 0), G, par, (const uint32_t*)d_step_, j),
                  "batch LB");
-      first = false;
     }
-    if (advance) k_add_step<<<1, 1, 0, s>>>(d_step_, 1);
     for (auto& e : eng_) e->flip();
   }
 
@@ -551,7 +605,7 @@ class BatchT final : public Batch {
     drop_graph();
     cudaGraph_t g = nullptr;
     cuda_check(cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal), "begin capture");
-    for (int j = 0; j < kGraph; ++j) launch_step(cap_, (uint32_t)j, false);
+    for (int j = 0; j < kGraph; ++j) launch_step(cap_, (uint32_t)j, j > 0);
     k_add_step<<<1, 1, 0, cap_>>>(d_step_, kGraph);
     cuda_check(cudaStreamEndCapture(cap_, &g), "end capture");
     cuda_check(cudaGraphInstantiate(&graph_exec_, g, 0), "instantiate graph");
@@ -571,6 +625,7 @@ class BatchT final : public Batch {
   ReplicaK<S, R>* d_reps_ = nullptr;
   uint32_t* d_step_ = nullptr;
   unsigned long long total_tiles_ = 0;
+  int bead_g_ = 1;
   int threads_ = 256, bps_ = 0, table_threads_ = -1, cap_max_ = 8;
   bool noise_ = true;
   cudaStream_t cap_ = nullptr;

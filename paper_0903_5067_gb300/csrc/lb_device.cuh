@@ -141,6 +141,9 @@ struct ChainK {
   int N;
   R m, zeta, kfene, R0sq, eps, sig2, rc2;
   R h, a, box, half_box;
+  // 1/(2m) and 1/a where they are exact (2m, a powers of two): the product is then the quotient,
+  // without a division; else 0
+  R inv_2m, inv_a;
   R amp;            // sqrt(2 kT zeta / h), 0 without bead noise
   uint32_t k0, k1;  // Philox key of the bead stream
   R ext[3];         // constant external force on each bead
@@ -167,9 +170,6 @@ struct ChainK {
   int* e_node;  // 8N corner nodes
   R* e_w;      // 8N trilinear weights
   R* e_mom;    // 4 x 8N: post-stream rho, Jx, Jy, Jz at the corner node
-  int4* p_pos; // pending force corrections: {node, x, y, z}, and 19 deltas [i][cap]
-  R* p_dn;
-  int* p_count;
   int cap;     // 8N
   unsigned* status;
   // FP64 snapshot of the state after each step, written by the bead kernel of step k into
@@ -179,9 +179,9 @@ struct ChainK {
 };
 
 // Force corrections in flight between consecutive steps of a multi-step run.  The bead kernel
-// of step k writes them twice: as a list (node, 19 deltas) for the final flush, and into a
-// dense correction field of the population layout [i][plane] that is zero except at pending
-// nodes; it also marks, in a bit mask over the nodes (one 32-bit word per 32 consecutive
+// of step k writes them into a dense correction field of the population layout [i][plane] that is
+// zero except at pending nodes, and lists the nodes (some list entries may be empty: node < 0);
+// it also marks, in a bit mask over the nodes (one 32-bit word per 32 consecutive
 // linear indices), every node that pulls from a corrected node.  The LB kernel of step k+1
 // adds the dense field to what it pulls at marked nodes, and the bead kernel of step k+1 to
 // what it gathers.  Two slots alternate by step; a bead kernel first clears its slot's dense
@@ -192,8 +192,7 @@ struct PendK {
   int have_prev;          // 0: nothing pending (the stored populations are complete)
   const unsigned* prev_mask;  // nodes that pull from the previous step's corrected nodes
   const R* prev_dense;    // the previous step's corrections, dense
-  int4* cur_pos;          // this step's list: {node, x, y, z}
-  R* cur_dn;              // 19 deltas [i][cap]
+  int4* cur_pos;          // this step's list: {node, x, y, z}, node < 0: empty
   int* cur_count;
   R* cur_dense;           // this step's slot of the dense field
   unsigned* cur_mask;     // this step's slot of the mask (cleared of the old list)
@@ -208,35 +207,40 @@ constexpr int kSegShift = 5;  // mask words of 32 consecutive nodes
 // ---------------------------------------------------------------------------------------
 // moment algebra
 // ---------------------------------------------------------------------------------------
-// scaled moments a_k = m_k / b_k  ->  populations n_i = w_i sum_k e_k(c_i) a_k
+// scaled moments a_k = m_k / b_k  ->  populations n_i = w_i sum_k e_k(c_i) a_k: the rest population
+// and the pair (2p + 1, 2p + 2) of opposite ones, p a constant after unrolling
+template <class R>
+__device__ __forceinline__ R pop_of_modes(const R a[Q], int i) {
+  R acc = R(0);
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    const int c = basis(k, i);
+    if (c != 0) acc += R(c) * a[k];
+  }
+  return acc * (R(w36(i)) / R(36));
+}
+template <class R>
+__device__ __forceinline__ void pair_of_modes(const R a[Q], const int p, R& n1, R& n2) {
+  const int i = 2 * p + 1;
+  R S = R(0), D = R(0);
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    const int c = basis(k, i);
+    if (c == 0) continue;
+    if (odd_mode(k))
+      D += R(c) * a[k];
+    else
+      S += R(c) * a[k];
+  }
+  const R w = R(w36(i)) / R(36);
+  n1 = w * (S + D);
+  n2 = w * (S - D);
+}
 template <class R>
 __device__ __forceinline__ void modes_to_pops(const R a[Q], R out[Q]) {
-  {
-    R acc = R(0);
+  out[0] = pop_of_modes<R>(a, 0);
 #pragma unroll
-    for (int k = 0; k < Q; ++k) {
-      const int c = basis(k, 0);
-      if (c != 0) acc += R(c) * a[k];
-    }
-    out[0] = acc * (R(w36(0)) / R(36));
-  }
-#pragma unroll
-  for (int p = 0; p < NPAIR; ++p) {
-    const int i = 2 * p + 1;
-    R S = R(0), D = R(0);
-#pragma unroll
-    for (int k = 0; k < Q; ++k) {
-      const int c = basis(k, i);
-      if (c == 0) continue;
-      if (odd_mode(k))
-        D += R(c) * a[k];
-      else
-        S += R(c) * a[k];
-    }
-    const R w = R(w36(i)) / R(36);
-    out[i] = w * (S + D);
-    out[i + 1] = w * (S - D);
-  }
+  for (int p = 0; p < NPAIR; ++p) pair_of_modes<R>(a, p, out[2 * p + 1], out[2 * p + 2]);
 }
 
 template <int K>
@@ -271,23 +275,21 @@ __device__ __forceinline__ void force_moments(R rho, R jx, R jy, R jz, R dx, R d
   dm[9] = cs * (ux * dz + uz * dx);
 }
 
-// population deltas of moment increments dm_0..9
-template <class R>
-__device__ __forceinline__ void dmoments_to_dpops(const R dm[10], R out[Q]) {
-  R a[Q];
-  a[0] = dm[0];
-  a[1] = dm[1] * R(InvB<1>::v);
-  a[2] = dm[2] * R(InvB<2>::v);
-  a[3] = dm[3] * R(InvB<3>::v);
-  a[4] = dm[4] * R(InvB<4>::v);
-  a[5] = dm[5] * R(InvB<5>::v);
-  a[6] = dm[6] * R(InvB<6>::v);
-  a[7] = dm[7] * R(InvB<7>::v);
-  a[8] = dm[8] * R(InvB<8>::v);
-  a[9] = dm[9] * R(InvB<9>::v);
+// scaled moments of the moment increments dm(1) .. dm(9) (the others zero)
+template <class R, class F>
+__device__ __forceinline__ void scaled_increments(F&& dm, R a[Q]) {
+  a[0] = R(0);
+  a[1] = dm(1) * R(InvB<1>::v);
+  a[2] = dm(2) * R(InvB<2>::v);
+  a[3] = dm(3) * R(InvB<3>::v);
+  a[4] = dm(4) * R(InvB<4>::v);
+  a[5] = dm(5) * R(InvB<5>::v);
+  a[6] = dm(6) * R(InvB<6>::v);
+  a[7] = dm(7) * R(InvB<7>::v);
+  a[8] = dm(8) * R(InvB<8>::v);
+  a[9] = dm(9) * R(InvB<9>::v);
 #pragma unroll
   for (int k = 10; k < Q; ++k) a[k] = R(0);
-  modes_to_pops(a, out);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -896,60 +898,53 @@ __device__ __forceinline__ R pair_coef(R r2, bool bonded, const ChainK<R>& C, un
   return coef;
 }
 
-// Conservative forces (FENE + WCA + external) on the beads bb0 .. bb1-1 from the positions of
-// all beads staged in shared memory; `lanes` threads per bead split the partners and combine
-// in a fixed shuffle tree.
+// Conservative force (FENE + WCA) on bead b from the positions of all beads staged in shared
+// memory; `lanes` neighbouring threads (lane: this one's) split the partners and combine in a
+// fixed shuffle tree.  Whole warps call it together (beads past the end: b = N).
+template <class R>
+__device__ __forceinline__ void bead_force(const R* __restrict__ sh, const R* __restrict__ sl, const ChainK<R>& C,
+                                           const int b, const int lane, const int lanes, R f[3]) {
+  const int N = C.N;
+  f[0] = f[1] = f[2] = R(0);
+  if (b < N) {
+    for (int j = lane; j < N; j += lanes) {
+      if (j == b) continue;
+      const bool bonded = (j == b - 1) || (j == b + 1);
+      R d[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        d[q] = pair_delta<R>(sh[3 * b + q], sl[3 * b + q], sh[3 * j + q], sl[3 * j + q], C.box, C.half_box);
+      const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+      const R coef = pair_coef<R>(r2, bonded, C, C.status);
+      f[0] += coef * d[0];
+      f[1] += coef * d[1];
+      f[2] += coef * d[2];
+    }
+  }
+  for (int o = lanes / 2; o > 0; o /= 2) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) f[q] += __shfl_xor_sync(0xffffffffu, f[q], o, lanes);
+  }
+}
+
+// Conservative forces (FENE + WCA + external) on every bead by a block; as many threads per bead
+// as fit
 template <class R>
 __device__ __forceinline__ void chain_forces_block(const R* __restrict__ sh, const R* __restrict__ sl,
-                                                   const ChainK<R>& C, R* __restrict__ out, const int bb0,
-                                                   const int bb1) {
+                                                   const ChainK<R>& C, R* __restrict__ out) {
   const int N = C.N, nt = blockDim.x * blockDim.y, tid = threadIdx.x + blockDim.x * threadIdx.y;
   int lanes = 1;
-  while (lanes < 32 && lanes * 2 * (bb1 - bb0) <= nt) lanes *= 2;
-  const int per = nt / lanes;
+  while (lanes < 32 && lanes * 2 * N <= nt) lanes *= 2;
   const int lane = tid % lanes;
-  for (int base = bb0; base < bb1; base += per) {
+  for (int base = 0; base < N; base += nt / lanes) {
     const int b = base + tid / lanes;
-    R f[3] = {R(0), R(0), R(0)};
-    if (b < bb1) {
-      for (int j = lane; j < N; j += lanes) {
-        if (j == b) continue;
-        const bool bonded = (j == b - 1) || (j == b + 1);
-        R d[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-          d[q] = pair_delta<R>(sh[3 * b + q], sl[3 * b + q], sh[3 * j + q], sl[3 * j + q], C.box, C.half_box);
-        const R r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-        const R coef = pair_coef<R>(r2, bonded, C, C.status);
-        f[0] += coef * d[0];
-        f[1] += coef * d[1];
-        f[2] += coef * d[2];
-      }
-    }
-    for (int o = lanes / 2; o > 0; o /= 2) {
-#pragma unroll
-      for (int q = 0; q < 3; ++q) f[q] += __shfl_xor_sync(0xffffffffu, f[q], o, lanes);
-    }
-    if (b < bb1 && lane == 0) {
+    R f[3];
+    bead_force<R>(sh, sl, C, b, lane, lanes, f);
+    if (b < N && lane == 0) {
 #pragma unroll
       for (int q = 0; q < 3; ++q) out[3 * b + q] = f[q] + C.ext[q];
     }
   }
-}
-
-constexpr int kGroupHashMax = 1024;  // entries grouped by hash table (else sorted)
-
-// Hash of a lattice node index onto a power-of-two table: the "lowbias32" integer finaliser
-// (xor-shift-multiply constants from C. Wellons' hash prospector).  Lattice neighbours differ
-// in few, structured bits, which a plain multiplicative hash maps to clustered low bits.
-__device__ __forceinline__ unsigned hash_node(int node, unsigned mask) {
-  unsigned h = (unsigned)node;
-  h ^= h >> 16;
-  h *= 0x7feb352du;
-  h ^= h >> 15;
-  h *= 0x846ca68bu;
-  h ^= h >> 16;
-  return h & mask;
 }
 
 // Bitonic sort (ascending) of M keys in shared memory, M a power of two >= 32, by a block of
@@ -1049,28 +1044,51 @@ __device__ __forceinline__ void gather_node(const S* __restrict__ pop, const Flu
   mom[3] = jz;
 }
 
-// The pending correction of one node (the coupling of Sec. II B, spread back to the fluid): the sum
-// of its entries' reactions in entry order (ent(base) .. ent(base + cnt - 1) ascending),
-// turned into population corrections at pending-list index u, written to the list and the
-// dense field, and the nodes pulling from it marked.
-template <class R, class Ent>
-__device__ __forceinline__ void node_correction(const FluidK<R>& P, const ChainK<R>& C, const PendK<R>& Pd, int L,
-                                                int N, int u, int node, Ent ent, int base, int cnt) {
-  const int e0 = ent(base);
-  R f[3] = {R(0), R(0), R(0)};
-  for (int r = base; r < base + cnt; ++r) {
-    const int e = ent(r);
-    const R w = C.e_w[e] * C.spread;
-    const int sub = e / (8 * N), b = (e - sub * 8 * N) >> 3;
-    const R* fch = C.fc_hist + sub * 3 * N;
-    f[0] -= w * fch[3 * b + 0] * C.inv_a3;
-    f[1] -= w * fch[3 * b + 1] * C.inv_a3;
-    f[2] -= w * fch[3 * b + 2] * C.inv_a3;
+// Mark the nodes of one row (dy, dz) that pull from node (px, py, pz), periodic: the three x
+// neighbours, or only px on a diagonal row; one atomic per word (the three bits lie in one word
+// unless they straddle two or wrap).
+__device__ __forceinline__ void mark_row(unsigned* mask, unsigned seg0, int L, int px, int py, int pz, int dy, int dz) {
+  int y = py + dy, z = pz + dz;
+  y = y < 0 ? L - 1 : (y >= L ? 0 : y);
+  z = z < 0 ? L - 1 : (z >= L ? 0 : z);
+  const int row = L * (y + L * z);
+  const unsigned c = (unsigned)(row + px);
+  unsigned bits = 1u << (c & 31u);
+  if (dy == 0 || dz == 0) {
+    const unsigned l = (unsigned)(row + (px ? px - 1 : L - 1)), r = (unsigned)(row + (px + 1 < L ? px + 1 : 0));
+    if ((l >> kSegShift) == (c >> kSegShift)) bits |= 1u << (l & 31u);
+    else atomicOr(mask + (seg0 + (l >> kSegShift)), 1u << (l & 31u));
+    if ((r >> kSegShift) == (c >> kSegShift)) bits |= 1u << (r & 31u);
+    else atomicOr(mask + (seg0 + (r >> kSegShift)), 1u << (r & 31u));
   }
-  const R rho = C.e_mom[e0], jx = C.e_mom[C.cap + e0], jy = C.e_mom[2 * C.cap + e0],
-          jz = C.e_mom[3 * C.cap + e0];
+  atomicOr(mask + (seg0 + (c >> kSegShift)), bits);
+}
+
+// Clear the mask words of the nodes that pull from node (px, py, pz) (whole words: in its slot
+// a word holds marks of one list only)
+__device__ __forceinline__ void clear_marks(unsigned* mask, unsigned seg0, int L, int px, int py, int pz) {
+  const int xm = px ? px - 1 : L - 1, xp = px + 1 < L ? px + 1 : 0;
+  const int ys[3] = {py ? py - 1 : L - 1, py, py + 1 < L ? py + 1 : 0};
+  const int zs[3] = {pz ? pz - 1 : L - 1, pz, pz + 1 < L ? pz + 1 : 0};
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    const int row = L * (ys[j % 3] + L * zs[j / 3]);
+    const unsigned c = (unsigned)(row + px) >> kSegShift;
+    mask[seg0 + c] = 0u;
+    if (j % 3 == 1 || j / 3 == 1) {
+      const unsigned l = (unsigned)(row + xm) >> kSegShift, r = (unsigned)(row + xp) >> kSegShift;
+      if (l != c) mask[seg0 + l] = 0u;
+      if (r != c) mask[seg0 + r] = 0u;
+    }
+  }
+}
+
+// Moment increments 1..9 of the force density f on a node of the given post-stream density and
+// momentum (the coupling of Sec. II B, spread back to the fluid)
+template <class R>
+__device__ __forceinline__ void coupling_moments(const FluidK<R>& P, const ChainK<R>& C, const R f[3], R rho, R jx,
+                                                 R jy, R jz, R dm[10]) {
   R dJ[3] = {f[0] * C.dJ_scale, f[1] * C.dJ_scale, f[2] * C.dJ_scale};
-  R dm[10];
   if (P.body_on) {
     // the LB kernel applies the body-force correction on every node; here add the
     // difference between the correction for the total force and the body-only one
@@ -1083,50 +1101,49 @@ __device__ __forceinline__ void node_correction(const FluidK<R>& P, const ChainK
   } else {
     force_moments(rho, jx, jy, jz, dJ[0], dJ[1], dJ[2], P.gs, P.gb, dm);
   }
-  R dn[Q];
-  dmoments_to_dpops(dm, dn);
+}
+
+// The pending correction of one node by one thread: population corrections written to the dense
+// field, the node listed at index u, and the nodes pulling from it marked.
+template <class R>
+__device__ __forceinline__ void node_correction(const FluidK<R>& P, const ChainK<R>& C, const PendK<R>& Pd, int L,
+                                                int u, int node, const R f[3], R rho, R jx, R jy, R jz) {
+  R dm[10], a[Q], dn[Q];
+  coupling_moments<R>(P, C, f, rho, jx, jy, jz, dm);
+  scaled_increments<R>([&](int k) { return dm[k]; }, a);
+  modes_to_pops(a, dn);
   const int pz = node / (L * L), py = (node / L) % L, px = node % L;
   Pd.cur_pos[u] = make_int4(node, px, py, pz);
 #pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    Pd.cur_dn[q * Pd.cap + u] = dn[q];
-    Pd.cur_dense[(unsigned long long)q * Pd.plane + (unsigned)node] = dn[q];
-  }
-  if (Pd.mark) {  // mark the nodes that pull from this node
-    // neighbour coordinates [c + 1] for c = -1, 0, +1 (periodic)
-    const int xs[3] = {px ? px - 1 : L - 1, px, px + 1 < L ? px + 1 : 0};
-    const int ys[3] = {py ? py - 1 : L - 1, py, py + 1 < L ? py + 1 : 0};
-    const int zs[3] = {pz ? pz - 1 : L - 1, pz, pz + 1 < L ? pz + 1 : 0};
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const unsigned idx = (unsigned)xs[cx(q) + 1] + (unsigned)L * ((unsigned)ys[cy(q) + 1] + (unsigned)L * (unsigned)zs[cz(q) + 1]);
-      atomicOr(&Pd.cur_mask[Pd.seg0 + (idx >> kSegShift)], 1u << (idx & 31u));
-    }
+  for (int q = 0; q < Q; ++q) Pd.cur_dense[(unsigned long long)q * Pd.plane + (unsigned)node] = dn[q];
+  if (Pd.mark) {
+#pragma unroll 1
+    for (int j = 0; j < 9; ++j) mark_row(Pd.cur_mask, Pd.seg0, L, px, py, pz, j % 3 - 1, j / 3 - 1);
   }
 }
 
-// Clear the mask words of the nodes that pull from node (px, py, pz) (whole words: in its slot
-// a word holds marks of one list only)
-__device__ __forceinline__ void clear_marks(unsigned* mask, unsigned seg0, int L, int px, int py, int pz) {
-  const int xs[3] = {px ? px - 1 : L - 1, px, px + 1 < L ? px + 1 : 0};
-  const int ys[3] = {py ? py - 1 : L - 1, py, py + 1 < L ? py + 1 : 0};
-  const int zs[3] = {pz ? pz - 1 : L - 1, pz, pz + 1 < L ? pz + 1 : 0};
-  unsigned last = 0xffffffffu;
+// Empty the list entry u (of this slot's list from two steps before, or already applied): its
+// node's corrections and the marks of the nodes pulling from it back to zero
+template <class R>
+__device__ __forceinline__ void clear_correction(const PendK<R>& Pd, int L, int u) {
+  const int4 p = Pd.cur_pos[u];
+  if (p.x < 0) return;
+  R* d = Pd.cur_dense + (unsigned)p.x;
 #pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const unsigned idx = (unsigned)xs[cx(q) + 1] + (unsigned)L * ((unsigned)ys[cy(q) + 1] + (unsigned)L * (unsigned)zs[cz(q) + 1]);
-    const unsigned w = seg0 + (idx >> kSegShift);
-    if (w != last) mask[w] = 0u;
-    last = w;
-  }
+  for (int i = 0; i < Q; ++i) d[(unsigned long long)i * Pd.plane] = R(0);
+  if (Pd.cur_mask) clear_marks(Pd.cur_mask, Pd.seg0, L, p.y, p.z, p.w);
 }
 
-// Generic address of the same shared-memory location in block 0 of the cluster
+// v into the same shared-memory location of block `rank` of the cluster
 template <class T>
-__device__ __forceinline__ const T* cluster_rank0(const T* p) {
-  unsigned long long d;
-  asm volatile("mapa.u64 %0, %1, 0;" : "=l"(d) : "l"(reinterpret_cast<unsigned long long>(p)));
-  return reinterpret_cast<const T*>(d);
+__device__ __forceinline__ void cluster_store(T* p, int rank, T v) {
+  static_assert(sizeof(T) == 4 || sizeof(T) == 8, "4- or 8-byte values");
+  unsigned d;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  if constexpr (sizeof(T) == 4)
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(d), "r"(__float_as_uint(v)) : "memory");
+  else
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(d), "l"(__double_as_longlong(v)) : "memory");
 }
 
 // Barrier over the thread blocks of a cluster; release/acquire order every memory access
@@ -1135,49 +1152,396 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// an arrival that orders no memory access (a release waits for the thread's writes in flight)
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// f / (2 m) and x / a, by the exact reciprocal where there is one
+template <class R>
+__device__ __forceinline__ R over_2m(R f, const ChainK<R>& C) {
+  return C.inv_2m != R(0) ? f * C.inv_2m : f / (R(2) * C.m);
+}
+template <class R>
+__device__ __forceinline__ R over_a(R x, const ChainK<R>& C) {
+  return C.inv_a != R(0) ? x * C.inv_a : x / C.a;
+}
+
+// First half kick and drift of one coordinate: v_half = v + h F/2m, x' = x + h v_half, in
+// compensated (hi, lo) arithmetic, then wrapped into [0, box) with the image counter
+template <class R>
+__device__ __forceinline__ void drift(const ChainK<R>& C, R v, R F, R xh, R xl, int& im, R& vh, R& hi, R& lo) {
+  vh = v + over_2m(C.h * F, C);
+  const R dx = C.h * vh;
+  hi = xh + dx;
+  const R bp = hi - xh;
+  lo = xl + ((xh - (hi - bp)) + (dx - bp));
+  {
+    const R s2 = hi + lo;
+    lo = lo - (s2 - hi);
+    hi = s2;
+  }
+  if (hi < R(0)) {
+    const R s2 = C.box + hi;
+    lo += hi - (s2 - C.box);
+    hi = s2;
+    --im;
+  }
+  if (hi >= C.box) {
+    hi -= C.box;
+    ++im;
+  }
+}
+
+// Entries (corners of beads over all substeps) up to which the bead step compares beads with one
+// another (bead_step_block); beyond, it sorts the entries (bead_step_sorted).
+constexpr int kGroupMax = 1024;
+
+// Shared memory of bead_step_block for N beads and nsub substeps of which a block has at most nb
+// beads.  A bead and substep is counted as "place" sub N + b, its corner c as entry 8 place + c.
+template <class R>
+struct BeadSmem {
+  R *x, *l, *vh;      // 3N each: drifted positions (high, low) and half-step velocities
+  R *fr;              // 3N: position inside the cell
+  R *v, *F;           // 2 x 3N each (nsub > 1): end of a substep, by its parity
+  R *fc;              // 3N nsub: coupling forces
+  R *w;               // 8 N nsub: trilinear weights of every entry
+  R *mom;             // 5 x own: density, momentum and 1/density at the block's corner nodes
+  R *fcons;           // 3 nb: conservative forces
+  R *g;               // 3 nb nsub: noise
+  int *node;          // own: the block's corner nodes
+  int *img;           // 3N
+  int *cell;          // 3N nsub
+  int *near;          // nb nsub x N nsub: of each of the block's places the ones whose cells touch its
+                      // cell: place | corners shared << 8 | (shift of the corner number + 8) << 16
+  int *nnear;         // nb nsub: their number
+  // lays the arrays out from base on; returns their size
+  __host__ __device__ __forceinline__ int carve(unsigned char* base, int N, int nsub, int nb) {
+    int off = 0;
+    auto take = [&](int bytes) {  // (no test of base: the compiler must see that these are shared)
+      unsigned char* p = base + off;
+      off += (bytes + 15) / 16 * 16;
+      return p;
+    };
+    const int r = (int)sizeof(R), n3 = 3 * N, own = 8 * nb * nsub;
+    x = (R*)take(n3 * r);
+    l = (R*)take(n3 * r);
+    vh = (R*)take(n3 * r);
+    fr = (R*)take(n3 * r);
+    v = (R*)take(nsub > 1 ? 2 * n3 * r : 0);
+    F = (R*)take(nsub > 1 ? 2 * n3 * r : 0);
+    fc = (R*)take(n3 * nsub * r);
+    w = (R*)take(8 * N * nsub * r);
+    mom = (R*)take(5 * own * r);
+    fcons = (R*)take(3 * nb * r);
+    g = (R*)take(3 * nb * nsub * r);
+    node = (int*)take(own * 4);
+    img = (int*)take(n3 * 4);
+    cell = (int*)take(n3 * nsub * 4);
+    near = (int*)take(nb * nsub * N * nsub * 4);
+    nnear = (int*)take(nb * nsub * 4);
+    return off;
+  }
+};
+
+// trilinear weight of corner c (bit q: the far side along q) at position fr inside the cell
+template <class R>
+__device__ __forceinline__ R corner_weight(const R* fr, int c) {
+  const R x = c & 1 ? fr[0] : R(1) - fr[0], y = c & 2 ? fr[1] : R(1) - fr[1], z = c & 4 ? fr[2] : R(1) - fr[2];
+  return x * y * z;
+}
+
 // One coupled bead step for one chain: velocity Verlet, FENE/WCA, interpolation of the
 // post-stream flow at the 8 corners, friction + Langevin force, and the deterministic
-// spreading of the reaction into a list of per-node population corrections.  Run by one
-// thread block (any size, multiple of 32), or by the G blocks of a cluster (rank: this
-// block's): each block computes the drift of every bead into its shared memory and then
-// takes a contiguous share of the beads (forces, corners and gathers, friction), of the old
-// list (clearing) and of the new list's nodes (corrections); block 0 writes the positions
-// and groups the corner entries by node in its shared memory, which the others read.
-// Most of this work is scattered global memory traffic, which G blocks issue from G SMs.
-// `smem` holds the positions (6N R; with G > 1 also the half-step velocities and image
-// counters, 9N R + 3N int), later the node grouping table (or the sort keys, G = 1 only), as
-// sized by the host.
-template <class S, class R, bool DEV>
+// spreading of the reaction into per-node population corrections.  Run by the G blocks of a
+// cluster (G = 1: one block; any size, a multiple of 32; rank: this block's).
+//
+// The step is a chain of dependent phases and bound by their latency, so what a phase hands
+// to the next stays in shared memory (through global memory each hand-over costs an L2 round
+// trip) and phases that do not depend on one another run on different warps:
+//   0  noise of the block's beads, before the wait for the previous grid;
+//   1  drift of every bead in every block (cheaper than an exchange); the threads left over
+//      clear the slot's old list meanwhile;
+//   2  the first warps gather density and momentum at the corner nodes of the block's beads (38
+//      loads each, in flight together), the others compute the weights and conservative forces;
+//   3  friction and second half kick of the block's beads; the coupling forces go to every block
+//      of the cluster (distributed shared memory); while they travel, the beads whose cells touch
+//      those of the block's beads;
+//   4  each node is corrected by the block that owns its first entry: the forces of all its
+//      entries, summed in entry order, need nothing from other blocks but the forces.
+// Comparing the cells of all beads (a corner is shared by beads of touching cells only) replaces
+// grouping the corners by a hash table with two scans on block 0 and two cluster barriers.
+// Kernel alone under ncu, before and after: N = 32 with two substeps 25 -> 11 us, N = 64 19 -> 11,
+// N = 16 14 -> 9 (FP32), N = 8 in FP64 50 -> 26.  Inside (clock stamps, N = 16): noise 0.6 us
+// (before the wait), drift 0.6, gathers and forces 1.2, friction 0.4, barrier 0.6, corrections 2.2:
+// single warps issuing dependent instructions, no longer memory.  (Spreading gathers and
+// corrections over all warps by population, which multiplies their index arithmetic, came out
+// slower: 7.1 against 6.9 us per step at L = 32, N = 16; 31 against 26 for 64 replicas of L = 15.)
+template <class S, class R, bool DEV, bool PDL>
 __device__ __forceinline__ void bead_step_block(const S* __restrict__ pop, const FluidK<R>& P, const ChainK<R>& C,
                                                 const PendK<R>& Pd, const uint32_t step, unsigned char* smem,
-                                                const int rank = 0, const int G = 1) {
+                                                const int rank, const int G) {
+  const int N = C.N, nsub = C.nsub;
+  const int tid = threadIdx.x + blockDim.x * threadIdx.y, nt = blockDim.x * blockDim.y;
+  const int lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
+  const int L = (int)P.L;
+  const R h = C.h;
+  const int b0 = rank * N / G, nb = (rank + 1) * N / G - b0;  // this block's beads
+  const int nc = 8 * nb;                                      // and their corners in one substep
+  const int own = nc * nsub, np = N * nsub;                   // entries of the block, places
+  BeadSmem<R> M;
+  M.carve(smem, N, nsub, (N + G - 1) / G);
+  // the chain's number of the block's place i (sub nb + b)
+  auto place = [&](int i) {
+    if (nsub == 1) return b0 + i;
+    const int sub = i / nb;
+    return sub * N + b0 + i - sub * nb;
+  };
+  // 0. noise
+  for (int i = tid; i < nb * nsub; i += nt) {
+    const int sub = i / nb, b = b0 + i - sub * nb;
+    R g[4] = {R(0), R(0), R(0), R(0)};
+    if (C.amp != R(0)) gauss4<R>(step * (uint32_t)nsub + (uint32_t)sub, (uint32_t)b, 0u, C.k0, C.k1, g);
+    M.g[3 * i] = g[0];
+    M.g[3 * i + 1] = g[1];
+    M.g[3 * i + 2] = g[2];
+  }
+  if (PDL) {
+    grid_dependency_wait();
+    allow_dependent_launch();
+  }
+  // clear this slot's old list; the list's entries are numbered alike every step, so that a block
+  // clears those it rewrites in phase 4.  Other blocks write new corrections (possibly at the
+  // same nodes) only after the second cluster barrier.
+  bool wrote = false;  // whether the warp has written what other blocks read or write after it
+  {
+    const int nd = 3 * N, c0 = nd < nt ? nd : 0;
+    if (tid >= c0 && *Pd.cur_count > 0)
+      for (int i = tid - c0; i < own; i += nt - c0) {
+        clear_correction<R>(Pd, L, 8 * place(i >> 3) + (i & 7));
+        wrote = true;
+      }
+  }
+  const R* corr = Pd.have_prev ? Pd.prev_dense : nullptr;
+  // MD substeps against the frozen post-stream fluid (one for LB step = MD step)
+  for (int sub = 0; sub < nsub; ++sub) {
+    const int poff = sub * 3 * N, ooff = sub * nc;
+    const bool last = sub + 1 == nsub;
+    // 1. drift of every bead, cells
+    const R* const pv = M.v + ((sub - 1) & 1) * 3 * N;
+    const R* const pF = M.F + ((sub - 1) & 1) * 3 * N;
+    for (int t = tid; t < 3 * N; t += nt) {
+      R vh, hi, lo;
+      int im;
+      if (sub == 0) {
+        im = C.img_in[t];
+        drift<R>(C, C.v_in[t], C.F_in[t], C.x_in[t], C.xl_in[t], im, vh, hi, lo);
+      } else {  // from the state the previous substep left here
+        im = M.img[t];
+        drift<R>(C, pv[t], pF[t], M.x[t], M.l[t], im, vh, hi, lo);
+      }
+      M.x[t] = hi;
+      M.l[t] = lo;
+      M.vh[t] = vh;
+      M.img[t] = im;
+      // cell = floor(x/a) mod L; the position inside it from the exact remainder x - floor(x/a) a
+      const R f = floor(over_a(hi, C));
+      int c = (int)f;
+      if ((unsigned)c >= (unsigned)L) {  // x/a rounded up to L, or not finite
+        R unused;
+        c = cell_of<R>(hi, C.a, L, unused);
+      }
+      M.cell[poff + t] = c;
+      M.fr[t] = over_a(fma(-f, C.a, hi) + lo, C);
+    }
+    // every block has started and read the state, once all have arrived: waited for before the
+    // first remote store and the first write of the state (its reads have returned)
+    if (G > 1 && sub == 0) cluster_arrive_relaxed();
+    __syncthreads();
+    // 2. post-stream density and momentum at the corner nodes of the block's beads ...
+    const int gw = (nc + 31) >> 5;            // warps that gather
+    const int g0 = gw < nwarp ? 32 * gw : 0;  // the other threads (all, when none is left over)
+    for (int i = tid; i < nc; i += nt) {
+      const int* cl = M.cell + poff + 3 * (b0 + (i >> 3));
+      int q[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        q[j] = cl[j] + ((i >> j) & 1);
+        if (q[j] >= L) q[j] -= L;
+      }
+      R mom[4];
+      gather_node_c<S, R, DEV>(pop, P, q[0], q[1], q[2], mom, corr);
+      const int o = ooff + i;
+      M.node[o] = q[0] + L * (q[1] + L * q[2]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) M.mom[j * own + o] = mom[j];
+      M.mom[4 * own + o] = R(1) / mom[0];
+    }
+    //    ... and on the other warps every corner's weight and the conservative forces at x': FENE on
+    //    bonds, WCA on all pairs, minimum image; the lanes of a bead split the partners and combine
+    //    in a fixed shuffle tree
+    if (tid >= g0) {
+      const int t1 = tid - g0, n1 = nt - g0;
+      for (int i = n1 - 1 - t1; i < 8 * N; i += n1) M.w[sub * 8 * N + i] = corner_weight(M.fr + 3 * (i >> 3), i & 7);
+      int lanes = 32;
+      while (lanes > 4 && nb * lanes > 2 * n1) lanes /= 2;
+      const int fl = t1 % lanes;
+      for (int base = 0; base < nb; base += n1 / lanes) {
+        const int i = base + t1 / lanes;
+        R f[3];
+        bead_force<R>(M.x, M.l, C, i < nb ? b0 + i : N, fl, lanes, f);
+        if (i < nb && fl < 3) M.fcons[3 * i + fl] = (fl == 0 ? f[0] : (fl == 1 ? f[1] : f[2])) + C.ext[fl];
+      }
+    }
+    if (G > 1 && sub == 0) cluster_wait();
+    __syncthreads();
+    // 3. friction + Langevin force, second half kick
+    auto write_state = [&](int t, R vn, R Ft, R fc) {
+      C.x[t] = M.x[t];
+      C.xl[t] = M.l[t];
+      C.img[t] = M.img[t];
+      C.v[t] = vn;
+      C.F[t] = Ft;
+      C.Fc[t] = fc;
+    };
+    R vn = R(0), Ft = R(0), fc = R(0);  // of coordinate 3 b0 + mine
+    int mine = -1;
+    for (int i = tid; i < 3 * nb; i += nt) {
+      if (mine >= 0 && last) write_state(3 * b0 + mine, vn, Ft, fc);
+      mine = i;
+      const int bl = i / 3, q = i - 3 * bl, t = 3 * b0 + i;
+      R ub = R(0);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const int o = ooff + 8 * bl + c;
+        ub += M.w[8 * (sub * N + b0 + bl) + c] * M.mom[(q + 1) * own + o] * M.mom[4 * own + o];
+      }
+      const R vh = M.vh[t];
+      fc = -C.zeta * (vh - ub * C.u_scale) + C.amp * M.g[3 * (sub * nb + bl) + q];
+      Ft = M.fcons[i] + fc;
+      vn = vh + over_2m(h * Ft, C);
+      R* const dst[3] = {M.fc + sub * 3 * N + t, M.v + (sub & 1) * 3 * N + t, M.F + (sub & 1) * 3 * N + t};
+      if (G == 1) {
+        *dst[0] = fc;
+        if (!last) {
+          *dst[1] = vn;
+          *dst[2] = Ft;
+        }
+      } else {
+        wrote = true;
+        for (int r = 0; r < G; ++r) {
+          cluster_store(dst[0], r, fc);
+          if (!last) {
+            cluster_store(dst[1], r, vn);
+            cluster_store(dst[2], r, Ft);
+          }
+        }
+      }
+    }
+    if (G > 1) {  // forces sent, old lists cleared
+      if (__any_sync(0xffffffffu, wrote)) cluster_arrive();
+      else cluster_arrive_relaxed();
+    }
+    if (!last) {
+      if (G > 1)
+        cluster_wait();
+      else
+        __syncthreads();
+    } else if (mine >= 0) {  // the end state (every block has read the state: first cluster barrier)
+      write_state(3 * b0 + mine, vn, Ft, fc);
+    }
+  }  // substeps
+
+  // The places whose cells touch the cell of each of the block's places, a warp per place: with the
+  // cells d apart (each component -1, 0 or 1), corner c of the one is corner c - d of the other
+  // where both lie in {0, 1}^3.
+  for (int i = nwarp - 1 - warp; i < nb * nsub; i += nwarp) {
+    const int* mine = M.cell + 3 * place(i);
+    int n = 0;
+    for (int j0 = 0; j0 < np; j0 += 32) {
+      const int j = j0 + lane;
+      int shared = 0, shift = 0;
+      if (j < np) {
+        shared = 0xff;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          int d = M.cell[3 * j + q] - mine[q];
+          d = d > 1 ? d - L : (d < -1 ? d + L : d);
+          const int far = q == 0 ? 0xaa : (q == 1 ? 0xcc : 0xf0);  // corners with bit q set
+          shared &= d == 0 ? 0xff : (d == 1 ? far : (d == -1 ? 0xff ^ far : 0));
+          shift += d << q;
+        }
+      }
+      const unsigned hit = __ballot_sync(0xffffffffu, shared != 0);
+      if (shared) M.near[i * np + n + __popc(hit & ((1u << lane) - 1u))] = j | shared << 8 | (shift + 8) << 16;
+      n += __popc(hit);
+    }
+    if (lane == 0) M.nnear[i] = n;
+  }
+  if (G > 1) cluster_wait();
+  __syncthreads();
+  // 4. deterministic spreading: the first entry of each node sums the node's contributions in
+  //    entry order and turns the node force into population corrections (the last threads, whose
+  //    warps are free)
+  for (int o = nt - 1 - tid; o < own; o += nt) {
+    const int i = o >> 3, c = o & 7, e = 8 * place(i) + c, node = M.node[o];
+    C.e_node[e] = node;
+    const int* near = M.near + i * np;
+    const int n = M.nnear[i];
+    R f[3] = {R(0), R(0), R(0)};
+    bool first = false;
+    for (int k = 0; k < n; ++k) {
+      const int code = near[k];
+      if (!((code >> (8 + c)) & 1)) continue;
+      const int j = code & 0xff, cj = c - ((code >> 16) - 8);
+      if (!first) {
+        if (8 * j + cj != e) break;  // an earlier entry has the node
+        first = true;
+      }
+      const R w = M.w[8 * j + cj] * C.spread;
+      const R* fc = M.fc + 3 * j;
+      f[0] -= w * fc[0] * C.inv_a3;
+      f[1] -= w * fc[1] * C.inv_a3;
+      f[2] -= w * fc[2] * C.inv_a3;
+    }
+    if (first)
+      node_correction<R>(P, C, Pd, L, e, node, f, M.mom[o], M.mom[own + o], M.mom[2 * own + o], M.mom[3 * own + o]);
+    else
+      Pd.cur_pos[e] = make_int4(-1, 0, 0, 0);
+  }
+  // the end state once more, as the bead read-back forms it
+  if (C.snap) {
+    double* sn = C.snap + (size_t)(step & 1u) * 6 * N;
+    for (int i = tid; i < 3 * nb; i += nt) {
+      const int t = 3 * b0 + i;
+      sn[t] = __dadd_rn(__dadd_rn((double)M.x[t], (double)M.l[t]), __dmul_rn((double)M.img[t], C.snap_box));
+      sn[3 * N + t] = (double)C.v[t];
+    }
+  }
+  if (rank == 0 && tid == 0) *Pd.cur_count = 8 * np;
+}
+
+// The same step by one block for more than kGroupMax entries: the entries are ordered by node by a
+// bitonic sort of (node, entry) keys, and hand-overs go through global memory.  `smem` holds the
+// positions (6N R), later the sort keys, leader slots and chunk counts.
+template <class S, class R, bool DEV>
+__device__ __forceinline__ void bead_step_sorted(const S* __restrict__ pop, const FluidK<R>& P, const ChainK<R>& C,
+                                                 const PendK<R>& Pd, const uint32_t step, unsigned char* smem) {
   const int N = C.N;
   const int tid = threadIdx.x + blockDim.x * threadIdx.y, nt = blockDim.x * blockDim.y;
   const int L = (int)P.L;
   const R h = C.h;
   R* sx = reinterpret_cast<R*>(smem);
   R* sl = sx + 3 * N;
-  R* svh = sl + 3 * N;                             // G > 1: half-step velocities
-  int* simg = reinterpret_cast<int*>(svh + 3 * N);  // G > 1: image counters
-  const R* vhp = G > 1 ? svh : C.vh;
-  const int b0 = rank * N / G, b1 = (rank + 1) * N / G;  // this block's beads
-  // clear this slot's dense entries of its old list (two steps back, or already applied);
-  // the new list overwrites the old one only in phase 5, after several barriers.  The threads
-  // the first drift leaves idle (t >= 3N; every block drifts every bead) clear while the others
-  // drift, so that the two chains of global round trips overlap; with no thread idle, every
-  // thread clears first.
+  // clear this slot's old list; the threads the first drift leaves idle do it while the others
+  // drift (with no thread idle, every thread first)
   {
-    const int nd = 3 * N;
-    const int c0 = nd < nt ? nd : 0, cn = nt - c0;  // the clearing threads [c0, nt)
+    const int nd = 3 * N, c0 = nd < nt ? nd : 0;
     if (tid >= c0) {
       const int old = *Pd.cur_count;
-      for (int u = (tid - c0) + rank * cn; u < old; u += G * cn) {
-        const int4 p = Pd.cur_pos[u];
-        R* d = Pd.cur_dense + (unsigned)p.x;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) d[(unsigned long long)i * Pd.plane] = R(0);
-        if (Pd.cur_mask) clear_marks(Pd.cur_mask, Pd.seg0, L, p.y, p.z, p.w);
-      }
+      for (int u = tid - c0; u < old; u += nt - c0) clear_correction<R>(Pd, L, u);
     }
   }
   const R* corr = Pd.have_prev ? Pd.prev_dense : nullptr;
@@ -1185,8 +1549,7 @@ __device__ __forceinline__ void bead_step_block(const S* __restrict__ pop, const
   // MD substeps against the frozen post-stream fluid (one for LB step = MD step)
   for (int sub = 0; sub < C.nsub; ++sub) {
   const int eoff = sub * 8 * N;
-  // 1. first half kick and drift: v_half = v + h F/2m, x' = x + h v_half, in compensated
-  //    (hi, lo) arithmetic, then wrapped into [0, box) with the image counter
+  // 1. first half kick and drift
   const bool first = sub == 0;  // later substeps continue from the written state
   const R* const vin = first ? C.v_in : C.v;
   const R* const Fin = first ? C.F_in : C.F;
@@ -1194,57 +1557,23 @@ __device__ __forceinline__ void bead_step_block(const S* __restrict__ pop, const
   const R* const xlin = first ? C.xl_in : C.xl;
   const int* const imgin = first ? C.img_in : C.img;
   for (int t = tid; t < 3 * N; t += nt) {
-    const R vh = vin[t] + h * Fin[t] / (R(2) * C.m);
-    const R dx = h * vh;
-    const R xh = xin[t];
-    R hi = xh + dx;
-    const R bp = hi - xh;
-    R lo = xlin[t] + ((xh - (hi - bp)) + (dx - bp));
-    {
-      const R s2 = hi + lo;
-      lo = lo - (s2 - hi);
-      hi = s2;
-    }
+    R vh, hi, lo;
     int im = imgin[t];
-    if (hi < R(0)) {
-      const R s2 = C.box + hi;
-      lo += hi - (s2 - C.box);
-      hi = s2;
-      --im;
-    }
-    if (hi >= C.box) {
-      hi -= C.box;
-      ++im;
-    }
-    if (G == 1) {
-      C.vh[t] = vh;
-      C.x[t] = hi;
-      C.xl[t] = lo;
-      C.img[t] = im;
-    } else {
-      svh[t] = vh;
-      simg[t] = im;
-    }
+    drift<R>(C, vin[t], Fin[t], xin[t], xlin[t], im, vh, hi, lo);
+    C.vh[t] = vh;
+    C.x[t] = hi;
+    C.xl[t] = lo;
+    C.img[t] = im;
     sx[t] = hi;
     sl[t] = lo;
   }
   __syncthreads();
-  if (G > 1) {
-    cluster_sync();  // every block has read the state of the previous (sub)step
-    if (rank == 0)
-      for (int t = tid; t < 3 * N; t += nt) {
-        C.vh[t] = svh[t];
-        C.x[t] = sx[t];
-        C.xl[t] = sl[t];
-        C.img[t] = simg[t];
-      }
-  }
 
   // 2. conservative forces at x': FENE on bonds, WCA on all pairs, minimum image
-  chain_forces_block<R>(sx, sl, C, C.fcons, b0, b1);
+  chain_forces_block<R>(sx, sl, C, C.fcons);
 
-  // 3. corners of the block's beads: cell, trilinear weight, post-stream rho and J at the node
-  for (int e0 = 8 * b0 + tid; e0 < 8 * b1; e0 += nt) {
+  // 3. corners: cell, trilinear weight, post-stream rho and J at the node
+  for (int e0 = tid; e0 < 8 * N; e0 += nt) {
     const int b = e0 >> 3, c = e0 & 7, e = eoff + e0;
     const int dx = c & 1, dy = (c >> 1) & 1, dz = (c >> 2) & 1;
     R fr[3];
@@ -1270,7 +1599,7 @@ __device__ __forceinline__ void bead_step_block(const S* __restrict__ pop, const
   __syncthreads();
 
   // 4. friction + Langevin force, second half kick
-  for (int b = b0 + tid; b < b1; b += nt) {
+  for (int b = tid; b < N; b += nt) {
     R ub[3] = {R(0), R(0), R(0)};
     for (int c = 0; c < 8; ++c) {
       const int e = eoff + 8 * b + c;
@@ -1285,238 +1614,131 @@ __device__ __forceinline__ void bead_step_block(const S* __restrict__ pop, const
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       const int t = 3 * b + q;
-      const R vh = vhp[t];
+      const R vh = C.vh[t];
       const R fc = -C.zeta * (vh - ub[q] * C.u_scale) + C.amp * g[q];
       const R Ft = C.fcons[t] + fc;
       C.Fc[t] = fc;
       C.fc_hist[sub * 3 * N + t] = fc;
       C.F[t] = Ft;
-      const R vn = vh + h * Ft / (R(2) * C.m);
+      const R vn = vh + over_2m(h * Ft, C);
       C.v[t] = vn;
       if (C.snap && sub == C.nsub - 1) {  // the step's end state, as the bead read-back forms it
         double* sn = C.snap + (size_t)(step & 1u) * 6 * N;
-        const int im = G > 1 ? simg[t] : C.img[t];
+        const int im = C.img[t];
         sn[t] = __dadd_rn(__dadd_rn((double)sx[t], (double)sl[t]), __dmul_rn((double)im, C.snap_box));
         sn[3 * N + t] = (double)vn;
       }
     }
   }
   __syncthreads();
-  if (G > 1) cluster_sync();  // every bead is done
   }  // substeps
 
-  // 5. deterministic spreading: group the corner entries by node, sum each node's
-  //    contributions in entry order, then turn the node force into population corrections.
-  //    Up to kGroupHashMax entries the grouping uses a hash table in shared memory; the
-  //    table's slots number the nodes of the pending list (that order depends on the table
-  //    layout; no value does).  Beyond, a bitonic sort of (node, entry) keys.
+  // 5. deterministic spreading: order the corner entries by node, sum each node's contributions in
+  //    entry order, then turn the node force into population corrections
   const int ne = 8 * N * C.nsub;
   const int lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
-  if (ne <= kGroupHashMax) {
-    int H = 64;
-    while (H < 2 * ne) H <<= 1;
-    int* tkey = reinterpret_cast<int*>(smem);  // node of the slot, -1 = empty
-    int* tcnt = tkey + H;                       // entries of the slot, then the fill cursor
-    int* toff = tcnt + H;                       // first list position of the slot's entries
-    int* lslot = toff + H;                      // slot of the u-th node of the pending list
-    int* eslot = lslot + H;                     // slot of each entry
-    int* elist = eslot + ne;                    // entries grouped by slot
-    int* wsum = elist + ne;                     // scan scratch: 2 x 32 warp totals, node count
-    if (rank == 0) {  // block 0 groups the entries
-      for (int h = tid; h < H; h += nt) {
-        tkey[h] = -1;
-        tcnt[h] = 0;
-      }
-      __syncthreads();
-      for (int e = tid; e < ne; e += nt) {
-        const int node = C.e_node[e];
-        unsigned h = hash_node(node, (unsigned)H - 1);
-        for (int it = 0; it < H; ++it) {  // at most half full: a free slot or the node is found
-          const int old = atomicCAS(&tkey[h], -1, node);
-          if (old == -1 || old == node) break;
-          h = (h + 1) & (unsigned)(H - 1);
-        }
-        eslot[e] = (int)h;
-        atomicAdd(&tcnt[h], 1);
-      }
-      __syncthreads();
-      // exclusive scans over the slots, in slot order: list offsets and node numbers.  Each
-      // thread owns a contiguous run of slots; warp scans, then a scan of the warp totals.
-      {
-        const int per = (H + nt - 1) / nt;
-        const int h0 = tid * per < H ? tid * per : H, h1 = h0 + per < H ? h0 + per : H;
-        int sc = 0, sl = 0;
-        for (int h = h0; h < h1; ++h) {
-          sc += tcnt[h];
-          sl += tcnt[h] > 0;
-        }
-        int ic = sc, il = sl;
+  int M = 32;  // at least one warp-wide chunk; padding keys sort to the end
+  while (M < ne) M <<= 1;
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem);
+  for (int i = tid; i < M; i += nt)
+    keys[i] = (i < ne) ? (((unsigned long long)(unsigned)C.e_node[i] << 32) | (unsigned)i) : ~0ull;
+  __syncthreads();
+  bitonic_sort_block(keys, M, tid, nt);
+  // leaders: first entry of each node run, numbered in order (chunks of 32 entries: each
+  // warp counts the leaders of its chunks, warp 0 scans the chunk counts)
+  int* slot = reinterpret_cast<int*>(keys + M);
+  int* cbase = slot + ne;
+  const int nchunk = (ne + 31) >> 5;
+  for (int c = warp; c < nchunk; c += nwarp) {
+    const int i = (c << 5) + lane;
+    const int lead = i < ne && ((i == 0) || ((keys[i] >> 32) != (keys[i - 1] >> 32)));
+    const unsigned mask = __ballot_sync(0xffffffffu, lead);
+    if (lane == 0) cbase[c] = __popc(mask);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int base = 0;
+    for (int c0 = 0; c0 < nchunk; c0 += 32) {
+      const int c = c0 + lane;
+      const int v = c < nchunk ? cbase[c] : 0;
+      int incl = v;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int yc = __shfl_up_sync(0xffffffffu, ic, o), yl = __shfl_up_sync(0xffffffffu, il, o);
-          if (lane >= o) {
-            ic += yc;
-            il += yl;
-          }
-        }
-        if (lane == 31) {
-          wsum[warp] = ic;
-          wsum[32 + warp] = il;
-        }
-        __syncthreads();
-        if (warp == 0) {
-          const int vc = lane < nwarp ? wsum[lane] : 0, vl = lane < nwarp ? wsum[32 + lane] : 0;
-          int jc = vc, jl = vl;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int yc = __shfl_up_sync(0xffffffffu, jc, o), yl = __shfl_up_sync(0xffffffffu, jl, o);
-            if (lane >= o) {
-              jc += yc;
-              jl += yl;
-            }
-          }
-          if (lane < nwarp) {
-            wsum[lane] = jc - vc;
-            wsum[32 + lane] = jl - vl;
-          }
-          if (lane == 31) {
-            *Pd.cur_count = jl;
-            wsum[64] = jl;
-          }
-        }
-        __syncthreads();
-        int bc = wsum[warp] + ic - sc, bl = wsum[32 + warp] + il - sl;
-        for (int h = h0; h < h1; ++h) {
-          const int c = tcnt[h];
-          toff[h] = bc;
-          if (c > 0) lslot[bl] = h;
-          tcnt[h] = bc;  // fill cursor
-          bc += c;
-          bl += c > 0;
-        }
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
       }
-      __syncthreads();
-      for (int e = tid; e < ne; e += nt) elist[atomicAdd(&tcnt[eslot[e]], 1)] = e;
-      __syncthreads();
-      for (int u = tid; u < wsum[64]; u += nt) {  // each node's entries in entry order
-        const int h = lslot[u];
-        const int base = toff[h], cnt = tcnt[h] - base;
-        for (int r = base + 1; r < base + cnt; ++r) {  // (insertion sort of a short list)
-          const int e = elist[r];
-          int q = r - 1;
-          while (q >= base && elist[q] > e) {
-            elist[q + 1] = elist[q];
-            --q;
-          }
-          elist[q + 1] = e;
-        }
-      }
-    }  // block 0
-    __syncthreads();
-    if (G > 1) cluster_sync();  // block 0's table is complete
-    // the table of block 0, read by every block of the cluster (distributed shared memory)
-    const int* tk = G > 1 ? cluster_rank0(tkey) : tkey;
-    const int* to = G > 1 ? cluster_rank0(toff) : toff;
-    const int* tc = G > 1 ? cluster_rank0(tcnt) : tcnt;
-    const int* ls = G > 1 ? cluster_rank0(lslot) : lslot;
-    const int* el = G > 1 ? cluster_rank0(elist) : elist;
-    const int nnode = (G > 1 ? cluster_rank0(wsum) : wsum)[64];
-    const int u0 = rank * nnode / G, u1 = (rank + 1) * nnode / G;  // this block's nodes
-    for (int u = u0 + tid; u < u1; u += nt) {  // one thread per node, in list order
-      const int h = ls[u];
-      const int base = to[h], cnt = tc[h] - base;
-      node_correction<R>(P, C, Pd, L, N, u, tk[h], [&](int r) { return el[r]; }, base, cnt);
+      if (c < nchunk) cbase[c] = base + incl - v;
+      base += __shfl_sync(0xffffffffu, incl, 31);
     }
-    if (G > 1) cluster_sync();  // block 0's table is read until here
-  } else {  // (one block: the host launches G = 1 beyond kGroupHashMax entries)
-    if (rank != 0) return;
-    int M = 32;  // at least one warp-wide chunk; padding keys sort to the end
-    while (M < ne) M <<= 1;
-    unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem);
-    for (int i = tid; i < M; i += nt)
-      keys[i] = (i < ne) ? (((unsigned long long)(unsigned)C.e_node[i] << 32) | (unsigned)i) : ~0ull;
-    __syncthreads();
-    bitonic_sort_block(keys, M, tid, nt);
-    // leaders: first entry of each node run, numbered in order (chunks of 32 entries: each
-    // warp counts the leaders of its chunks, warp 0 scans the chunk counts)
-    int* slot = reinterpret_cast<int*>(keys + M);
-    int* cbase = slot + ne;
-    const int nchunk = (ne + 31) >> 5;
-    for (int c = warp; c < nchunk; c += nwarp) {
-      const int i = (c << 5) + lane;
-      const int lead = i < ne && ((i == 0) || ((keys[i] >> 32) != (keys[i - 1] >> 32)));
-      const unsigned mask = __ballot_sync(0xffffffffu, lead);
-      if (lane == 0) cbase[c] = __popc(mask);
+    if (lane == 0) *Pd.cur_count = base;
+  }
+  __syncthreads();
+  for (int c = warp; c < nchunk; c += nwarp) {
+    const int i = (c << 5) + lane;
+    const int lead = i < ne && ((i == 0) || ((keys[i] >> 32) != (keys[i - 1] >> 32)));
+    const unsigned mask = __ballot_sync(0xffffffffu, lead);
+    if (i < ne) slot[i] = lead ? cbase[c] + __popc(mask & ((1u << lane) - 1u)) : -1;
+  }
+  __syncthreads();
+  for (int i = tid; i < ne; i += nt) {
+    const int u = slot[i];
+    if (u < 0) continue;
+    const int node = (int)(keys[i] >> 32);
+    int cnt = 1;
+    while (i + cnt < ne && (int)(keys[i + cnt] >> 32) == node) ++cnt;
+    const int e0 = (int)(keys[i] & 0xffffffffu);
+    R f[3] = {R(0), R(0), R(0)};
+    for (int r = i; r < i + cnt; ++r) {
+      const int e = (int)(keys[r] & 0xffffffffu);
+      const R w = C.e_w[e] * C.spread;
+      const int sub = e / (8 * N), b = (e - sub * 8 * N) >> 3;
+      const R* fch = C.fc_hist + sub * 3 * N;
+      f[0] -= w * fch[3 * b + 0] * C.inv_a3;
+      f[1] -= w * fch[3 * b + 1] * C.inv_a3;
+      f[2] -= w * fch[3 * b + 2] * C.inv_a3;
     }
-    __syncthreads();
-    if (warp == 0) {
-      int base = 0;
-      for (int c0 = 0; c0 < nchunk; c0 += 32) {
-        const int c = c0 + lane;
-        const int v = c < nchunk ? cbase[c] : 0;
-        int incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += y;
-        }
-        if (c < nchunk) cbase[c] = base + incl - v;
-        base += __shfl_sync(0xffffffffu, incl, 31);
-      }
-      if (lane == 0) *Pd.cur_count = base;
-    }
-    __syncthreads();
-    for (int c = warp; c < nchunk; c += nwarp) {
-      const int i = (c << 5) + lane;
-      const int lead = i < ne && ((i == 0) || ((keys[i] >> 32) != (keys[i - 1] >> 32)));
-      const unsigned mask = __ballot_sync(0xffffffffu, lead);
-      if (i < ne) slot[i] = lead ? cbase[c] + __popc(mask & ((1u << lane) - 1u)) : -1;
-    }
-    __syncthreads();
-    for (int i = tid; i < ne; i += nt) {
-      const int u = slot[i];
-      if (u < 0) continue;
-      const int node = (int)(keys[i] >> 32);
-      int cnt = 1;
-      while (i + cnt < ne && (int)(keys[i + cnt] >> 32) == node) ++cnt;
-      node_correction<R>(P, C, Pd, L, N, u, node, [&](int r) { return (int)(keys[r] & 0xffffffffu); }, i, cnt);
-    }
+    node_correction<R>(P, C, Pd, L, u, node, f, C.e_mom[e0], C.e_mom[C.cap + e0], C.e_mom[2 * C.cap + e0],
+                       C.e_mom[3 * C.cap + e0]);
   }
 }
 
-// The bead step as its own grid.  Launched with programmatic stream serialization
-// after the previous step's LB kernel (which completes only after the previous bead kernel),
-// it waits for that grid before reading; then it releases the LB kernel of the same step,
-// which reads neither its outputs nor anything it writes and runs alongside.
-// The grid is one cluster of G blocks (G = 1: a single block).
-template <class S, class R, bool DEV>
+// The bead step as its own grid (one cluster of G blocks; SORTED: one block).  Launched with
+// programmatic stream serialization after the previous step's LB kernel (which completes only
+// after the previous bead kernel), it waits for that grid before reading; then it releases the LB
+// kernel of the same step, which reads neither its outputs nor anything it writes and runs
+// alongside.
+template <class S, class R, bool DEV, bool SORTED>
 __global__ void __launch_bounds__(512) k_bead_step(const S* __restrict__ pop, const FluidK<R> P,
                                                     const ChainK<R> C, const PendK<R> Pd, const uint32_t step) {
   extern __shared__ __align__(16) unsigned char smem[];
-  unsigned rank, G;
-  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(G));
-  grid_dependency_wait();
-  allow_dependent_launch();
-  bead_step_block<S, R, DEV>(pop, P, C, Pd, launch_step(P, step), smem, (int)rank, (int)G);
+  if constexpr (SORTED) {
+    grid_dependency_wait();
+    allow_dependent_launch();
+    bead_step_sorted<S, R, DEV>(pop, P, C, Pd, launch_step(P, step), smem);
+  } else {
+    unsigned rank, G;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(G));
+    bead_step_block<S, R, DEV, true>(pop, P, C, Pd, launch_step(P, step), smem, (int)rank, (int)G);
+  }
 }
 
-// B[i][node] += dn_i at every pending node (each node appears once in the list), and the
-// applied entries of the dense correction field and the list's mask words (mask may be null)
-// back to zero; one thread per (node, population): blockIdx.y is the population
+// B[i][node] += the dense field's corrections at every listed node (each appears once in the list),
+// and those entries and the list's mask words (mask may be null) back to zero; one thread per
+// (list entry, population): blockIdx.y is the population
 template <class S, class R>
 __global__ void __launch_bounds__(256) k_apply_pending(S* __restrict__ pop, const FluidK<R> P,
                                                         const int4* __restrict__ p_pos,
-                                                        const R* __restrict__ p_dn,
-                                                        const int* __restrict__ p_count, int cap,
+                                                        const int* __restrict__ p_count,
                                                         R* __restrict__ dense, unsigned* __restrict__ mask,
                                                         unsigned seg0) {
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
   if (u >= *p_count) return;
   const int i = blockIdx.y;
   const int4 p = p_pos[u];
+  if (p.x < 0) return;
   const unsigned long long off = (unsigned long long)i * P.plane + (unsigned)p.x;
-  st<S, R>(pop + off, ld<S, R>(pop + off) + p_dn[i * cap + u]);
+  st<S, R>(pop + off, ld<S, R>(pop + off) + dense[off]);
   dense[off] = R(0);
   if (mask && i == 0) clear_marks(mask, seg0, (int)P.L, p.y, p.z, p.w);
 }
@@ -1763,7 +1985,7 @@ __global__ void __launch_bounds__(512) k_chain_init_forces(const ChainK<R> C) {
     sl[t] = C.xl[t];
   }
   __syncthreads();
-  chain_forces_block<R>(sx, sl, C, C.F, 0, C.N);
+  chain_forces_block<R>(sx, sl, C, C.F);
   __syncthreads();
   for (int t = threadIdx.x; t < 3 * C.N; t += blockDim.x) C.Fc[t] = R(0);
 }

@@ -60,8 +60,7 @@ class EngineT final : public Engine {
     }
     if (own_tables_) launch_fill_noise_tables(noise_tab_, s);
     if (bead_smem() > 48 * 1024)
-      cuda_check(cudaFuncSetAttribute(k_bead_step<S, R, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)bead_smem()),
+      cuda_check(cudaFuncSetAttribute(bead_kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bead_smem()),
                  "bead kernel shared memory");
     const unsigned long long nb = (nnodes_ + 255) / 256;
     k_init_rest<S, R, DEV><<<(unsigned)nb, 256, 0, s>>>(pop_[0], nnodes_, plane_, (R)cfg_.rho);
@@ -491,11 +490,11 @@ class EngineT final : public Engine {
   int pending_capacity() const { return cap_; }
   // pending-correction lists of slot j (the batched driver keeps its own slot order)
   int4* pending_pos(int j) const { return p_pos_[j]; }
-  R* pending_dn(int j) const { return p_dn_[j]; }
   int* pending_count(int j) const { return p_count_[j]; }
   R* pending_dense(int j) const { return corr_[j]; }
   unsigned long long plane() const { return plane_; }
-  size_t bead_smem_bytes() const { return bead_smem(); }
+  size_t bead_smem_bytes(int G) const { return bead_smem_for(G); }
+  bool sorted_beads() const { return bead_sorted(); }
   int chain_length() const { return N_; }
   const Config& config() const { return cfg_; }
 
@@ -733,7 +732,7 @@ class EngineT final : public Engine {
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof(lc));
     lc.gridDim = dim3((unsigned)G);
-    lc.blockDim = dim3(512);
+    lc.blockDim = dim3(kBeadThreads);
     lc.dynamicSmemBytes = bead_smem();
     lc.stream = s;
     cudaLaunchAttribute at[2];
@@ -750,7 +749,7 @@ class EngineT final : public Engine {
     }
     lc.attrs = at;
     lc.numAttrs = (unsigned)na;
-    cuda_check(cudaLaunchKernelEx(&lc, k_bead_step<S, R, DEV>, A, P, Cover ? *Cover : chain(), Pd, k), "bead kernel");
+    cuda_check(cudaLaunchKernelEx(&lc, bead_kernel(), A, P, Cover ? *Cover : chain(), Pd, k), "bead kernel");
     cuda_check(cudaGetLastError(), "bead kernel");
   }
 
@@ -791,9 +790,8 @@ class EngineT final : public Engine {
   }
 
   void apply(S* buf, const FluidK<R>& P, int slot, cudaStream_t s) {
-    k_apply_pending<S, R><<<dim3((cap_ + 255) / 256, Q), 256, 0, s>>>(buf, P, p_pos_[slot], p_dn_[slot],
-                                                                     p_count_[slot], cap_, corr_[slot],
-                                                                     masks_[slot], 0u);
+    k_apply_pending<S, R><<<dim3((cap_ + 255) / 256, Q), 256, 0, s>>>(buf, P, p_pos_[slot], p_count_[slot],
+                                                                     corr_[slot], masks_[slot], 0u);
     cuda_check(cudaGetLastError(), "apply kernel");
   }
 
@@ -809,7 +807,6 @@ class EngineT final : public Engine {
     Pd.cur_dense = corr_[c];
     Pd.plane = plane_;
     Pd.cur_pos = p_pos_[c];
-    Pd.cur_dn = p_dn_[c];
     Pd.cur_count = p_count_[c];
     Pd.cur_mask = masks_[c];
     Pd.mark = deferred ? 1 : 0;
@@ -912,31 +909,38 @@ class EngineT final : public Engine {
     grd = dim3((row + bx - 1) / bx, ((unsigned)L_ + by - 1) / by, (unsigned)L_);
   }
 
-  size_t bead_smem() const {
-    // phase 5: up to kGroupHashMax entries a node table (4 x H ints, H >= 2 x entries), entry
-    // slots and lists and scan scratch; beyond, sort keys, leader slots and chunk counts
-    const size_t ne = 8 * (size_t)N_ * nsub_;
-    size_t groupb;
-    if (ne <= (size_t)kGroupHashMax) {
-      size_t H = 64;
-      while (H < 2 * ne) H <<= 1;
-      groupb = (4 * H + 2 * ne + 65) * sizeof(int);
-    } else {
-      size_t M = 32;
-      while (M < ne) M <<= 1;
-      groupb = M * 8 + ne * 4 + ((ne + 31) / 32) * 4;
-    }
-    // positions (hi, lo); in a cluster also half-step velocities and image counters
-    const size_t posb = bead_cluster() > 1 ? 9 * (size_t)N_ * sizeof(R) + 3 * (size_t)N_ * sizeof(int)
-                                           : 6 * (size_t)N_ * sizeof(R);
-    return groupb > posb ? groupb : posb;
+  // threads of a bead block: measured 11.0 against 10.6 us per step with 256 at L = 25, N = 32, two
+  // substeps (FP32), 17.6 against 16.4 us with 512 at L = 16, N = 8 (FP64, whose pipe the additional
+  // warps do not help)
+  static constexpr int kBeadThreads = sizeof(R) == 8 ? 256 : 512;
+  bool bead_sorted() const { return 8 * (size_t)N_ * nsub_ > (size_t)kGroupMax; }
+  using BeadKernel = void (*)(const S*, const FluidK<R>, const ChainK<R>, const PendK<R>, const uint32_t);
+  BeadKernel bead_kernel() const {
+    return bead_sorted() ? k_bead_step<S, R, DEV, true> : k_bead_step<S, R, DEV, false>;
   }
 
-  // Blocks of the bead kernel's cluster: one per 16 beads, at most 8 (the portable cluster
-  // size); one block when the entries need the sorted grouping
+  // shared memory of the bead step by clusters of G blocks
+  size_t bead_smem_for(int G) const {
+    if (!bead_sorted()) {
+      BeadSmem<R> M;
+      return M.carve(nullptr, N_, nsub_, (N_ + G - 1) / G);
+    }
+    // positions; later sort keys, leader slots and chunk counts
+    const size_t ne = 8 * (size_t)N_ * nsub_;
+    size_t M = 32;
+    while (M < ne) M <<= 1;
+    const size_t groupb = M * 8 + ne * 4 + ((ne + 31) / 32) * 4, posb = 6 * (size_t)N_ * sizeof(R);
+    return groupb > posb ? groupb : posb;
+  }
+  size_t bead_smem() const { return bead_smem_for(bead_cluster()); }
+
+  // Blocks of the bead kernel's cluster: one per kBeadsPerBlock beads, at most 8 (the portable
+  // cluster size); one block when the entries need the sorted grouping.  (8 beads per block: 11.8
+  // against 10.6 us per step at L = 25, N = 32, two substeps; 2 per block: the same.)
+  static constexpr int kBeadsPerBlock = sizeof(R) == 8 ? 2 : 4;
   int bead_cluster() const {
-    if (8 * (size_t)N_ * nsub_ > (size_t)kGroupHashMax) return 1;
-    const int g = N_ / 16;
+    if (bead_sorted()) return 1;
+    const int g = (N_ + kBeadsPerBlock - 1) / kBeadsPerBlock;
     return g < 1 ? 1 : (g > 8 ? 8 : g);
   }
 
@@ -1000,6 +1004,9 @@ class EngineT final : public Engine {
     C.rc2 = (R)(pow(2.0, 1.0 / 3.0) * c.sigma * c.sigma);
     C.h = (R)(c.h / nsub_);  // the MD step
     C.a = (R)c.a;
+    int e2;
+    C.inv_2m = frexp(2.0 * c.m, &e2) == 0.5 ? (R)(1.0 / (2.0 * c.m)) : (R)0;
+    C.inv_a = frexp(c.a, &e2) == 0.5 ? (R)(1.0 / c.a) : (R)0;
     C.box = (R)(c.L * c.a);
     C.half_box = (R)(0.5 * c.L * c.a);
     const bool noise = c.noise_beads && c.kT > 0.0;
@@ -1029,9 +1036,6 @@ class EngineT final : public Engine {
     C.e_node = e_node_;
     C.e_w = e_w_;
     C.e_mom = e_mom_;
-    C.p_pos = p_pos_[0];
-    C.p_dn = p_dn_[0];
-    C.p_count = p_count_[0];
     C.cap = cap_;
     C.status = status_;
     C.snap = N_ > 0 ? snap_ : nullptr;
@@ -1096,7 +1100,6 @@ class EngineT final : public Engine {
     e_mom_ = reinterpret_cast<R*>(take(4 * cap_ * sizeof(R)));
     for (int j = 0; j < 2; ++j) {
       p_pos_[j] = reinterpret_cast<int4*>(take(cap_ * sizeof(int4)));
-      p_dn_[j] = reinterpret_cast<R*>(take((size_t)Q * cap_ * sizeof(R)));
       p_count_[j] = reinterpret_cast<int*>(take(sizeof(int)));
       masks_[j] = reinterpret_cast<unsigned*>(take(nsegs() * sizeof(unsigned)));
       corr_[j] = N_ > 0 ? reinterpret_cast<R*>(take((size_t)Q * plane_ * sizeof(R))) : nullptr;
@@ -1134,7 +1137,6 @@ class EngineT final : public Engine {
   int* e_node_ = nullptr;
   R *e_w_ = nullptr, *e_mom_ = nullptr;
   int4* p_pos_[2] = {nullptr, nullptr};
-  R* p_dn_[2] = {nullptr, nullptr};
   int* p_count_[2] = {nullptr, nullptr};
   unsigned* masks_[2] = {nullptr, nullptr};  // marks of the nodes that pull from pending nodes, by slot
   R* corr_[2] = {nullptr, nullptr};     // dense correction fields [i][plane], zero but at pending nodes

@@ -192,7 +192,7 @@ struct NoiseTab {
   const double2* angle;  // (cos, sin)(2 pi (u1 - 1/2)), u1 = (k + 1/2) 2^-11, k < 2048
 };
 constexpr unsigned kRadii = 1u << 21, kAngles = 1u << 11;
-__global__ inline void fill_noise_tables(double* radius, double2* angle) {
+static __global__ void fill_noise_tables(double* radius, double2* angle) {
   for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < kRadii; k += gridDim.x * blockDim.x) {
     radius[k] = sqrt(-2.0 * log(((double)k + 0.5) * 0x1p-21));
     if (k < kAngles) {
