@@ -8,6 +8,7 @@
 #include <memory>
 #include <string>
 #include <utility>
+#include <algorithm>
 #include <vector>
 
 #include "../../include/lb.h"
@@ -348,17 +349,26 @@ int lb_step(lb_ctx* ctx, int64_t n) {
   if (!ctx || n < 0) return fail(LB_ERR_ARG, "invalid argument: !ctx || n < 0");
   return guarded([&] {
     materialise(ctx);
-    for (int64_t t = 0; t < n; ++t) {
-      cudaEvent_t e0 = nullptr, e1 = nullptr;
+    for (int64_t t = 0; t < n;) {
+      // steps up to the next one that something follows: a sample, a frame, a timing event
+      int64_t m = n - t;
+      auto until = [&](int64_t done, int64_t stride) { m = std::min(m, stride - done % stride); };
+      const bool sample = ctx->obs_stride > 0 && ctx->cfg.N > 0;
+      if (sample) until(ctx->step, ctx->obs_stride);
+      if (ctx->traj) until(ctx->step - ctx->traj_origin, ctx->traj_stride);
       if (ctx->timing) {
+        m = 1;
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
         cuda_check(cudaEventCreate(&e0), "event");
         cuda_check(cudaEventCreate(&e1), "event");
         ctx->evs.emplace_back(e0, e1);
+        ctx->eng->step_deferred((uint32_t)ctx->step, ctx->stream, e0, e1);
+      } else {
+        ctx->eng->steps_deferred((uint32_t)ctx->step, m, ctx->stream);
       }
-      ctx->eng->step_deferred((uint32_t)ctx->step, ctx->stream, e0, e1);
-      ctx->step += 1;
-      if (ctx->obs_stride > 0 && ctx->cfg.N > 0 && ctx->step % ctx->obs_stride == 0)
-        ctx->eng->observables(nullptr, ctx->step, 1, ctx->stream);
+      t += m;
+      ctx->step += m;
+      if (sample && ctx->step % ctx->obs_stride == 0) ctx->eng->observables(nullptr, ctx->step, 1, ctx->stream);
       if (ctx->traj && (ctx->step - ctx->traj_origin) % ctx->traj_stride == 0) record_frame(ctx);
     }
     // the last step's force correction stays pending: every call that reads or replaces the

@@ -135,6 +135,8 @@ __device__ __forceinline__ uint32_t launch_step(const FluidK<R>& P, uint32_t ste
 // *p = v on the stream (a device step counter before a graph replay)
 template <class T>
 __global__ void k_store_value(T* p, T v) { *p = v; }
+template <class T>
+__global__ void k_add_value(T* p, T v) { *p += v; }
 
 template <class R>
 struct ChainK {

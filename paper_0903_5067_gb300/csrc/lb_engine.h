@@ -58,6 +58,8 @@ class Engine {
   // one step whose bead force correction stays pending until the next deferred step reads
   // it or flush() applies it; every other method flushes first
   virtual void step_deferred(uint32_t k, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1) = 0;
+  // n such steps k .. k + n - 1, as CUDA graphs of several steps where there are enough
+  virtual void steps_deferred(uint32_t k, int64_t n, cudaStream_t s) = 0;
   virtual void flush(cudaStream_t s) = 0;
   virtual void get_populations(double* out, cudaStream_t s) = 0;
   virtual void set_populations(const double* in, cudaStream_t s) = 0;

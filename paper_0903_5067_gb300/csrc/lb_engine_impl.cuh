@@ -43,9 +43,15 @@ class EngineT final : public Engine {
 
   size_t workspace_bytes() const override { return bytes_; }
 
-  void bind(void* base) override { layout(static_cast<unsigned char*>(base)); }
+  void bind(void* base) override {
+    drop_graphs();
+    layout(static_cast<unsigned char*>(base));
+  }
 
-  void set_config(const Config& c) override { cfg_ = c; }
+  void set_config(const Config& c) override {
+    drop_graphs();
+    cfg_ = c;
+  }
   void set_noise_tables(void* base) { noise_tab_ = base; }
 
   void initialise(const double* x0, const double* v0, cudaStream_t s) override {
@@ -132,11 +138,17 @@ class EngineT final : public Engine {
   // the LB kernel of step k, released early, touches nothing the bead kernel of step k
   // reads or writes.
   void step_deferred(uint32_t k, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1) override {
+    step_deferred(k, s, ev0, ev1, nullptr);
+  }
+  // d_step: a device counter the kernels add k to (null: k is the step number)
+  void step_deferred(uint32_t k, cudaStream_t s, cudaEvent_t ev0, cudaEvent_t ev1, const uint32_t* d_step) {
+    FluidK<R> P = fluid();
+    P.d_step = d_step;
     if (N_ == 0) {
-      step(k, s, ev0, ev1);
+      launch_lb(pop_[cur_], pop_[cur_ ^ 1], P, pend(false), k, s, ev0, ev1);
+      cur_ ^= 1;
       return;
     }
-    const FluidK<R> P = fluid();
     const S* A = pop_[cur_];
     S* Bo = pop_[cur_ ^ 1];
     if (open_) pslot_ ^= 1;
@@ -147,6 +159,37 @@ class EngineT final : public Engine {
     launch_lb(A, Bo, P, Pd, k, s, ev0, ev1);
     open_ = true;
     cur_ ^= 1;
+  }
+
+  // n deferred steps.  Launching a step's two kernels costs the host 17 us (two extended launches
+  // with kilobyte parameter blocks), more than the step of a small box takes the GPU, so kGraphSteps
+  // steps are captured once as a CUDA graph, whose kernels add their place in it to a device
+  // counter, and replayed: 16 steps leave the buffers and correction slots as they found them, so
+  // there is one graph per state of the two.  Capturing and instantiating one costs about as
+  // much as 30 launched steps: only calls of kGraphFirst steps start one.  A stream that is being
+  // captured gets the launches themselves.
+  void steps_deferred(uint32_t k, int64_t n, cudaStream_t s) override {
+    int64_t t = 0;
+    if (n > kGraphSteps && graphs_usable(s)) {
+      if (N_ > 0 && !open_) step_deferred(k + (uint32_t)t++, s, nullptr, nullptr);  // the first has nothing pending
+      cudaGraphExec_t& g = graph_[cur_][pslot_];
+      if (!g && n >= kGraphFirst) g = capture_steps();
+      if (g) {
+        for (int j = 0; j < 2; ++j)
+          if (snap_pending_[j]) {  // the graph rewrites both snapshot slots
+            cuda_check(cudaStreamWaitEvent(s, copy_ev_[j], 0), "wait read-back");
+            snap_pending_[j] = false;
+          }
+        k_store_value<uint32_t><<<1, 1, 0, s>>>(d_step_, k + (uint32_t)t);
+        cuda_check(cudaGetLastError(), "step counter");
+        for (; n - t >= kGraphSteps; t += kGraphSteps) cuda_check(cudaGraphLaunch(g, s), "step graph");
+        if (N_ > 0) {
+          snap_valid_ = true;
+          snap_k_ = k + (uint32_t)t - 1;
+        }
+      }
+    }
+    for (; t < n; ++t) step_deferred(k + (uint32_t)t, s, nullptr, nullptr);
   }
 
   // One complete step with the bead kernel's state arrays given (the adjoint's recomputation:
@@ -606,6 +649,8 @@ class EngineT final : public Engine {
   }
 
   ~EngineT() override {
+    drop_graphs();
+    if (capture_) cudaStreamDestroy(capture_);
     if (side_) {
       cudaStreamSynchronize(side_);
       cudaStreamDestroy(side_);
@@ -717,6 +762,72 @@ class EngineT final : public Engine {
     mv(acc_, 4 * sizeof(double));
     mv(nonpos_, sizeof(unsigned long long));
     return p;
+  }
+
+  static constexpr int kGraphSteps = 16;  // even: buffers and slots alternate
+  static constexpr int64_t kGraphFirst = 48;
+
+  // whether work for s may go through a graph launch: not while s is being captured
+  bool graphs_usable(cudaStream_t s) const {
+    if (graphs_off_) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return st == cudaStreamCaptureStatusNone;
+  }
+
+  // kGraphSteps deferred steps from the present buffers and slots as an executable graph; null (and
+  // no further attempt) when the driver refuses one
+  cudaGraphExec_t capture_steps() {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // whatever the calling thread captures
+    cuda_check(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t ge = nullptr;
+    cudaError_t e = capture_ ? cudaSuccess : cudaStreamCreateWithFlags(&capture_, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(capture_, cudaStreamCaptureModeRelaxed);
+    if (e == cudaSuccess) {
+      const bool pending[2] = {snap_pending_[0], snap_pending_[1]};
+      const bool valid = snap_valid_;
+      const uint32_t sk = snap_k_;
+      const int cur = cur_, slot = pslot_;
+      const bool open = open_;
+      snap_pending_[0] = snap_pending_[1] = false;  // waited for at the replay
+      bool ok = true;
+      try {
+        for (int j = 0; j < kGraphSteps; ++j) step_deferred((uint32_t)j, capture_, nullptr, nullptr, d_step_);
+        k_add_value<uint32_t><<<1, 1, 0, capture_>>>(d_step_, (uint32_t)kGraphSteps);
+      } catch (const LbError&) {
+        ok = false;
+      }
+      snap_pending_[0] = pending[0];
+      snap_pending_[1] = pending[1];
+      snap_valid_ = valid;
+      snap_k_ = sk;
+      cur_ = cur;
+      pslot_ = slot;
+      open_ = open;
+      e = cudaStreamEndCapture(capture_, &g);
+      if (e == cudaSuccess && ok) e = cudaGraphInstantiate(&ge, g, 0);
+      if (g) cudaGraphDestroy(g);
+      if (!ok) e = cudaErrorUnknown;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      graphs_off_ = true;
+      return nullptr;
+    }
+    return ge;
+  }
+
+  void drop_graphs() {
+    for (auto& gs : graph_)
+      for (cudaGraphExec_t& g : gs) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+      }
   }
 
   // Bead kernel of step k: one cluster of bead_cluster() blocks; with `chained`, launched with
@@ -1105,6 +1216,7 @@ class EngineT final : public Engine {
       corr_[j] = N_ > 0 ? reinterpret_cast<R*>(take((size_t)Q * plane_ * sizeof(R))) : nullptr;
     }
     status_ = reinterpret_cast<unsigned*>(take(sizeof(unsigned)));
+    d_step_ = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t)));
     nonpos_ = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long)));
     acc_ = reinterpret_cast<double*>(take(4 * sizeof(double)));
     obs_ = reinterpret_cast<double*>(take(kNObs * sizeof(double)));
@@ -1143,6 +1255,11 @@ class EngineT final : public Engine {
   int pslot_ = 0;
   bool open_ = false;  // a deferred step's correction is pending
   unsigned* status_ = nullptr;
+  // graphs of kGraphSteps deferred steps by cur_ and pslot_, their step counter, the capture's stream
+  cudaGraphExec_t graph_[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+  uint32_t* d_step_ = nullptr;
+  cudaStream_t capture_ = nullptr;
+  bool graphs_off_ = false;
   unsigned long long* nonpos_ = nullptr;
   double *acc_ = nullptr, *obs_ = nullptr, *parts_ = nullptr;
 };
