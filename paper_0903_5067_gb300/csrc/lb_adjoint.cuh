@@ -36,15 +36,15 @@ __device__ __forceinline__ R pair_coef_deriv(R r2, bool bonded, const ChainK<R>&
 }
 
 // xbar_b += sum_j [coef I + 2 coef' d d^T] (Fbar_b - Fbar_j): the chain-force Hessian applied
-// to the force adjoint.  Positions in shared memory (hi, lo); lanes per bead as in
-// chain_forces_block; the result is added to out.
+// to the force adjoint.  Positions in shared memory (hi, lo); by nt threads (whole warps; tid: this
+// one's number among them), lanes per bead as in chain_forces_block; the result is added to out.
 template <class R>
 __device__ __forceinline__ void chain_force_vjp_block(const R* __restrict__ sh, const R* __restrict__ sl,
                                                       const R* __restrict__ fbar, const ChainK<R>& C,
-                                                      R* __restrict__ out) {
-  const int N = C.N, nt = blockDim.x, tid = threadIdx.x;
-  int lanes = 1;
-  while (lanes < 32 && lanes * 2 * N <= nt) lanes *= 2;
+                                                      R* __restrict__ out, const int tid, const int nt) {
+  const int N = C.N;
+  int lanes = 1;  // (more than N lanes would add zeros)
+  while (lanes < 32 && lanes < N && lanes * 2 * N <= (int)blockDim.x) lanes *= 2;
   const int per = nt / lanes;
   const int lane = tid % lanes;
   for (int base = 0; base < N; base += per) {
@@ -200,108 +200,116 @@ __global__ void __launch_bounds__(256) k_adj_lb(const S* __restrict__ state, con
   }
 }
 
-// Chain part of the adjoint of one step, one thread block.
-// In:  bead state of step k (C.x/xl/img/v/F hold it), post-collision populations n*_k
-//      (`state`), lambda(n*_{k+1}) (`lam`), xbar/vbar/fbar of step k+1.
-// Out: xbar/vbar/fbar of step k (in place), zbar (+= d/dzeta), and lambda(n*_k) (`lam_out`)
-//      completed: lambda_k,i(r - e_i) += rho-bar(r) + c_i . J-bar(r) at the forced nodes r.
-// Launched with programmatic stream serialization after k_adj_lb of the same step, which writes
-// the rest of lambda(n*_k): everything up to that last addition runs beside it, and the
-// addition waits for it.
+// What the chain part of the adjoint of a step needs of the forward step alone: for each step of a
+// segment one region of global memory, written by k_adj_prep.
 template <class R>
-struct AdjK {
-  R *xbar, *vbar, *fbar;  // 3N each, in/out across the reverse steps (global)
-  double* zbar;           // accumulated d objective / d zeta (global)
-  // scratch of one reverse step: carved from the kernel's dynamic shared memory at byte
-  // offset smem_off when smem_scratch is set (small chains), else global memory
-  R *vh, *ub, *g, *fc, *fct, *vhb, *xpb;  // 3N each
-  R* e_gw;      // 3 x 8N weight gradients (per unit length)
-  R* e_rb;      // 4 x 8N (rho-bar, J-bar) per entry
-  R* u_fb;      // 3 x cap: f-bar per unique node
-  R* u_rb;      // 4 x cap: forced-node (rho, J) adjoint per unique node
-  R* u_sp;      // 4 x cap: (rho-bar, J-bar) summed per unique forced node
-  R* zb_b;      // N: zeta-bar per bead
-  R* ce_w;      // 8N: trilinear weight of each corner entry
-  R* ce_mom;    // 4 x 8N: post-stream rho and J at each entry's node
-  int* e_slot;  // 8N: unique-node slot of each entry
-  int* u_node;  // cap: the unique forced nodes
-  int* ce_node; // 8N: node of each corner entry
-  int smem_scratch;
-  unsigned smem_off;
+struct AdjPrep {
+  R *vh, *ub, *g, *fc, *sx, *sl;  // 3N each: half-step velocity, fluid velocity, noise, coupling force,
+                                  // drifted position (high, low)
+  R* gw;       // 3 x 8N weight gradients (per unit length) of the corner entries
+  R* w;        // 8N trilinear weights
+  R* mom;      // 4 x 8N post-stream density and momentum at the entries' nodes
+  R* uf;       // 3 x 8N force density on the u-th forced node
+  int* order;  // 8N entries grouped by node, in entry order within a node
+  int* first;  // 8N + 1: the u-th node's entries are order[first[u]] .. order[first[u + 1] - 1]
+  int* slot;   // 8N: the entry's node u
+  int* node;   // 8N: index of the u-th forced node
+  int* nu;     // number of forced nodes
+  __host__ __device__ int carve(unsigned char* base, int N) {  // returns its size, a multiple of 16
+    int off = 0;
+    auto take = [&](int bytes) {
+      unsigned char* q = base + off;
+      off += (bytes + 15) / 16 * 16;
+      return q;
+    };
+    const int r = (int)sizeof(R), n3 = 3 * N, ne = 8 * N;
+    vh = (R*)take(n3 * r);
+    ub = (R*)take(n3 * r);
+    g = (R*)take(n3 * r);
+    fc = (R*)take(n3 * r);
+    sx = (R*)take(n3 * r);
+    sl = (R*)take(n3 * r);
+    gw = (R*)take(3 * ne * r);
+    w = (R*)take(ne * r);
+    mom = (R*)take(4 * ne * r);
+    uf = (R*)take(3 * ne * r);
+    order = (int*)take(ne * 4);
+    first = (int*)take((ne + 1) * 4);
+    slot = (int*)take(ne * 4);
+    node = (int*)take(ne * 4);
+    nu = (int*)take(4);
+    return off;
+  }
 };
 
-// Carve the per-step scratch of AdjK from one region starting at base (16-byte aligned pieces,
-// in a fixed order); returns its size.  base may be null to compute the size only.
+// shared memory of k_adj_prep: positions, sort keys, leader slots
 template <class R>
-__host__ __device__ inline size_t carve_adj_scratch(AdjK<R>& A, unsigned char* base, int N, int cap) {
-  size_t off = 0;
-  auto piece = [&](size_t bytes) {
-    unsigned char* p = base ? base + off : nullptr;
-    off += (bytes + 15) / 16 * 16;
-    return p;
-  };
-  const size_t n3 = 3 * (size_t)N, ne = (size_t)cap;
-  A.vh = reinterpret_cast<R*>(piece(n3 * sizeof(R)));
-  A.ub = reinterpret_cast<R*>(piece(n3 * sizeof(R)));
-  A.g = reinterpret_cast<R*>(piece(n3 * sizeof(R)));
-  A.fc = reinterpret_cast<R*>(piece(n3 * sizeof(R)));
-  A.fct = reinterpret_cast<R*>(piece(n3 * sizeof(R)));
-  A.vhb = reinterpret_cast<R*>(piece(n3 * sizeof(R)));
-  A.xpb = reinterpret_cast<R*>(piece(n3 * sizeof(R)));
-  A.e_gw = reinterpret_cast<R*>(piece(3 * ne * sizeof(R)));
-  A.e_rb = reinterpret_cast<R*>(piece(4 * ne * sizeof(R)));
-  A.u_fb = reinterpret_cast<R*>(piece(3 * ne * sizeof(R)));
-  A.u_rb = reinterpret_cast<R*>(piece(4 * ne * sizeof(R)));
-  A.u_sp = reinterpret_cast<R*>(piece(4 * ne * sizeof(R)));
-  A.zb_b = reinterpret_cast<R*>(piece((size_t)N * sizeof(R)));
-  A.ce_w = reinterpret_cast<R*>(piece(ne * sizeof(R)));
-  A.ce_mom = reinterpret_cast<R*>(piece(4 * ne * sizeof(R)));
-  A.e_slot = reinterpret_cast<int*>(piece(ne * sizeof(int)));
-  A.u_node = reinterpret_cast<int*>(piece(ne * sizeof(int)));
-  A.ce_node = reinterpret_cast<int*>(piece(ne * sizeof(int)));
-  return off;
+__host__ __device__ inline size_t adj_prep_smem(int N) {
+  size_t M = 1;
+  while (M < 8 * (size_t)N) M <<= 1;
+  return 6 * (size_t)N * sizeof(R) + 32 + M * 8 + 8 * (size_t)N * 4 + 64;
+}
+
+// The forward recomputation of the bead step for the steps step_arg + j, j = blockIdx.x, of a segment,
+// a block per step: it depends on no other step and on no adjoint, so it is off the chain of
+// reverse steps (of whose 15 us per step, N = 16, it took 5 as the first part of k_adj_bead).
+// The state of step j lies j * state_stride bytes behind `state` and the arrays of C, its region
+// j * prep_stride bytes behind `prep`.
+// A checkpoint of the forward pass: the populations (16-byte words) and the bead arrays behind them
+// (4-byte words) to checkpoint (*d_step - k0) / K of those that lie `stride` bytes apart from `to` on
+__global__ static void k_adj_checkpoint(const int4* __restrict__ pops, size_t npops, const int* __restrict__ beads, int nbeads,
+                                        unsigned char* __restrict__ to, size_t stride, const uint32_t* __restrict__ d_step,
+                                        uint32_t k0, uint32_t K) {
+  unsigned char* dst = to + (size_t)((*d_step - k0) / K) * stride;
+  int4* p = reinterpret_cast<int4*>(dst);
+  int* b = reinterpret_cast<int*>(dst + npops * 16);
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, n = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = t; i < npops; i += n) p[i] = pops[i];
+  for (size_t i = t; i < (size_t)nbeads; i += n) b[i] = beads[i];
+}
+
+// xbar of the last step: d/dx of sum (x - x0)^2 from the FP64 positions
+template <class R>
+__global__ void k_adj_seed(const double* __restrict__ x0, const double* __restrict__ x, int n, R* __restrict__ xbar) {
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x)
+    xbar[t] = (R)(2.0 * (x[t] - x0[t]));
 }
 
 template <class S, class R, bool DEV>
-__global__ void __launch_bounds__(512) k_adj_bead(const S* __restrict__ state, const R* __restrict__ lam,
-                                                   R* __restrict__ lam_out, const FluidK<R> P, const ChainK<R> C,
-                                                   const AdjK<R> A0, const uint32_t step_arg) {
-  const uint32_t step = launch_step(P, step_arg);
+__global__ void __launch_bounds__(512) k_adj_prep(const S* __restrict__ state, const FluidK<R> P, const ChainK<R> C,
+                                                   unsigned char* prep, int prep_stride, size_t state_stride,
+                                                   const uint32_t step_arg) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int N = C.N, tid = threadIdx.x, nt = blockDim.x, L = (int)P.L;
-  AdjK<R> A = A0;
-  if (A0.smem_scratch) carve_adj_scratch(A, smem + A0.smem_off, N, C.cap);
-  const R h = C.h;
+  const int N = C.N, ne = 8 * N, tid = threadIdx.x, nt = blockDim.x, L = (int)P.L;
+  const uint32_t step = launch_step(P, step_arg) + blockIdx.x;
+  auto behind = [&](const void* q) {
+    return reinterpret_cast<const unsigned char*>(q) + (size_t)blockIdx.x * state_stride;
+  };
+  const S* pop = reinterpret_cast<const S*>(behind(state));
+  const R *cx_ = reinterpret_cast<const R*>(behind(C.x)), *cxl = reinterpret_cast<const R*>(behind(C.xl)),
+          *cv = reinterpret_cast<const R*>(behind(C.v)), *cF = reinterpret_cast<const R*>(behind(C.F));
+  AdjPrep<R> A;
+  A.carve(prep + (size_t)blockIdx.x * prep_stride, N);
   R* sx = reinterpret_cast<R*>(smem);
   R* sl = sx + 3 * N;
-  // d/dzeta so far, read now so that the update at the end is a plain store (no other grid
-  // writes it while this one runs: the previous reverse step has completed)
-  const double zbar_in = tid == 0 ? *A.zbar : 0.0;
-  // ---- forward recomputation of step k ------------------------------------------------
   for (int t = tid; t < 3 * N; t += nt) {
-    const R vh = C.v[t] + h * C.F[t] / (R(2) * C.m);
-    const R dx = h * vh;
-    const R xh = C.x[t];
-    R hi = xh + dx;
-    const R bp = hi - xh;
-    R lo = C.xl[t] + ((xh - (hi - bp)) + (dx - bp));
-    {
-      const R s2 = hi + lo;
-      lo = lo - (s2 - hi);
-      hi = s2;
-    }
-    if (hi < R(0)) {
-      const R s2 = C.box + hi;
-      lo += hi - (s2 - C.box);
-      hi = s2;
-    }
-    if (hi >= C.box) hi -= C.box;
+    R vh, hi, lo;
+    int im = 0;
+    drift<R>(C, cv[t], cF[t], cx_[t], cxl[t], im, vh, hi, lo);
     A.vh[t] = vh;
-    sx[t] = hi;
-    sl[t] = lo;
+    A.sx[t] = sx[t] = hi;
+    A.sl[t] = sl[t] = lo;
   }
   __syncthreads();
-  for (int e = tid; e < 8 * N; e += nt) {
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(
+      (reinterpret_cast<uintptr_t>(smem + 6 * N * sizeof(R)) + 15) & ~(uintptr_t)15);
+  int M = 1;
+  while (M < ne) M <<= 1;
+  for (int e = tid; e < M; e += nt) {
+    if (e >= ne) {
+      keys[e] = ~0ull;
+      continue;
+    }
     const int b = e >> 3, c = e & 7;
     const int d3[3] = {c & 1, (c >> 1) & 1, (c >> 2) & 1};
     R fr[3];
@@ -317,28 +325,27 @@ __global__ void __launch_bounds__(512) k_adj_bead(const S* __restrict__ state, c
     R ws[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) ws[q] = d3[q] ? fr[q] : R(1) - fr[q];
-    const R w = ws[0] * ws[1] * ws[2];
     // dw/dx_q = (+-1/a) * product of the other two factors
-    A.e_gw[0 * C.cap + e] = (d3[0] ? R(1) : R(-1)) * ws[1] * ws[2] / C.a;
-    A.e_gw[1 * C.cap + e] = (d3[1] ? R(1) : R(-1)) * ws[0] * ws[2] / C.a;
-    A.e_gw[2 * C.cap + e] = (d3[2] ? R(1) : R(-1)) * ws[0] * ws[1] / C.a;
+    A.gw[0 * ne + e] = (d3[0] ? R(1) : R(-1)) * ws[1] * ws[2] / C.a;
+    A.gw[1 * ne + e] = (d3[1] ? R(1) : R(-1)) * ws[0] * ws[2] / C.a;
+    A.gw[2 * ne + e] = (d3[2] ? R(1) : R(-1)) * ws[0] * ws[1] / C.a;
     const int qx = (cl[0] + d3[0]) % L, qy = (cl[1] + d3[1]) % L, qz = (cl[2] + d3[2]) % L;
     R mom[4];
-    gather_node<S, R, DEV>(state, P, qx, qy, qz, mom);
-    A.ce_node[e] = qx + L * (qy + L * qz);
-    A.ce_w[e] = w;
+    gather_node<S, R, DEV>(pop, P, qx, qy, qz, mom);
+    A.w[e] = ws[0] * ws[1] * ws[2];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) A.ce_mom[q * C.cap + e] = mom[q];
+    for (int q = 0; q < 4; ++q) A.mom[q * ne + e] = mom[q];
+    keys[e] = ((unsigned long long)(unsigned)(qx + L * (qy + L * qz)) << 32) | (unsigned)e;
   }
   __syncthreads();
   for (int b = tid; b < N; b += nt) {
     R ub[3] = {R(0), R(0), R(0)};
     for (int c = 0; c < 8; ++c) {
       const int e = 8 * b + c;
-      const R w = A.ce_w[e], ir = R(1) / A.ce_mom[e];
-      ub[0] += w * A.ce_mom[C.cap + e] * ir;
-      ub[1] += w * A.ce_mom[2 * C.cap + e] * ir;
-      ub[2] += w * A.ce_mom[3 * C.cap + e] * ir;
+      const R w = A.w[e], ir = R(1) / A.mom[e];
+      ub[0] += w * A.mom[ne + e] * ir;
+      ub[1] += w * A.mom[2 * ne + e] * ir;
+      ub[2] += w * A.mom[3 * ne + e] * ir;
     }
     R g[4] = {R(0), R(0), R(0), R(0)};
     if (C.amp != R(0)) gauss4<R>(step, (uint32_t)b, 0u, C.k0, C.k1, g);
@@ -349,22 +356,9 @@ __global__ void __launch_bounds__(512) k_adj_bead(const S* __restrict__ state, c
       A.ub[t] = u;
       A.g[t] = g[q];
       A.fc[t] = -C.zeta * (A.vh[t] - u) + C.amp * g[q];
-      // adjoint of the total force of step k+1 and of v_h (from v' = v_h + h F'/2m)
-      A.fct[t] = A.fbar[t] + h / (R(2) * C.m) * A.vbar[t];
-      A.vhb[t] = A.vbar[t];
-      A.xpb[t] = A.xbar[t];  // x' is the position output of this step
     }
   }
-  __syncthreads();
-  // ---- unique forced nodes (same deterministic sort as the forward step) ----------------
-  const int ne = 8 * N;
-  int M = 1;
-  while (M < ne) M <<= 1;
-  unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem + 6 * N * sizeof(R) + 16);
-  keys = reinterpret_cast<unsigned long long*>((reinterpret_cast<uintptr_t>(keys) + 15) & ~(uintptr_t)15);
-  for (int i = tid; i < M; i += nt)
-    keys[i] = (i < ne) ? (((unsigned long long)(unsigned)A.ce_node[i] << 32) | (unsigned)i) : ~0ull;
-  __syncthreads();
+  // entries ordered by node (and by entry within a node)
   if (ne <= nt) {
     // few entries: each thread places its key by its rank among all keys (distinct: the entry
     // index is in the low bits), two barriers instead of the bitonic network's log2(M)^2 / 2
@@ -393,38 +387,134 @@ __global__ void __launch_bounds__(512) k_adj_bead(const S* __restrict__ state, c
       }
     }
   }
-  int* slot = reinterpret_cast<int*>(keys + M);
-  __shared__ int s_nu;  // number of unique forced nodes
+  int* lead = reinterpret_cast<int*>(keys + M);
   if (tid < 32) {
     int base = 0;
     for (int c0 = 0; c0 < ne; c0 += 32) {
       const int i = c0 + tid;
-      int lead = 0;
-      if (i < ne) lead = (i == 0) || ((keys[i] >> 32) != (keys[i - 1] >> 32));
-      const unsigned mask = __ballot_sync(0xffffffffu, lead);
-      if (i < ne) slot[i] = lead ? base + __popc(mask & ((1u << tid) - 1u)) : -1;
+      int l = 0;
+      if (i < ne) l = (i == 0) || ((keys[i] >> 32) != (keys[i - 1] >> 32));
+      const unsigned mask = __ballot_sync(0xffffffffu, l);
+      if (i < ne) lead[i] = l ? base + __popc(mask & ((1u << tid) - 1u)) : -1;
       base += __popc(mask);
     }
-    if (tid == 0) s_nu = base;
+    if (tid == 0) {
+      *A.nu = base;
+      A.first[base] = ne;
+    }
   }
   __syncthreads();
-  // per unique node p: forward force density f(p), force-correction adjoint -> fbar(p),
-  // forced-node (rho, J) adjoint; entry -> slot map
   for (int i = tid; i < ne; i += nt) {
-    const int u = slot[i];
+    A.order[i] = (int)(keys[i] & 0xffffffffu);
+    const int u = lead[i];
     if (u < 0) continue;
     const int node = (int)(keys[i] >> 32);
-    const int e0 = (int)(keys[i] & 0xffffffffu);
     R f[3] = {R(0), R(0), R(0)};
     for (int r = i; r < ne && (int)(keys[r] >> 32) == node; ++r) {
       const int e = (int)(keys[r] & 0xffffffffu);
       const int b = e >> 3;
-      A.e_slot[e] = u;
-      f[0] -= A.ce_w[e] * A.fc[3 * b + 0] * C.inv_a3;
-      f[1] -= A.ce_w[e] * A.fc[3 * b + 1] * C.inv_a3;
-      f[2] -= A.ce_w[e] * A.fc[3 * b + 2] * C.inv_a3;
+      A.slot[e] = u;
+      f[0] -= A.w[e] * A.fc[3 * b + 0] * C.inv_a3;
+      f[1] -= A.w[e] * A.fc[3 * b + 1] * C.inv_a3;
+      f[2] -= A.w[e] * A.fc[3 * b + 2] * C.inv_a3;
     }
-    const R rho = A.ce_mom[e0], jx = A.ce_mom[C.cap + e0], jy = A.ce_mom[2 * C.cap + e0], jz = A.ce_mom[3 * C.cap + e0];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) A.uf[q * ne + u] = f[q];
+    A.first[u] = i;
+    A.node[u] = node;
+  }
+}
+
+// Chain part of the adjoint of one step, one thread block.
+// In:  the step's AdjPrep region, lambda(n*_{k+1}) (`lam`), xbar/vbar/fbar of step k+1.
+// Out: xbar/vbar/fbar of step k (in place), zbar (+= d/dzeta), and lambda(n*_k) (`lam_out`)
+//      completed: lambda_k,i(r - e_i) += rho-bar(r) + c_i . J-bar(r) at the forced nodes r.
+// Launched with programmatic stream serialization after k_adj_lb of the same step, which writes
+// the rest of lambda(n*_k): everything up to that last addition runs beside it, and the
+// addition waits for it.  Bound by the latency of its phases: 19 us alone before the forward
+// recomputation moved to k_adj_prep (8 us for ten steps at once), 9.5 us now at N = 16 (copy of the
+// region and the adjoints 1.5 us, per-node adjoints and Hessian side by side 1.8, per-bead and
+// per-entry adjoints 1.2, integrator, sums and additions 1.6).  (Releasing the next step's k_adj_lb
+// from here, before this grid ends, cost more than it gave: its waiting blocks hold the SMs that the
+// recomputation beside the sweep needs, 3.39 against 3.28 ms per call at L = 32, T = 100.)
+template <class R>
+struct AdjK {
+  R *xbar, *vbar, *fbar;  // 3N each, in/out across the reverse steps (global)
+  double* zbar;           // accumulated d objective / d zeta (global)
+  // scratch of one reverse step: carved from the kernel's dynamic shared memory, with the step's
+  // AdjPrep region copied in front of it, when in_smem is set (small chains), else global memory
+  R *fct, *vhb, *xpb, *hes;  // 3N each
+  R* e_rb;      // 4 x 8N (rho-bar, J-bar) per entry
+  R* u_fb;      // 3 x 8N: f-bar per unique node
+  R* u_rb;      // 4 x 8N: forced-node (rho, J) adjoint per unique node
+  R* u_sp;      // 4 x 8N: (rho-bar, J-bar) summed per unique forced node
+  R* e_wb;      // 8N: weight adjoint per entry
+  R* zb_b;      // N: zeta-bar per bead
+  unsigned char* scratch;  // global scratch (in_smem not set)
+  int in_smem;
+  __host__ __device__ int carve(unsigned char* base, int N) {
+    int off = 0;
+    auto take = [&](int bytes) {
+      unsigned char* q = base + off;
+      off += (bytes + 15) / 16 * 16;
+      return q;
+    };
+    const int r = (int)sizeof(R), n3 = 3 * N, ne = 8 * N;
+    fct = (R*)take(n3 * r);
+    vhb = (R*)take(n3 * r);
+    xpb = (R*)take(n3 * r);
+    hes = (R*)take(n3 * r);
+    e_rb = (R*)take(4 * ne * r);
+    u_fb = (R*)take(3 * ne * r);
+    u_rb = (R*)take(4 * ne * r);
+    u_sp = (R*)take(4 * ne * r);
+    e_wb = (R*)take(ne * r);
+    zb_b = (R*)take(N * r);
+    return off;
+  }
+};
+
+template <class R>
+__global__ void __launch_bounds__(512) k_adj_bead(const R* __restrict__ lam, R* __restrict__ lam_out, const FluidK<R> P,
+                                                   const ChainK<R> C, const AdjK<R> A0, unsigned char* prep,
+                                                   const int prep_bytes) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int N = C.N, ne = 8 * N, tid = threadIdx.x, nt = blockDim.x, L = (int)P.L;
+  AdjK<R> A = A0;
+  AdjPrep<R> F;
+  if (A0.in_smem) {
+    F.carve(smem, N);
+    A.carve(smem + prep_bytes, N);
+  } else {
+    F.carve(prep, N);
+    A.carve(A0.scratch, N);
+  }
+  const R h = C.h;
+  // d/dzeta so far, read now so that the update at the end is a plain store (no other grid
+  // writes it while this one runs: the previous reverse step has completed)
+  const double zbar_in = tid == nt - 32 ? *A.zbar : 0.0;
+  for (int t = tid; t < 3 * N; t += nt) {
+    // adjoint of the total force of step k+1 and of v_h (from v' = v_h + h F'/2m)
+    const R vb = A.vbar[t];
+    A.fct[t] = A.fbar[t] + h / (R(2) * C.m) * vb;
+    A.vhb[t] = vb;
+    A.xpb[t] = A.xbar[t];  // x' is the position output of this step
+    A.hes[t] = R(0);
+  }
+  if (A0.in_smem) {
+    const int4* from = reinterpret_cast<const int4*>(prep);
+    int4* to = reinterpret_cast<int4*>(smem);
+    for (int i = nt - 1 - tid; i < prep_bytes / 16; i += nt) to[i] = from[i];
+  }
+  __syncthreads();
+  const int nu = *F.nu;
+  // per unique node p: force-correction adjoint -> fbar(p), forced-node (rho, J) adjoint; on the
+  // warps left over the chain forces: Hessian . F_cons-bar (F_cons-bar = F_total-bar)
+  const int nodew = (nu + 31) / 32 * 32;
+  const int h0 = nodew + 128 <= nt ? nodew : 0;  // the Hessian's first thread
+  for (int u = tid; u < nu; u += nt) {
+    const int node = F.node[u], e0 = F.order[F.first[u]];
+    const R rho = F.mom[e0], jx = F.mom[ne + e0], jy = F.mom[2 * ne + e0], jz = F.mom[3 * ne + e0];
     R nb[Q], ab[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) nb[q] = lam[(unsigned long long)q * P.plane + (unsigned)node];
@@ -441,126 +531,133 @@ __global__ void __launch_bounds__(512) k_adj_bead(const S* __restrict__ state, c
     dmb[8] = ab[8] * R(InvB<8>::v);
     dmb[9] = ab[9] * R(InvB<9>::v);
     R rb, Jb[3], dJb[3];
-    force_moments_vjp<R>(rho, jx, jy, jz, f[0] * C.dJ_scale, f[1] * C.dJ_scale, f[2] * C.dJ_scale, P.gs, P.gb, dmb,
-                         rb, Jb, dJb);
+    force_moments_vjp<R>(rho, jx, jy, jz, F.uf[u] * C.dJ_scale, F.uf[ne + u] * C.dJ_scale, F.uf[2 * ne + u] * C.dJ_scale,
+                         P.gs, P.gb, dmb, rb, Jb, dJb);
     A.u_fb[u] = dJb[0] * C.dJ_scale;
-    A.u_fb[C.cap + u] = dJb[1] * C.dJ_scale;
-    A.u_fb[2 * C.cap + u] = dJb[2] * C.dJ_scale;
+    A.u_fb[ne + u] = dJb[1] * C.dJ_scale;
+    A.u_fb[2 * ne + u] = dJb[2] * C.dJ_scale;
     A.u_rb[u] = rb;
-    A.u_rb[C.cap + u] = Jb[0];
-    A.u_rb[2 * C.cap + u] = Jb[1];
-    A.u_rb[3 * C.cap + u] = Jb[2];
+    A.u_rb[ne + u] = Jb[0];
+    A.u_rb[2 * ne + u] = Jb[1];
+    A.u_rb[3 * ne + u] = Jb[2];
   }
+  if (tid >= h0) chain_force_vjp_block<R>(F.sx, F.sl, A.fct, C, A.hes, tid - h0, nt - h0);
   __syncthreads();
-  // ---- per bead: spreading, friction, interpolation adjoints ---------------------------
-  for (int b = tid; b < N; b += nt) {
-    R fcb[3] = {A.fct[3 * b], A.fct[3 * b + 1], A.fct[3 * b + 2]};
-    R fc[3] = {A.fc[3 * b], A.fc[3 * b + 1], A.fc[3 * b + 2]};
-    R xpb[3] = {R(0), R(0), R(0)};
-    // spreading: f(p) = -sum_e w_e F_c,b / a^3
-    R wb[8];
-    for (int c = 0; c < 8; ++c) {
-      const int e = 8 * b + c, u = A.e_slot[e];
-      const R fbx = A.u_fb[u], fby = A.u_fb[C.cap + u], fbz = A.u_fb[2 * C.cap + u];
-      const R w = A.ce_w[e];
-      fcb[0] -= w * C.inv_a3 * fbx;
-      fcb[1] -= w * C.inv_a3 * fby;
-      fcb[2] -= w * C.inv_a3 * fbz;
-      wb[c] = -C.inv_a3 * (fc[0] * fbx + fc[1] * fby + fc[2] * fbz);
-    }
-    // friction + noise: F_c = -zeta (v_h - u_b) + amp(zeta) g
-    R Ub[3], zb = R(0);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const int t = 3 * b + q;
-      A.vhb[t] -= C.zeta * fcb[q];
-      Ub[q] = C.zeta * fcb[q];
-      const R damp = C.zeta > R(0) ? C.amp / (R(2) * C.zeta) : R(0);
-      zb += fcb[q] * (-(A.vh[t] - A.ub[t]) + damp * A.g[t]);
-    }
-    A.zb_b[b] = zb;
-    // interpolation: u_b = sum_e w_e J_e / rho_e (a/h)
+  // ---- per bead and component: spreading, friction adjoints ----------------------------
+  for (int t = tid; t < 3 * N; t += nt) {
+    const int b = t / 3, q = t - 3 * b;
+    R fcb = A.fct[t];
     for (int c = 0; c < 8; ++c) {
       const int e = 8 * b + c;
-      const R w = A.ce_w[e], rho = A.ce_mom[e], ir = R(1) / rho;
-      const R J[3] = {A.ce_mom[C.cap + e], A.ce_mom[2 * C.cap + e], A.ce_mom[3 * C.cap + e]};
-      R ue[3], uJ = R(0);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) ue[q] = J[q] * ir * C.u_scale;
-      wb[c] += ue[0] * Ub[0] + ue[1] * Ub[1] + ue[2] * Ub[2];
-      R ueb[3];
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        ueb[q] = w * Ub[q];
-        uJ += J[q] * ueb[q];
-      }
-      A.e_rb[e] = -C.u_scale * uJ * ir * ir;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) A.e_rb[(q + 1) * C.cap + e] = C.u_scale * ueb[q] * ir;
-      // trilinear weight gradient
-#pragma unroll
-      for (int q = 0; q < 3; ++q) xpb[q] += wb[c] * A.e_gw[q * C.cap + e];
+      fcb -= F.w[e] * C.inv_a3 * A.u_fb[q * ne + F.slot[e]];
     }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) A.xpb[3 * b + q] += xpb[q];
+    // friction + noise: F_c = -zeta (v_h - u_b) + amp(zeta) g
+    A.vhb[t] -= C.zeta * fcb;
+    A.fct[t] = fcb;  // from here on the adjoint of F_c (the Hessian has used that of the total)
   }
   __syncthreads();
-  // ---- chain forces: x'bar += Hessian . F_cons-bar (F_cons-bar = F_total-bar) ---------
-  chain_force_vjp_block<R>(sx, sl, A.fct, C, A.xpb);
+  // ---- per entry: interpolation u_b = sum_e w_e J_e / rho_e (a/h), weight adjoint ---------
+  for (int e = tid; e < ne; e += nt) {
+    const int b = e >> 3, u = F.slot[e];
+    const R fc[3] = {F.fc[3 * b], F.fc[3 * b + 1], F.fc[3 * b + 2]};
+    const R fbx = A.u_fb[u], fby = A.u_fb[ne + u], fbz = A.u_fb[2 * ne + u];
+    // spreading: f(p) = -sum_e w_e F_c,b / a^3
+    R wb = -C.inv_a3 * (fc[0] * fbx + fc[1] * fby + fc[2] * fbz);
+    R Ub[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) Ub[q] = C.zeta * A.fct[3 * b + q];
+    const R w = F.w[e], rho = F.mom[e], ir = R(1) / rho;
+    const R J[3] = {F.mom[ne + e], F.mom[2 * ne + e], F.mom[3 * ne + e]};
+    R ue[3], uJ = R(0);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) ue[q] = J[q] * ir * C.u_scale;
+    wb += ue[0] * Ub[0] + ue[1] * Ub[1] + ue[2] * Ub[2];
+    R ueb[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      ueb[q] = w * Ub[q];
+      uJ += J[q] * ueb[q];
+    }
+    A.e_rb[e] = -C.u_scale * uJ * ir * ir;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) A.e_rb[(q + 1) * ne + e] = C.u_scale * ueb[q] * ir;
+    A.e_wb[e] = wb;
+  }
   __syncthreads();
   // ---- integrator: x' = x + h v_h ; v_h = v + h F / 2m ------------------------------------
-  for (int t = tid; t < 3 * N; t += nt) {
-    const R xpb = A.xpb[t];
+  for (int t = nt - 1 - tid; t < 3 * N; t += nt) {
+    const int b = t / 3, q = t - 3 * b;
+    R xpb = R(0);
+    for (int c = 0; c < 8; ++c) xpb += A.e_wb[8 * b + c] * F.gw[q * ne + 8 * b + c];  // trilinear weight gradient
+    xpb = (A.xpb[t] + xpb) + A.hes[t];
     const R vhb = A.vhb[t] + h * xpb;
     A.xbar[t] = xpb;
     A.vbar[t] = vhb;
     A.fbar[t] = h / (R(2) * C.m) * vhb;
   }
   // ---- sparse (rho, J) adjoint per unique node, entries summed in entry order -----------
-  for (int i = tid; i < ne; i += nt) {
-    const int u = slot[i];
-    if (u < 0) continue;
-    const int node = (int)(keys[i] >> 32);
-    R v[4] = {A.u_rb[u], A.u_rb[C.cap + u], A.u_rb[2 * C.cap + u], A.u_rb[3 * C.cap + u]};
-    for (int r = i; r < ne && (int)(keys[r] >> 32) == node; ++r) {
-      const int e = (int)(keys[r] & 0xffffffffu);
+  for (int u = tid; u < nu; u += nt) {
+    R v[4] = {A.u_rb[u], A.u_rb[ne + u], A.u_rb[2 * ne + u], A.u_rb[3 * ne + u]};
+    for (int r = F.first[u]; r < F.first[u + 1]; ++r) {
+      const int e = F.order[r];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) v[q] += A.e_rb[q * C.cap + e];
+      for (int q = 0; q < 4; ++q) v[q] += A.e_rb[q * ne + e];
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) A.u_sp[q * C.cap + u] = v[q];
-    A.u_node[u] = node;
+    for (int q = 0; q < 4; ++q) A.u_sp[q * ne + u] = v[q];
   }
-  // ---- zeta-bar: fixed-order block sum ----------------------------------------------------
+  // ---- zeta-bar: per bead, then a fixed-order block sum ------------------------------------
+  for (int b = tid; b < N; b += nt) {
+    const R damp = C.zeta > R(0) ? C.amp / (R(2) * C.zeta) : R(0);
+    R zb = R(0);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int t = 3 * b + q;
+      zb += A.fct[t] * (-(F.vh[t] - F.ub[t]) + damp * F.g[t]);
+    }
+    A.zb_b[b] = zb;
+  }
   __syncthreads();
-  if (tid == 0) {
+  if (tid >= nt - 32) {  // the last warp: in a fixed tree
     double acc = 0.0;
-    for (int b = 0; b < N; ++b) acc += (double)A.zb_b[b];
-    *A.zbar = zbar_in + acc;
+    for (int b = tid & 31; b < N; b += 32) acc += (double)A.zb_b[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (tid == nt - 32) *A.zbar = zbar_in + acc;
   }
   // ---- lambda_k,i(r - e_i) += rho-bar(r) + c_i . J-bar(r) at the forced nodes, once the
   //      adjoint LB kernel of this step has written lambda_k (each (i, r - e_i) target belongs
   //      to one forced node r, so the additions do not collide) --------------------------
   //      In chunks of kAddBatch targets per thread: all loads of a chunk, then its stores (one
-  //      memory round trip per chunk instead of one per target).
-  grid_dependency_wait();
-  const int nu = s_nu, total = Q * nu;
+  //      memory round trip per chunk instead of one per target); the first chunk's targets and
+  //      terms are formed before the wait.
+  const int total = Q * nu;
   constexpr int kAddBatch = 8;
-  for (int k0 = tid; k0 < total; k0 += kAddBatch * nt) {
-    unsigned long long at[kAddBatch];
-    R v[kAddBatch], old[kAddBatch];
+  unsigned long long at[kAddBatch];
+  R v[kAddBatch];
+  auto form = [&](int k0) {
 #pragma unroll
     for (int j = 0; j < kAddBatch; ++j) {
       const int k = k0 + j * nt;
       if (k >= total) break;
       const int i = k / nu, u = k - i * nu;
-      const int node = A.u_node[u];
+      const int node = F.node[u];
       const int x = node % L, y = (node / L) % L, z = node / (L * L);
       const int ex = unpack_component(pack_component(0), i), ey = unpack_component(pack_component(1), i),
                 ez = unpack_component(pack_component(2), i);
       const int sx = (x - ex + L) % L, sy = (y - ey + L) % L, sz = (z - ez + L) % L;
-      v[j] = A.u_sp[u] + R(ex) * A.u_sp[C.cap + u] + R(ey) * A.u_sp[2 * C.cap + u] + R(ez) * A.u_sp[3 * C.cap + u];
+      v[j] = A.u_sp[u] + R(ex) * A.u_sp[ne + u] + R(ey) * A.u_sp[2 * ne + u] + R(ez) * A.u_sp[3 * ne + u];
       at[j] = (unsigned long long)i * P.plane + (unsigned)(sx + L * (sy + L * sz));
+    }
+  };
+  form(tid);
+  grid_dependency_wait();
+  for (int k0 = tid; k0 < total; k0 += kAddBatch * nt) {
+    if (k0 != tid) form(k0);
+    R old[kAddBatch];
+#pragma unroll
+    for (int j = 0; j < kAddBatch; ++j) {
+      if (k0 + j * nt >= total) break;
       old[j] = lam_out[at[j]];
     }
 #pragma unroll
@@ -584,7 +681,7 @@ __global__ void __launch_bounds__(512) k_chain_force_vjp(const ChainK<R> C, cons
     sl[t] = C.xl[t];
   }
   __syncthreads();
-  chain_force_vjp_block<R>(sx, sl, fbar, C, xbar);
+  chain_force_vjp_block<R>(sx, sl, fbar, C, xbar, threadIdx.x, blockDim.x);
 }
 
 }  // namespace gblb

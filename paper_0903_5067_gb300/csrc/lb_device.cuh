@@ -198,6 +198,8 @@ struct PendK {
   int* cur_count;
   R* cur_dense;           // this step's slot of the dense field
   unsigned* cur_mask;     // this step's slot of the mask (cleared of the old list)
+  R* apply_to;            // null, or FP32/FP64 populations the old list's corrections, not yet applied
+                          // to them, are added to where they are cleared
   int mark;               // 1: mark the pulling nodes of this step's list (deferred steps)
   int cap;
   unsigned long long plane;  // element stride between the 19 planes
@@ -1125,12 +1127,21 @@ __device__ __forceinline__ void node_correction(const FluidK<R>& P, const ChainK
 }
 
 // Empty the list entry u (of this slot's list from two steps before, or already applied): its
-// node's corrections and the marks of the nodes pulling from it back to zero
+// node's corrections (added to apply_to where given) and the marks of the nodes pulling from it back
+// to zero
 template <class R>
 __device__ __forceinline__ void clear_correction(const PendK<R>& Pd, int L, int u) {
   const int4 p = Pd.cur_pos[u];
   if (p.x < 0) return;
   R* d = Pd.cur_dense + (unsigned)p.x;
+  if (Pd.apply_to) {
+    R* n = Pd.apply_to + (unsigned)p.x;
+    R c[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) c[i] = n[(unsigned long long)i * Pd.plane] + d[(unsigned long long)i * Pd.plane];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) n[(unsigned long long)i * Pd.plane] = c[i];
+  }
 #pragma unroll
   for (int i = 0; i < Q; ++i) d[(unsigned long long)i * Pd.plane] = R(0);
   if (Pd.cur_mask) clear_marks(Pd.cur_mask, Pd.seg0, L, p.y, p.z, p.w);

@@ -192,19 +192,6 @@ class EngineT final : public Engine {
     for (; t < n; ++t) step_deferred(k + (uint32_t)t, s, nullptr, nullptr);
   }
 
-  // One complete step with the bead kernel's state arrays given (the adjoint's recomputation:
-  // read a saved state, write the next one); the context's own bead arrays are not touched.
-  void step_with_chain(uint32_t k, cudaStream_t s, const ChainK<R>& C, const FluidK<R>& P) {
-    flush(s);
-    const S* A = pop_[cur_];
-    S* Bo = pop_[cur_ ^ 1];
-    const PendK<R> Pd = pend(false);
-    launch_bead(A, P, Pd, k, s, true, &C);
-    launch_lb(A, Bo, P, Pd, k, s, nullptr, nullptr);
-    apply(Bo, P, pslot_, s);
-    cur_ ^= 1;
-  }
-
   // apply the pending force correction of the last deferred step
   void flush(cudaStream_t s) override {
     if (!open_) return;
@@ -253,33 +240,28 @@ class EngineT final : public Engine {
     const size_t o_fin = take(stb);
     const size_t o_lam0 = take(lamb), o_lam1 = take(lamb);
     const size_t o_bar = take(3 * n3 * sizeof(R));
-    // bead adjoint scratch with its own corner entries (the recomputation running beside it
-    // uses the context's): in the kernel's shared memory when it fits, else here
+    // what the chain part of each reverse step needs of its forward step: a region per step and pool
+    AdjPrep<R> prep_layout;
+    const int prep_bytes = prep_layout.carve(nullptr, N_);
+    const size_t o_prep = take(2 * (size_t)K * prep_bytes);
+    // its scratch: with that region in the kernel's shared memory when they fit, else here
     AdjK<R> A;
     memset(&A, 0, sizeof(A));
-    const size_t adj_scratch = carve_adj_scratch<R>(A, nullptr, N_, cap_);
-    const size_t ne = 8 * (size_t)N_;
-    size_t M = 1;
-    while (M < ne) M <<= 1;
-    const size_t smem_base = align_up(align_up(6 * n3 / 3 * sizeof(R) + 32, 16) + M * 8 + ne * 4 + 64, 16);
-    const bool scratch_in_smem = smem_base + adj_scratch <= 200 * 1024;
+    const size_t adj_scratch = (size_t)A.carve(nullptr, N_);
+    const bool scratch_in_smem = prep_bytes + adj_scratch <= 200 * 1024;
     const size_t o_adj = take(scratch_in_smem ? 16 : adj_scratch);
     const size_t o_z = take(sizeof(double));
-    const size_t o_ctr = take(2 * sizeof(uint32_t));  // step counters of the segment graphs
+    const size_t o_x0 = take(2 * n3 * sizeof(double)), o_xT = take(2 * n3 * sizeof(double));  // read-backs
+    const size_t o_ctr = take(3 * sizeof(uint32_t));  // step counters of the segment graphs
     unsigned char* base = nullptr;
     cuda_check(cudaMalloc(&base, off), "adjoint scratch");
-    S* const own_pop[2] = {pop_[0], pop_[1]};
-    struct Restore {  // the context's own population buffers, the scratch, the second stream
-      EngineT* e;     // and the events, also on an error
-      S* p0;
-      S* p1;
+    struct Guard {  // the scratch, the second stream, the graphs and the events, also on an error
       unsigned char* p;
       cudaStream_t s2, cs;
       std::vector<cudaEvent_t> ev;
-      cudaGraphExec_t g[6];  // recomputation by pool, reverse sweep by pool and lambda parity
-      ~Restore() {
-        e->pop_[0] = p0;
-        e->pop_[1] = p1;
+      // recomputation by pool, reverse sweep by pool and lambda parity, forward by buffer
+      cudaGraphExec_t g[8];
+      ~Guard() {
         for (cudaStream_t x : {s2, cs})
           if (x) {
             cudaStreamSynchronize(x);
@@ -290,7 +272,7 @@ class EngineT final : public Engine {
         for (cudaEvent_t x : ev) cudaEventDestroy(x);
         cudaFree(p);
       }
-    } guard{this, own_pop[0], own_pop[1], base, nullptr, nullptr, {}, {}};
+    } guard{base, nullptr, nullptr, {}, {}};
     auto new_event = [&]() {
       cudaEvent_t x = nullptr;
       cuda_check(cudaEventCreateWithFlags(&x, cudaEventDisableTiming), "adjoint event");
@@ -303,6 +285,7 @@ class EngineT final : public Engine {
     };
     auto ck = [&](int i) { return base + o_ck + (size_t)i * stb; };
     auto pool = [&](int pid, int i) { return base + o_pool + ((size_t)pid * (K + 1) + i) * stb; };
+    auto prep = [&](int pid, int i) { return base + o_prep + ((size_t)pid * K + i) * prep_bytes; };
     // a state's bead arrays, at their offsets within the saved span
     auto at = [&](unsigned char* st, const void* arr) {
       return st + popb + (size_t)(reinterpret_cast<const unsigned char*>(arr) - bead0);
@@ -310,29 +293,81 @@ class EngineT final : public Engine {
     // 1. forward pass with checkpoints every K steps (deferred force corrections between
     //    checkpoints, the same arithmetic as complete steps when the storage type is the
     //    arithmetic type; complete steps otherwise)
-    std::vector<double> x0h(n3), xTh(n3);
-    get_beads(x0h.data(), nullptr, s);
+    double* const x0d = reinterpret_cast<double*>(base + o_x0);
+    double* const xTd = reinterpret_cast<double*>(base + o_xT);
+    auto read_beads = [&](double* to) {
+      k_bead_readback<R><<<(unsigned)((n3 + 255) / 256), 256, 0, s>>>(x_, xl_, img_, v_, (int)n3, cfg_.L * cfg_.a, to);
+      cuda_check(cudaGetLastError(), "bead read-back");
+    };
+    read_beads(x0d);
+    cuda_check(cudaStreamCreateWithFlags(&guard.s2, cudaStreamNonBlocking), "adjoint stream");
     const bool deferred = sizeof(S) == sizeof(R);
-    for (int64_t t = 0; t < T; ++t) {
-      if (t % K == 0) {
+    // A run of launches captured as a graph on a stream of its own
+    auto capture = [&](auto&& ops) {
+      if (!guard.cs) cuda_check(cudaStreamCreateWithFlags(&guard.cs, cudaStreamNonBlocking), "capture stream");
+      cudaGraph_t gr = nullptr;
+      cudaGraphExec_t g = nullptr;
+      cuda_check(cudaStreamBeginCapture(guard.cs, cudaStreamCaptureModeThreadLocal), "begin capture");
+      ops(guard.cs);
+      cuda_check(cudaStreamEndCapture(guard.cs, &gr), "end capture");
+      const cudaError_t ie = cudaGraphInstantiate(&g, gr, 0);
+      cudaGraphDestroy(gr);
+      cuda_check(ie, "instantiate segment graph");
+      return g;
+    };
+    // Full segments, each with its checkpoint, as graphs when there are enough of them (launching a
+    // step costs the host 20 us, more than it runs); for odd K one graph per population buffer.  With
+    // nothing pending either correction slot may come first: always the first.
+    const bool forward_graphs = deferred && T / K >= 4;
+    uint32_t* const d_fwd = reinterpret_cast<uint32_t*>(base + o_ctr) + 2;
+    if (forward_graphs) {
+      for (int j = 0; j < 2; ++j)
+        if (snap_pending_[j]) {
+          cuda_check(cudaStreamWaitEvent(s, copy_ev_[j], 0), "wait read-back");
+          snap_pending_[j] = false;
+        }
+      k_store_value<uint32_t><<<1, 1, 0, s>>>(d_fwd, k0);
+      cuda_check(cudaGetLastError(), "step counter");
+    }
+    for (int64_t t = 0; t < T;) {
+      const int64_t m = t + K <= T ? K : T - t;
+      if (forward_graphs && m == K) {
+        pslot_ = 0;
+        cudaGraphExec_t& g = guard.g[6 + cur_];
+        if (!g) {
+          g = capture([&](cudaStream_t st) {
+            k_adj_checkpoint<<<304, 256, 0, st>>>(reinterpret_cast<const int4*>(pop_[cur_]), popb / 16,
+                                                  reinterpret_cast<const int*>(bead0), (int)(beadb / 4), ck(0), stb, d_fwd,
+                                                  k0, (uint32_t)K);
+            for (int j = 0; j < K; ++j) step_deferred((uint32_t)j, st, nullptr, nullptr, d_fwd);
+            flush(st);
+            k_add_value<uint32_t><<<1, 1, 0, st>>>(d_fwd, (uint32_t)K);
+          });
+        } else {
+          cur_ ^= K & 1;  // the captured sequence's effect on the buffers
+        }
+        cuda_check(cudaGraphLaunch(g, s), "segment graph");
+        snap_k_ = (uint32_t)(k0 + t + K - 1);
+      } else {
         flush(s);
         save_state(ck((int)(t / K)));
+        for (int64_t j = t; j < t + m; ++j) {
+          if (deferred)
+            step_deferred((uint32_t)(k0 + j), s, nullptr, nullptr);
+          else
+            step((uint32_t)(k0 + j), s, nullptr, nullptr);
+        }
       }
-      if (deferred)
-        step_deferred((uint32_t)(k0 + t), s, nullptr, nullptr);
-      else
-        step((uint32_t)(k0 + t), s, nullptr, nullptr);
+      t += m;
     }
     flush(s);
-    save_state(base + o_fin);
-    get_beads(xTh.data(), nullptr, s);
-    double obj = 0.0;
-    std::vector<R> xb0(n3);
-    for (size_t t = 0; t < n3; ++t) {
-      const double d = xTh[t] - x0h[t];
-      obj += d * d;
-      xb0[t] = (R)(2.0 * d);
+    {  // the recomputations use the context's correction fields and lists: after the forward pass
+      cudaEvent_t fwd = new_event();
+      cuda_check(cudaEventRecord(fwd, s), "event");
+      cuda_check(cudaStreamWaitEvent(guard.s2, fwd, 0), "wait");
     }
+    save_state(base + o_fin);
+    read_beads(xTd);
     // 2. adjoint state at T
     R* lam[2] = {reinterpret_cast<R*>(base + o_lam0), reinterpret_cast<R*>(base + o_lam1)};
     cuda_check(cudaMemsetAsync(lam[0], 0, lamb, s), "lambda");
@@ -342,19 +377,19 @@ class EngineT final : public Engine {
     A.vbar = bars + n3;
     A.fbar = bars + 2 * n3;
     cuda_check(cudaMemsetAsync(bars, 0, 3 * n3 * sizeof(R), s), "bars");
-    cuda_check(cudaMemcpyAsync(A.xbar, xb0.data(), n3 * sizeof(R), cudaMemcpyHostToDevice, s), "xbar");
-    if (scratch_in_smem) {
-      A.smem_scratch = 1;
-      A.smem_off = (unsigned)smem_base;
-    } else {
-      carve_adj_scratch<R>(A, base + o_adj, N_, cap_);
-    }
+    k_adj_seed<R><<<(unsigned)((n3 + 255) / 256), 256, 0, s>>>(x0d, xTd, (int)n3, A.xbar);
+    cuda_check(cudaGetLastError(), "xbar");
+    A.in_smem = scratch_in_smem ? 1 : 0;
+    A.scratch = base + o_adj;
     A.zbar = reinterpret_cast<double*>(base + o_z);
     cuda_check(cudaMemsetAsync(A.zbar, 0, sizeof(double), s), "zbar");
     const ChainK<R> C = chain();
-    const size_t smem = scratch_in_smem ? smem_base + adj_scratch : smem_base;
+    const size_t smem = scratch_in_smem ? prep_bytes + adj_scratch : 0, prep_smem = adj_prep_smem<R>(N_);
     if (smem > 48 * 1024)
-      cuda_check(cudaFuncSetAttribute(k_adj_bead<S, R, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+      cuda_check(cudaFuncSetAttribute(k_adj_bead<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                 "adjoint smem");
+    if (prep_smem > 48 * 1024)
+      cuda_check(cudaFuncSetAttribute(k_adj_prep<S, R, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prep_smem),
                  "adjoint smem");
     dim3 blk, grd;
     lb_launch_shape(blk, grd, false);  // the adjoint LB kernel: one node per thread
@@ -362,7 +397,8 @@ class EngineT final : public Engine {
     // 3. reverse sweep over the segments.  The states t0 .. t1 - 1 of a segment sit in the
     //    slots of a pool: slot 0 a copy of its checkpoint, slots 1 .. written by the
     //    recomputation, whose steps read the populations and bead state of slot i and write
-    //    those of slot i + 1 (the context's population buffers pointed at the slots).  The
+    //    those of slot i + 1 (a step's force correction reaches slot i + 1's populations with the bead
+    //    kernel two steps on, when nothing reads them any more, so that a step is two launches).  The
     //    reverse steps read a slot's state in place.  The recomputation of segment k - 1 needs
     //    only its checkpoint, so it runs on a second stream beside the reverse sweep of segment
     //    k, in the other pool.  A full segment's recomputation or reverse sweep is the same
@@ -373,12 +409,11 @@ class EngineT final : public Engine {
     Prec.d_step = d_ctr;
     Prev.d_step = d_ctr + 1;
     auto recompute_ops = [&](int64_t t0, int64_t t1, int pid, cudaStream_t st, const FluidK<R>& Pk, bool rel) {
-      for (int64_t t = t0; t < t1; ++t) {
-        const int i = (int)(t - t0);
+      const int m = (int)(t1 - t0);
+      auto pops = [&](int i) { return reinterpret_cast<S*>(pool(pid, i)); };
+      for (int i = 0; i < m; ++i) {
         unsigned char* a = pool(pid, i);
         unsigned char* b = pool(pid, i + 1);
-        pop_[cur_] = reinterpret_cast<S*>(a);
-        pop_[cur_ ^ 1] = reinterpret_cast<S*>(b);
         ChainK<R> Cs = C;  // read the bead state of slot i, write the next state into slot i + 1
         Cs.x_in = reinterpret_cast<const R*>(at(a, x_));
         Cs.xl_in = reinterpret_cast<const R*>(at(a, xl_));
@@ -392,20 +427,35 @@ class EngineT final : public Engine {
         Cs.F = reinterpret_cast<R*>(at(b, F_));
         Cs.Fc = reinterpret_cast<R*>(at(b, Fc_));
         Cs.snap = nullptr;
-        step_with_chain(rel ? (uint32_t)(t - t0) : (uint32_t)(k0 + t), st, Cs, Pk);
+        const uint32_t k = rel ? (uint32_t)i : (uint32_t)(k0 + t0 + i);
+        PendK<R> Pd;
+        if (deferred) {  // step i's corrections, of slot i + 1's populations, are applied by step i + 2
+          Pd = pend_slots(i & 1, i > 0, true);
+          if (i >= 2) Pd.apply_to = reinterpret_cast<R*>(pool(pid, i - 1));
+        } else {
+          Pd = pend_slots(pslot_, false, false);
+        }
+        launch_bead(pops(i), Pk, Pd, k, st, true, &Cs);
+        launch_lb(pops(i), pops(i + 1), Pk, Pd, k, st, nullptr, nullptr);
+        if (!deferred) apply(pops(i + 1), Pk, pslot_, st);
       }
+      if (deferred)  // the last two steps' corrections
+        for (int i = m >= 2 ? m - 2 : 0; i < m; ++i) apply(pops(i + 1), Pk, i & 1, st);
+      // the segment's steps once more, all at once: what their reverse steps need of them
+      ChainK<R> C0 = C;
+      unsigned char* p0 = pool(pid, 0);
+      C0.x = reinterpret_cast<R*>(at(p0, x_));
+      C0.xl = reinterpret_cast<R*>(at(p0, xl_));
+      C0.v = reinterpret_cast<R*>(at(p0, v_));
+      C0.F = reinterpret_cast<R*>(at(p0, F_));
+      k_adj_prep<S, R, DEV><<<(unsigned)(t1 - t0), 512, prep_smem, st>>>(
+          reinterpret_cast<const S*>(p0), Pk, C0, prep(pid, 0), prep_bytes, stb, rel ? 0u : (uint32_t)(k0 + t0));
+      cuda_check(cudaGetLastError(), "adjoint preparation");
     };
     auto reverse_ops = [&](int64_t t0, int64_t t1, int pid, cudaStream_t st, const FluidK<R>& Pk, bool rel) {
       for (int64_t t = t1 - 1; t >= t0; --t) {
         unsigned char* stt = pool(pid, (int)(t - t0));
         const S* pops = reinterpret_cast<const S*>(stt);
-        ChainK<R> Ct = C;
-        Ct.x = reinterpret_cast<R*>(at(stt, x_));
-        Ct.xl = reinterpret_cast<R*>(at(stt, xl_));
-        Ct.img = reinterpret_cast<int*>(at(stt, img_));
-        Ct.v = reinterpret_cast<R*>(at(stt, v_));
-        Ct.F = reinterpret_cast<R*>(at(stt, F_));
-        Ct.Fc = reinterpret_cast<R*>(at(stt, Fc_));
         const uint32_t kt = rel ? (uint32_t)(t - t0) : (uint32_t)(k0 + t);
         // the adjoint LB kernel (all nodes) and, beside it, the bead adjoint (one block), which
         // adds its forced-node terms to lambda once the LB kernel has written it
@@ -429,7 +479,8 @@ class EngineT final : public Engine {
         lbd.gridDim = dim3(1);
         lbd.blockDim = dim3(512);
         lbd.dynamicSmemBytes = smem;
-        cuda_check(cudaLaunchKernelEx(&lbd, k_adj_bead<S, R, DEV>, pops, lin, lout, Pk, Ct, A, kt), "adjoint bead");
+        cuda_check(cudaLaunchKernelEx(&lbd, k_adj_bead<R>, lin, lout, Pk, C, A, prep(pid, (int)(t - t0)), prep_bytes),
+                   "adjoint bead");
         cur_lam ^= 1;
       }
     };
@@ -446,14 +497,7 @@ class EngineT final : public Engine {
       k_store_value<uint32_t><<<1, 1, 0, st>>>(ctr, (uint32_t)(k0 + t0));
       cuda_check(cudaGetLastError(), "step counter");
       if (!g) {
-        if (!guard.cs) cuda_check(cudaStreamCreateWithFlags(&guard.cs, cudaStreamNonBlocking), "capture stream");
-        cudaGraph_t gr = nullptr;
-        cuda_check(cudaStreamBeginCapture(guard.cs, cudaStreamCaptureModeThreadLocal), "begin capture");
-        ops(guard.cs, true);
-        cuda_check(cudaStreamEndCapture(guard.cs, &gr), "end capture");
-        const cudaError_t ie = cudaGraphInstantiate(&g, gr, 0);
-        cudaGraphDestroy(gr);
-        cuda_check(ie, "instantiate segment graph");
+        g = capture([&](cudaStream_t cs) { ops(cs, true); });
       } else {
         book();
       }
@@ -473,12 +517,6 @@ class EngineT final : public Engine {
           [&](cudaStream_t st, bool rel) { reverse_ops(t0, t1, pid, st, rel ? Prev : P, rel); },
           [&] { cur_lam ^= (int)((t1 - t0) & 1); });  // the captured sequence's effect on the parity
     };
-    cuda_check(cudaStreamCreateWithFlags(&guard.s2, cudaStreamNonBlocking), "adjoint stream");
-    {
-      cudaEvent_t fwd = new_event();  // the forward pass and its checkpoints are complete
-      cuda_check(cudaEventRecord(fwd, s), "event");
-      cuda_check(cudaStreamWaitEvent(guard.s2, fwd, 0), "wait");
-    }
     std::vector<cudaEvent_t> rec_done(nck), rev_done(nck);
     recompute(nck - 1, 0);
     rec_done[nck - 1] = new_event();
@@ -496,8 +534,6 @@ class EngineT final : public Engine {
       rev_done[sgi] = new_event();
       cuda_check(cudaEventRecord(rev_done[sgi], s), "event");
     }
-    pop_[0] = own_pop[0];
-    pop_[1] = own_pop[1];
     auto load_state = [&](const unsigned char* src) {
       cuda_check(cudaMemcpyAsync(pop_[cur_], src, popb, cudaMemcpyDeviceToDevice, s), "load pops");
       cuda_check(cudaMemcpyAsync(bead0, src + popb, beadb, cudaMemcpyDeviceToDevice, s), "load beads");
@@ -512,12 +548,20 @@ class EngineT final : public Engine {
     }
     cuda_check(cudaGetLastError(), "initial force adjoint");
     std::vector<R> xbh(n3);
+    std::vector<double> x0h(n3), xTh(n3);
     double zb = 0.0;
+    cuda_check(cudaMemcpyAsync(x0h.data(), x0d, n3 * sizeof(double), cudaMemcpyDeviceToHost, s), "dl x0");
+    cuda_check(cudaMemcpyAsync(xTh.data(), xTd, n3 * sizeof(double), cudaMemcpyDeviceToHost, s), "dl xT");
     cuda_check(cudaMemcpyAsync(xbh.data(), A.xbar, n3 * sizeof(R), cudaMemcpyDeviceToHost, s), "dl xbar");
     cuda_check(cudaMemcpyAsync(&zb, A.zbar, sizeof(double), cudaMemcpyDeviceToHost, s), "dl zbar");
     // 5. leave the context at the end of the forward run
     load_state(base + o_fin);
     cuda_check(cudaStreamSynchronize(s), "adjoint sync");
+    double obj = 0.0;
+    for (size_t t = 0; t < n3; ++t) {
+      const double d = xTh[t] - x0h[t];
+      obj += d * d;
+    }
     *O = obj;
     for (size_t t = 0; t < n3; ++t) gx[t] = (double)xbh[t] - 2.0 * (xTh[t] - x0h[t]);
     *gz = zb;
@@ -908,11 +952,13 @@ class EngineT final : public Engine {
 
   // pending-correction block: deferred steps read slot pslot_^1 (when open) and write
   // pslot_ with node marks; complete steps write slot pslot_ only, without marks
-  PendK<R> pend(bool deferred) const {
+  PendK<R> pend(bool deferred) const { return pend_slots(pslot_, deferred && open_, deferred); }
+  // a step that writes slot c and, with have_prev, reads the other
+  PendK<R> pend_slots(int c, bool have_prev, bool mark) const {
     PendK<R> Pd;
     memset(&Pd, 0, sizeof(Pd));
-    const int c = pslot_, p = pslot_ ^ 1;
-    Pd.have_prev = (deferred && open_) ? 1 : 0;
+    const int p = c ^ 1;
+    Pd.have_prev = have_prev ? 1 : 0;
     Pd.prev_mask = masks_[p];
     Pd.prev_dense = corr_[p];
     Pd.cur_dense = corr_[c];
@@ -920,7 +966,7 @@ class EngineT final : public Engine {
     Pd.cur_pos = p_pos_[c];
     Pd.cur_count = p_count_[c];
     Pd.cur_mask = masks_[c];
-    Pd.mark = deferred ? 1 : 0;
+    Pd.mark = mark ? 1 : 0;
     Pd.cap = cap_;
     Pd.seg0 = 0;
     return Pd;
