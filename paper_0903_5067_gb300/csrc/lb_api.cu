@@ -381,7 +381,6 @@ int lb_sync(lb_ctx* ctx) {
   if (!ctx) return fail(LB_ERR_ARG, "invalid argument: !ctx");
   return guarded([&] {
     if (!ctx->live) return (int)LB_OK;
-    cuda_check(cudaStreamSynchronize(ctx->stream), "stream sync");
     return status_from_device(ctx->eng->read_status(ctx->stream));
   });
 }
@@ -392,8 +391,7 @@ int lb_get_populations(lb_ctx* ctx, double* out, size_t cap) {
   if (cap < need) return fail(LB_ERR_ARG, "population buffer too small");
   return guarded([&] {
     materialise(ctx);
-    ctx->eng->get_populations(out, ctx->stream);
-    return status_from_device(ctx->eng->read_status(ctx->stream));
+    return status_from_device(ctx->eng->get_populations(out, ctx->stream));
   });
 }
 
@@ -422,8 +420,7 @@ int lb_get_beads(lb_ctx* ctx, double* x, double* v, size_t cap) {
   }
   return guarded([&] {
     materialise(ctx);
-    ctx->eng->get_beads(x, v, ctx->stream);
-    return status_from_device(ctx->eng->read_status(ctx->stream));
+    return status_from_device(ctx->eng->get_beads(x, v, ctx->stream));
   });
 }
 
@@ -459,8 +456,7 @@ int lb_get_observables(lb_ctx* ctx, double* out, size_t cap) {
   if (cap < LB_NOBS) return fail(LB_ERR_ARG, "observable buffer too small");
   return guarded([&] {
     materialise(ctx);
-    ctx->eng->observables(out, ctx->step, 0, ctx->stream);
-    return status_from_device(ctx->eng->read_status(ctx->stream));
+    return status_from_device(ctx->eng->observables(out, ctx->step, 0, ctx->stream));
   });
 }
 

@@ -311,6 +311,7 @@ class BatchT final : public Batch {
   ~BatchT() override {
     if (graph_exec_) cudaGraphExecDestroy(graph_exec_);
     if (cap_) cudaStreamDestroy(cap_);
+    if (page_) cudaFreeHost(page_);
   }
 
   size_t workspace_bytes() const override { return bytes_; }
@@ -330,6 +331,12 @@ class BatchT final : public Batch {
 
   void initialise(cudaStream_t s) override {
     bead_g_ = bead_cluster();
+    if (!page_) {  // one page for the read-backs of all replicas
+      int longest = 0;
+      for (auto& e : eng_) longest = std::max(longest, e->chain_length());
+      page_ = new_host_page(longest);
+      for (auto& e : eng_) e->set_host_page(page_);
+    }
     if (sizeof(R) == 8) launch_fill_noise_tables(base_ + noise_off_, s);
     for (size_t r = 0; r < eng_.size(); ++r)
       eng_[r]->initialise(x0_[r].empty() ? nullptr : x0_[r].data(), nullptr, s);
@@ -626,6 +633,7 @@ class BatchT final : public Batch {
   uint32_t* d_step_ = nullptr;
   unsigned long long total_tiles_ = 0;
   int bead_g_ = 1;
+  HostPage* page_ = nullptr;
   int threads_ = 256, bps_ = 0, table_threads_ = -1, cap_max_ = 8;
   bool noise_ = true;
   cudaStream_t cap_ = nullptr;

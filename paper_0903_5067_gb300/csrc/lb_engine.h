@@ -61,9 +61,10 @@ class Engine {
   // n such steps k .. k + n - 1, as CUDA graphs of several steps where there are enough
   virtual void steps_deferred(uint32_t k, int64_t n, cudaStream_t s) = 0;
   virtual void flush(cudaStream_t s) = 0;
-  virtual void get_populations(double* out, cudaStream_t s) = 0;
+  // the synchronising read-backs return the device status word as of their synchronisation
+  virtual unsigned get_populations(double* out, cudaStream_t s) = 0;
   virtual void set_populations(const double* in, cudaStream_t s) = 0;
-  virtual void get_beads(double* x, double* v, cudaStream_t s) = 0;
+  virtual unsigned get_beads(double* x, double* v, cudaStream_t s) = 0;
   // the same read-back enqueued on s without waiting (x, v: host memory that stays valid
   // until the stream reaches the copies; pinned memory makes them asynchronous)
   virtual void enqueue_beads(double* x, double* v, cudaStream_t s) = 0;
@@ -75,7 +76,8 @@ class Engine {
                                    cudaStream_t s) = 0;
   // wait for read-backs in flight on the engine's own stream
   virtual void drain() = 0;
-  virtual void observables(double* out, int64_t step, int accumulate, cudaStream_t s) = 0;
+  // (out null: enqueued only, returns 0)
+  virtual unsigned observables(double* out, int64_t step, int accumulate, cudaStream_t s) = 0;
   virtual void reset_reference(cudaStream_t s) = 0;
   // write the current unwrapped bead positions (3N doubles) to device memory
   virtual void record_frame(double* dst, cudaStream_t s) = 0;

@@ -26,6 +26,21 @@ inline void launch_fill_noise_tables(void* base, cudaStream_t s) {
   cuda_check(cudaGetLastError(), "noise tables");
 }
 
+// A page of page-locked host memory that the device writes read-backs into
+struct HostPage {
+  unsigned status;
+  unsigned pad;
+  double beads[1];  // 6N: positions, velocities
+};
+inline HostPage* new_host_page(int N) {  // null when there is none to be had
+  void* p = nullptr;
+  if (cudaHostAlloc(&p, sizeof(HostPage) + 6 * (size_t)N * sizeof(double), cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return static_cast<HostPage*>(p);
+}
+
 template <class S, class R, bool DEV>
 class EngineT final : public Engine {
  public:
@@ -53,6 +68,7 @@ class EngineT final : public Engine {
     cfg_ = c;
   }
   void set_noise_tables(void* base) { noise_tab_ = base; }
+  void set_host_page(HostPage* p) { page_ = p; }  // of the owner's, for at least this many beads
 
   void initialise(const double* x0, const double* v0, cudaStream_t s) override {
     snap_valid_ = false;
@@ -296,7 +312,8 @@ class EngineT final : public Engine {
     double* const x0d = reinterpret_cast<double*>(base + o_x0);
     double* const xTd = reinterpret_cast<double*>(base + o_xT);
     auto read_beads = [&](double* to) {
-      k_bead_readback<R><<<(unsigned)((n3 + 255) / 256), 256, 0, s>>>(x_, xl_, img_, v_, (int)n3, cfg_.L * cfg_.a, to);
+      k_bead_readback<R><<<(unsigned)((n3 + 255) / 256), 256, 0, s>>>(x_, xl_, img_, v_, (int)n3, cfg_.L * cfg_.a, to, nullptr,
+                                                                          nullptr);
       cuda_check(cudaGetLastError(), "bead read-back");
     };
     read_beads(x0d);
@@ -590,7 +607,7 @@ class EngineT final : public Engine {
   // allocation) is written or read by one conversion kernel over all 19 planes, with no
   // staging copy; other host memory goes through the second population buffer in chunks of
   // as many FP64 planes as it holds, one conversion kernel and one copy per chunk.
-  void get_populations(double* out, cudaStream_t s) override {
+  unsigned get_populations(double* out, cudaStream_t s) override {
     flush(s);
     double* direct = static_cast<double*>(device_view(out, (size_t)Q * nnodes_ * sizeof(double)));
     if (direct) {
@@ -608,7 +625,7 @@ class EngineT final : public Engine {
                    "download planes");
       }
     }
-    cuda_check(cudaStreamSynchronize(s), "sync download");
+    return read_status(s);
   }
 
   void set_populations(const double* in, cudaStream_t s) override {
@@ -634,18 +651,32 @@ class EngineT final : public Engine {
   }
 
   // bead arrays are final once the bead kernel of the last step has run (pending fluid
-  // corrections do not touch them): no flush.  One kernel forms the FP64 unwrapped positions
-  // and velocities in a device staging area, then one copy per output array.
-  void get_beads(double* x, double* v, cudaStream_t s) override {
-    if (N_ == 0) return;
-    enqueue_beads(x, v, s);
+  // corrections do not touch them): no flush.  One kernel writes the FP64 unwrapped positions, the
+  // velocities and the status word straight into a page of page-locked memory, so that a
+  // read-back is one launch and one synchronisation: 33 -> 19 us for a
+  // replica of a batch through Python (a kernel, two copies to the caller's pageable arrays, the status word's
+  // copy, two synchronisations).  Without such a page, device staging and copies.
+  unsigned get_beads(double* x, double* v, cudaStream_t s) override {
+    if (N_ == 0) return read_status(s);
+    const int n3 = 3 * N_;
+    HostPage* pg = page_for_beads();
+    if (!pg) {
+      enqueue_beads(x, v, s);
+      return read_status(s);
+    }
+    k_bead_readback<R><<<(n3 + 255) / 256, 256, 0, s>>>(x_, xl_, img_, v_, n3, cfg_.L * cfg_.a, pg->beads, status_,
+                                                      &pg->status);
+    cuda_check(cudaGetLastError(), "bead read-back");
     cuda_check(cudaStreamSynchronize(s), "sync beads");
+    if (x) memcpy(x, pg->beads, n3 * sizeof(double));
+    if (v) memcpy(v, pg->beads + n3, n3 * sizeof(double));
+    return pg->status;
   }
 
   void enqueue_beads(double* x, double* v, cudaStream_t s) override {
     if (N_ == 0) return;
     const int n3 = 3 * N_;
-    k_bead_readback<R><<<(n3 + 255) / 256, 256, 0, s>>>(x_, xl_, img_, v_, n3, cfg_.L * cfg_.a, rb_);
+    k_bead_readback<R><<<(n3 + 255) / 256, 256, 0, s>>>(x_, xl_, img_, v_, n3, cfg_.L * cfg_.a, rb_, nullptr, nullptr);
     cuda_check(cudaGetLastError(), "bead read-back");
     if (x) cuda_check(cudaMemcpyAsync(x, rb_, n3 * sizeof(double), cudaMemcpyDeviceToHost, s), "dl x");
     if (v) cuda_check(cudaMemcpyAsync(v, rb_ + n3, n3 * sizeof(double), cudaMemcpyDeviceToHost, s), "dl v");
@@ -694,6 +725,7 @@ class EngineT final : public Engine {
 
   ~EngineT() override {
     drop_graphs();
+    if (page_ && own_page_) cudaFreeHost(page_);
     if (capture_) cudaStreamDestroy(capture_);
     if (side_) {
       cudaStreamSynchronize(side_);
@@ -704,7 +736,7 @@ class EngineT final : public Engine {
     }
   }
 
-  void observables(double* out, int64_t step, int accumulate, cudaStream_t s) override {
+  unsigned observables(double* out, int64_t step, int accumulate, cudaStream_t s) override {
     flush(s);
     ObsK<R> O = obs(step, accumulate);
     if (!accumulate) {
@@ -714,10 +746,9 @@ class EngineT final : public Engine {
     }
     k_observables<R><<<1, 256, 0, s>>>(O);
     cuda_check(cudaGetLastError(), "observables");
-    if (out) {
-      cuda_check(cudaMemcpyAsync(out, obs_, kNObs * sizeof(double), cudaMemcpyDeviceToHost, s), "dl obs");
-      cuda_check(cudaStreamSynchronize(s), "sync obs");
-    }
+    if (!out) return 0;
+    cuda_check(cudaMemcpyAsync(out, obs_, kNObs * sizeof(double), cudaMemcpyDeviceToHost, s), "dl obs");
+    return read_status(s);
   }
 
   void reset_reference(cudaStream_t s) override {
@@ -749,11 +780,13 @@ class EngineT final : public Engine {
       for (size_t t = 0; t < xs.size(); ++t) x_stored[t] = (double)xs[t];
   }
 
+  // waits for s
   unsigned read_status(cudaStream_t s) override {
     unsigned st = 0;
-    cuda_check(cudaMemcpyAsync(&st, status_, sizeof(unsigned), cudaMemcpyDeviceToHost, s), "status");
+    unsigned* to = page_ ? &page_->status : &st;  // pageable: the copy itself would wait as well
+    cuda_check(cudaMemcpyAsync(to, status_, sizeof(unsigned), cudaMemcpyDeviceToHost, s), "status");
     cuda_check(cudaStreamSynchronize(s), "sync status");
-    return st;
+    return *to;
   }
 
   // checkpoint: populations (storage type, L^3 per plane), bead arrays, xref, acc, counter
@@ -806,6 +839,15 @@ class EngineT final : public Engine {
     mv(acc_, 4 * sizeof(double));
     mv(nonpos_, sizeof(unsigned long long));
     return p;
+  }
+
+  // the page, from the second bead read-back on (allocating it costs as much as one saves)
+  HostPage* page_for_beads() {
+    if (!page_ && ++bead_reads_ == 2) {
+      page_ = new_host_page(N_);
+      own_page_ = page_ != nullptr;
+    }
+    return page_;
   }
 
   static constexpr int kGraphSteps = 16;  // even: buffers and slots alternate
@@ -1272,6 +1314,9 @@ class EngineT final : public Engine {
   }
 
   Config cfg_;
+  HostPage* page_ = nullptr;
+  bool own_page_ = false;
+  int bead_reads_ = 0;
   bool own_tables_ = false;
   void* noise_tab_ = nullptr;
   int L_ = 0, N_ = 0, cap_ = 8, nparts_ = 0, nsub_ = 1;
