@@ -78,7 +78,7 @@ struct BatchLB {
 // (Sec. II B), one or two nodes per thread.  A node marked by the previous step adds that
 // step's corrections to what it pulls (replicas without a chain have no correction field and
 // are never marked); the pull is issued before the mark is known, and one copy of the
-// collision follows, as in lb_tile.  Coordinates come from the slot by two multiply-highs.
+// collision follows, as in lb_node.  Coordinates come from the slot by two multiply-highs.
 template <class S, class R, bool DEV, bool NOISE>
 __device__ __forceinline__ void batch_tile(const BatchLB<S, R>& B, const int r, const unsigned long long tile,
                                            const int parity, const uint32_t step, unsigned char* dsm) {
@@ -86,6 +86,7 @@ __device__ __forceinline__ void batch_tile(const BatchLB<S, R>& B, const int r, 
   const int pslot = parity ^ 1;  // the previous step's corrections
   const BatchRep<S, R>& rp = B.rep[r];
   const unsigned sl = (unsigned)(tile - rp.tile0) * T + threadIdx.x;
+  const unsigned part = __ballot_sync(~0u, sl < rp.nslots);
   if (sl >= rp.nslots) return;
   const unsigned L = rp.L;
   const unsigned row = div_magic(sl, rp.mag_row);
@@ -94,39 +95,21 @@ __device__ __forceinline__ void batch_tile(const BatchLB<S, R>& B, const int r, 
   const unsigned y = row - z * L;
   const unsigned pl = (unsigned)rp.plane;
   const bool corr = rp.p_dense[pslot] != nullptr;
-  R* col = reinterpret_cast<R*>(dsm);
   if (sizeof(R) == 4 && rp.pair) {
     const unsigned x0 = 2 * xs;
     const unsigned node = x0 + L * row;
     const unsigned mw = corr ? B.mask[pslot][rp.seg0 + (node >> kSegShift)] >> (node & 31u) : 0u;
     R n0[Q], n1[Q];
     lb_pull2<S, R, unsigned>(rp.pop[parity], L, pl, x0, y, z, n0, n1);
-    if (mw & 3u) {  // marked nodes stage their corrections one after the other
-#pragma unroll 1
-      for (unsigned j = 0; j < 2; ++j) {
-        if (!((mw >> j) & 1u)) continue;
-        stage_corrections<R>(rp.p_dense[pslot], rp.plane, L, x0 + j, y, z, col + threadIdx.x, T);
-        if (j == 0) {
-#pragma unroll
-          for (int i = 0; i < Q; ++i) n0[i] += col[threadIdx.x + i * T];
-        } else {
-#pragma unroll
-          for (int i = 0; i < Q; ++i) n1[i] += col[threadIdx.x + i * T];
-        }
-      }
-    }
+    add_corrections<R, true>(rp.p_dense[pslot], rp.plane, L, node, mw, part, dsm, n0, n1);
     lb_collide2_store<S, R, DEV, NOISE, unsigned>(n0, n1, rp.pop[parity ^ 1], B.P, pl, B.rk[r], rp.nonpos, step,
                                                   node);
   } else {
     const unsigned node = xs + L * row;
-    const unsigned mw = corr ? B.mask[pslot][rp.seg0 + (node >> kSegShift)] : 0u;
+    const unsigned mw = corr ? B.mask[pslot][rp.seg0 + (node >> kSegShift)] >> (node & 31u) : 0u;
     R n[Q];
     lb_pull<S, R, unsigned>(rp.pop[parity], L, pl, xs, y, z, n);
-    if ((mw >> (node & 31u)) & 1u) {
-      stage_corrections<R>(rp.p_dense[pslot], rp.plane, L, xs, y, z, col + threadIdx.x, T);
-#pragma unroll
-      for (int i = 0; i < Q; ++i) n[i] += col[threadIdx.x + i * T];
-    }
+    add_corrections<R, false>(rp.p_dense[pslot], rp.plane, L, node, mw, part, dsm, n, n);
     lb_collide_store<S, R, DEV, NOISE, unsigned>(n, rp.pop[parity ^ 1], B.P, pl, B.rk[r], rp.nonpos, step, node);
   }
 }
@@ -146,7 +129,7 @@ constexpr unsigned kChunk = 2;
 template <class S, class R, bool DEV, bool NOISE, bool PERSIST>
 __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_batch_lb(const __grid_constant__ BatchLB<S, R> B, int parity,
                                                    const uint32_t* __restrict__ d_step, uint32_t j) {
-  extern __shared__ __align__(16) unsigned char dsm[];  // staged corrections, 19 x T
+  extern __shared__ __align__(16) unsigned char dsm[];  // staged corrections, by warp
   // every grid releases the next at once, and one more block than there are tiles (!PERSIST), or
   // every block at its end, waits for the grid before: the bead kernel of this step or the previous
   // group's LB kernel, so that this grid's completion stands for all before it
@@ -180,6 +163,7 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_batch_lb(const 
     for (unsigned long long tile = cur; tile < t_end; ++tile) {
       while (r + 1 < B.nrep && B.rep[r + 1].tile0 <= tile) ++r;  // uniform
       batch_tile<S, R, DEV, NOISE>(B, r, tile, parity, step, dsm);
+      __syncwarp();
     }
     __syncthreads();
     cur = s_next;
@@ -352,7 +336,7 @@ class BatchT final : public Batch {
     for (auto& e : eng_) cap_max_ = e->pending_capacity() > cap_max_ ? e->pending_capacity() : cap_max_;
     // the engines zeroed their pending counts; no node is marked
     cuda_check(cudaMemsetAsync(flags_[0], 0, 2 * max_segs_ * sizeof(unsigned), s), "memset marks");
-    const size_t lbsm = (size_t)Q * 512 * sizeof(R);
+    const size_t lbsm = 512 / 32 * (size_t)WarpStage<R>::kBytes;
     if (lbsm > 48 * 1024) {  // FP64: staged corrections of a 512-thread tile
       for (int v = 0; v < 4; ++v)
         cuda_check(cudaFuncSetAttribute(lb_kernel(v & 1, v >> 1), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -593,7 +577,7 @@ class BatchT final : public Batch {
       memset(&lc, 0, sizeof(lc));
       lc.gridDim = dim3(grid);
       lc.blockDim = dim3(threads_);
-      lc.dynamicSmemBytes = (size_t)Q * threads_ * sizeof(R);
+      lc.dynamicSmemBytes = threads_ / 32 * (size_t)WarpStage<R>::kBytes;
       lc.stream = s;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

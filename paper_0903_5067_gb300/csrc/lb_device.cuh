@@ -635,38 +635,121 @@ __device__ __forceinline__ void lb_pull(const S* __restrict__ src, const unsigne
   }
 }
 
-// Stage the previous step's corrections at the 19 pull sources of node (x, y, z) into
-// col[i * stride] (shared memory).  A rolled loop with the directions unpacked from constants
-// (this rare path must not raise the register count of the LB kernels), issuing asynchronous
-// global-to-shared copies (cp.async) so that the 19 loads are in flight together; the
-// calling thread waits for its own copies.
+// Shared memory of one warp that adds the previous step's corrections: coordinates and 19 values
+// of up to 32 marked nodes.
 template <class R>
-__device__ __forceinline__ void stage_corrections(const R* __restrict__ corr, unsigned long long plane, unsigned L,
-                                                  unsigned x, unsigned y, unsigned z, R* col, unsigned stride) {
+struct WarpStage {
+  static constexpr unsigned kNodes = 32;
+  static constexpr unsigned kBytes = kNodes * (sizeof(uint2) + Q * sizeof(R));
+  uint2* at;  // x | y << 16, z
+  R* v;       // v[19 slot + i]
+  __device__ __forceinline__ WarpStage(unsigned char* smem, unsigned warp)
+      : at(reinterpret_cast<uint2*>(smem + warp * kBytes)), v(reinterpret_cast<R*>(at + kNodes)) {}
+};
+
+// Slots of a thread's marked nodes in the pass that begins at slot `base` (2^31 and more: not in it).
+template <bool PAIR>
+struct MarkedSlots {
+  unsigned s0, s1, total, below;
+  __device__ __forceinline__ MarkedSlots(unsigned mw, unsigned part, unsigned base) {
+    const unsigned b0 = __ballot_sync(part, mw & 1u), b1 = PAIR ? __ballot_sync(part, mw & 2u) : 0u;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(below));
+    total = __popc(b0) + __popc(b1);
+    s0 = (mw & 1u) ? __popc(b0 & below) - base : ~0u;
+    s1 = PAIR && (mw & 2u) ? __popc(b0) + __popc(b1 & below) - base : ~0u;
+  }
+};
+
+// Stage the corrections at the 19 pull sources of the warp's marked nodes of slots base ... base +
+// kNodes - 1 (the first nodes' slots, then, with PAIR, the second ones', in the order of the lanes).
+// The coordinates are listed in shared memory and the 19 sources of all of them dealt out to the
+// lanes of `part`.
+template <class R, bool PAIR>
+__device__ __forceinline__ void stage_marked(const R* __restrict__ corr, unsigned long long plane, unsigned L,
+                                          unsigned node, unsigned mw, unsigned part, unsigned base,
+                                          unsigned char* smem) {
   static_assert(sizeof(R) == 4 || sizeof(R) == 8, "cp.async copies 4 or 8 bytes");
   constexpr unsigned long long PX = pack_component(0), PY = pack_component(1), PZ = pack_component(2);
+  constexpr unsigned kNodes = WarpStage<R>::kNodes;
+  const WarpStage<R> W(smem, (threadIdx.x + blockDim.x * threadIdx.y) / 32);
+  const MarkedSlots<PAIR> m(mw, part, base);
+  const unsigned row = node / L, x = node - row * L, z = row / L, y = row - z * L;
+  if (m.s0 < kNodes) W.at[m.s0] = make_uint2(x | y << 16, z);
+  if (PAIR && m.s1 < kNodes) W.at[m.s1] = make_uint2((x + 1) | y << 16, z);
+  __syncwarp(part);
+  const unsigned items = Q * (m.total - base < kNodes ? m.total - base : kNodes);
 #pragma unroll 1
-  for (int i = 0; i < Q; ++i) {
-    int sx = (int)x - unpack_component(PX, i), sy = (int)y - unpack_component(PY, i),
-        sz = (int)z - unpack_component(PZ, i);
+  for (unsigned k = __popc(part & m.below); k < items; k += __popc(part)) {
+    const unsigned slot = k / Q, i = k - slot * Q;
+    const uint2 c = W.at[slot];
+    int sx = (int)(c.x & 0xFFFFu) - unpack_component(PX, i), sy = (int)(c.x >> 16) - unpack_component(PY, i),
+        sz = (int)c.y - unpack_component(PZ, i);
     sx = sx < 0 ? sx + (int)L : (sx >= (int)L ? sx - (int)L : sx);
     sy = sy < 0 ? sy + (int)L : (sy >= (int)L ? sy - (int)L : sy);
     sz = sz < 0 ? sz + (int)L : (sz >= (int)L ? sz - (int)L : sz);
-    const unsigned idx = (unsigned)sx + L * ((unsigned)sy + L * (unsigned)sz);
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(col + i * stride);
-    const R* src = corr + (unsigned long long)i * plane + idx;
+    const R* from = corr + ((unsigned long long)i * plane + ((unsigned)sx + L * ((unsigned)sy + L * (unsigned)sz)));
+    const unsigned to = (unsigned)__cvta_generic_to_shared(W.v + k);
     if (sizeof(R) == 4)
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(from) : "memory");
     else
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to), "l"(from) : "memory");
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp(part);
+}
+
+// The same as a call, for the FP32 kernels: they hold 19 or 38 populations across it in as many
+// registers as they have, and what has to make room is then saved around the call, on this rare
+// path.  (Inlined, the spills were on every warp's path: 53.0 against 50.2 us per step at L = 128.
+// Kernels that had spilled before gained by the call: 43.9 to 42.5 us in BF16 at L = 128, 131.7 to
+// 127.2 us for 64 replicas of L = 16 ... 64.  The FP64 kernels have the registers: 18.9 us with the
+// call against 18.2 at L = 24.)
+template <bool PAIR>
+__device__ __noinline__ void stage_marked_call(const float* __restrict__ corr, unsigned long long plane, unsigned L,
+                                               unsigned node, unsigned mw, unsigned part, unsigned base,
+                                               unsigned char* smem) {
+  stage_marked<float, PAIR>(corr, plane, L, node, mw, part, base, smem);
+}
+
+// Add the previous step's corrections at the pull sources of the warp's marked nodes to what they
+// pulled: bit 0 of mw marks the thread's node, with PAIR bit 1 its second one, `node` + 1.  Called by
+// all lanes of `part`.  A warp with m marked nodes runs 19 m / 32 rounds of index arithmetic
+// (stage_marked) and waits for one flight of asynchronous copies (cp.async).  A bead marks about 4
+// nodes of a row, and a kernel whose blocks are all resident ends with its slowest warp: with
+// every marked thread staging its own nodes one after the other, 19 rounds and one flight each,
+// the step at L = 64, N = 64 (FP32) took 11.4 us, of which 3.2 went with the corrections left out;
+// now 8.6 (7.4 without a chain).
+template <class R, bool PAIR>
+__device__ __forceinline__ void add_corrections(const R* __restrict__ corr, unsigned long long plane, unsigned L,
+                                                unsigned node, unsigned mw, unsigned part, unsigned char* smem,
+                                                R* n0, R* n1) {
+  if (!__any_sync(part, mw & (PAIR ? 3u : 1u))) return;
+  constexpr unsigned kNodes = WarpStage<R>::kNodes;
+#pragma unroll 1
+  for (unsigned base = 0;; base += kNodes) {
+    if constexpr (sizeof(R) == 4)
+      stage_marked_call<PAIR>(corr, plane, L, node, mw, part, base, smem);
+    else
+      stage_marked<R, PAIR>(corr, plane, L, node, mw, part, base, smem);
+    const WarpStage<R> W(smem, (threadIdx.x + blockDim.x * threadIdx.y) / 32);
+    const MarkedSlots<PAIR> m(mw, part, base);
+    if (m.s0 < kNodes) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) n0[i] += W.v[Q * m.s0 + i];
+    }
+    if (PAIR && m.s1 < kNodes) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) n1[i] += W.v[Q * m.s1 + i];
+    }
+    __syncwarp(part);  // all have read before the next pass or tile writes
+    if (!PAIR || m.total <= base + kNodes) break;
+  }
 }
 
 // One node: pull-stream + collide (Sec. II B, Eq. 3).  Every thread loads its 19 populations and
-// its mark word together; a node marked by the previous deferred step then stages that step's
-// corrections at its pull sources (in shared memory at stage[i * T], T threads per block) and
-// adds them to what it pulled, and one copy of the collision follows.  (Branching on the mark
+// its mark word together; a node marked by the previous deferred step then adds that step's
+// corrections at its pull sources to what it pulled (add_corrections: `part` are the warp's lanes
+// that have a node), and one copy of the collision follows.  (Branching on the mark
 // before the loads put an L2 round trip in front of every warp's loads, 1.4 us per launch at
 // L = 128 with no node marked; with two inlined copies of the update, a warp holding marked and
 // unmarked nodes ran both: 67.8 against 64.0 us with 1.5 % of the nodes marked.)
@@ -675,18 +758,14 @@ __device__ __forceinline__ void stage_corrections(const R* __restrict__ corr, un
 template <class S, class R, bool DEV, bool NOISE, class I, bool CORR>
 __device__ __forceinline__ void lb_node(const S* __restrict__ src, S* __restrict__ dst, const FluidK<R>& P,
                                         const PendK<R>& Pd, const uint32_t step, unsigned x, unsigned y, unsigned z,
-                                        R* stage, unsigned T) {
+                                        unsigned char* smem, unsigned part) {
   const unsigned L = P.L;
   const unsigned node = x + L * (y + L * z);
-  const unsigned mw = CORR && Pd.have_prev ? Pd.prev_mask[Pd.seg0 + (node >> kSegShift)] : 0u;
+  const unsigned mw = CORR && Pd.have_prev ? Pd.prev_mask[Pd.seg0 + (node >> kSegShift)] >> (node & 31u) : 0u;
   const I pl = (I)P.plane;
   R n[Q];
   lb_pull<S, R, I>(src, L, pl, x, y, z, n);
-  if (CORR && ((mw >> (node & 31u)) & 1u)) {
-    stage_corrections<R>(Pd.prev_dense, Pd.plane, L, x, y, z, stage, T);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) n[i] += stage[i * T];
-  }
+  if (CORR) add_corrections<R, false>(Pd.prev_dense, Pd.plane, L, node, mw, part, smem, n, n);
   lb_collide_store<S, R, DEV, NOISE, I>(n, dst, P, pl, P.rk, P.nonpos, step, node);
 }
 
@@ -743,32 +822,18 @@ __device__ __forceinline__ void lb_pull2(const S* __restrict__ src, const unsign
 }
 
 // Two nodes (x0, y, z) and (x0 + 1, y, z), x0 even, L even: the same update as lb_node, node by
-// node, with the 19 post-collision pairs written by two-element stores.  Marked nodes stage their
-// corrections one node after the other into the same 19 T values.
+// node, with the 19 post-collision pairs written by two-element stores.
 template <class S, class R, bool DEV, bool NOISE, class I, bool CORR>
 __device__ __forceinline__ void lb_nodes2(const S* __restrict__ src, S* __restrict__ dst, const FluidK<R>& P,
                                           const PendK<R>& Pd, const uint32_t step, unsigned x0, unsigned y,
-                                          unsigned z, R* stage, unsigned T) {
+                                          unsigned z, unsigned char* smem, unsigned part) {
   const unsigned L = P.L;
   const unsigned node = x0 + L * (y + L * z);
   const unsigned mw = CORR && Pd.have_prev ? Pd.prev_mask[Pd.seg0 + (node >> kSegShift)] >> (node & 31u) : 0u;
   const I pl = (I)P.plane;
   R n0[Q], n1[Q];
   lb_pull2<S, R, I>(src, L, pl, x0, y, z, n0, n1);
-  if (CORR && (mw & 3u)) {
-#pragma unroll 1
-    for (unsigned j = 0; j < 2; ++j) {
-      if (!((mw >> j) & 1u)) continue;
-      stage_corrections<R>(Pd.prev_dense, Pd.plane, L, x0 + j, y, z, stage, T);
-      if (j == 0) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) n0[i] += stage[i * T];
-      } else {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) n1[i] += stage[i * T];
-      }
-    }
-  }
+  if (CORR) add_corrections<R, true>(Pd.prev_dense, Pd.plane, L, node, mw, part, smem, n0, n1);
   lb_collide2_store<S, R, DEV, NOISE, I>(n0, n1, dst, P, pl, P.rk, P.nonpos, step, node);
 }
 
@@ -808,15 +873,14 @@ __global__ void __launch_bounds__(256, LbMinBlocks<R, PAIR>::value) k_lb_step(co
   if (P.pdl & 1) grid_dependency_wait();
   allow_dependent_launch();
   const uint32_t k = launch_step(P, step);
-  const unsigned T = blockDim.x * blockDim.y;
-  R* const stage = reinterpret_cast<R*>(lsm) + (threadIdx.x + blockDim.x * threadIdx.y);
   const unsigned xt = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  if constexpr (PAIR) {
-    if (2 * xt < P.L && y < P.L)
-      lb_nodes2<S, R, DEV, NOISE, I, CORR>(src, dst, P, Pd, k, 2 * xt, y, blockIdx.z, stage, T);
-  } else {
-    if (xt < P.L && y < P.L) lb_node<S, R, DEV, NOISE, I, CORR>(src, dst, P, Pd, k, xt, y, blockIdx.z, stage, T);
-  }
+  const bool in = (PAIR ? 2 * xt : xt) < P.L && y < P.L;
+  const unsigned part = CORR ? __ballot_sync(~0u, in) : 0u;
+  if (!in) return;
+  if constexpr (PAIR)
+    lb_nodes2<S, R, DEV, NOISE, I, CORR>(src, dst, P, Pd, k, 2 * xt, y, blockIdx.z, lsm, part);
+  else
+    lb_node<S, R, DEV, NOISE, I, CORR>(src, dst, P, Pd, k, xt, y, blockIdx.z, lsm, part);
 }
 
 // n / d for n < 2^24 and 2 <= d <= 256 by one multiply-high with m = ceil(2^32 / d): with
@@ -846,12 +910,12 @@ __global__ void __launch_bounds__(256) k_lb_linear(const S* __restrict__ src, S*
     grid_dependency_wait();
     return;
   }
+  const unsigned part = CORR ? __ballot_sync(~0u, node < nnodes) : 0u;
   if (node >= nnodes) return;
   const uint32_t k = launch_step(P, step);
   const unsigned row = div_magic(node, mag_L), x = node - row * P.L;
   const unsigned z = div_magic(row, mag_L), y = row - z * P.L;
-  lb_node<S, R, DEV, NOISE, unsigned, CORR>(src, dst, P, Pd, k, x, y, z, reinterpret_cast<R*>(lsm) + threadIdx.x,
-                                            blockDim.x);
+  lb_node<S, R, DEV, NOISE, unsigned, CORR>(src, dst, P, Pd, k, x, y, z, lsm, part);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -1080,7 +1080,7 @@ class EngineT final : public Engine {
   struct LbLaunch {
     bool linear;
     dim3 blk, grd;
-    size_t stage_bytes;  // staged corrections of marked nodes: 19 values per thread
+    size_t stage_bytes;  // staged corrections of marked nodes, by warp
   };
   LbLaunch lb_launch(bool waiting) const {
     LbLaunch q;
@@ -1094,7 +1094,7 @@ class EngineT final : public Engine {
       lb_launch_shape(q.blk, q.grd, pair_nodes());
       if (waiting) q.grd.z += 1;  // the plane of waiting blocks
     }
-    q.stage_bytes = (size_t)Q * q.blk.x * q.blk.y * sizeof(R);
+    q.stage_bytes = (size_t)(q.blk.x * q.blk.y / 32) * WarpStage<R>::kBytes;
     return q;
   }
   // threads along x cover a row of L nodes (L/2 threads with two nodes each), up to 256 per
