@@ -120,6 +120,7 @@ struct FluidK {
   unsigned long long* nonpos;  // counter of non-positive densities met by the noise
   int pdl;         // launch chaining of the LB kernel: bit 0 waits for the previous grid before
                    // reading, bit 1 waits for it before completing (see k_lb_step)
+  unsigned row, mag_row, rows;  // k_lb_step: threads per row segment, its reciprocal, rows per block
   NoiseTab tab;    // double precision: the noise's radii and angles
   // null, or a device counter the step kernels add their step argument to (graph replays of a
   // fixed sequence of launches at other step numbers)
@@ -843,7 +844,8 @@ __device__ __forceinline__ void lb_nodes2(const S* __restrict__ src, S* __restri
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_dependent_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// LB kernel: 3D grid of (x-row segments) x (y rows) x z planes, plus (when it follows the
+// LB kernel: 3D grid of (x-row segments) x (groups of y rows) x z planes (a block's threads take
+// P.rows row segments of P.row threads, one after the other: lb_row_shape), plus (when it follows the
 // bead kernel of its step) one more plane of blocks that only wait.  Every grid releases the
 // next one at once.  Launched after the previous LB kernel (no chain): it waits for that grid
 // before reading (P.pdl bit 0), so that only the launch latency and block scheduling overlap.
@@ -860,6 +862,14 @@ struct LbMinBlocks {
   static constexpr int value = sizeof(R) == 4 ? (PAIR ? 4 : 6) : 1;
 };
 
+// n / d for n < 2^24 and 2 <= d <= 256 by one multiply-high with m = ceil(2^32 / d): with
+// e = m d - 2^32 < d, n m / 2^32 = n / d + n e / (d 2^32) and n e < 2^32 keeps the error below
+// the distance of n / d to the next integer (checked exhaustively for every d and n in range).
+__host__ __device__ __forceinline__ unsigned magic_of(unsigned d) {
+  return (unsigned)((0x100000000ull + d - 1) / d);
+}
+__device__ __forceinline__ unsigned div_magic(unsigned n, unsigned m) { return __umulhi(n, m); }
+
 // PAIR: two nodes per thread along x (lb_nodes2, L even), else one (lb_node).
 template <class S, class R, bool DEV, bool NOISE, class I, bool CORR, bool PAIR>
 __global__ void __launch_bounds__(256, LbMinBlocks<R, PAIR>::value) k_lb_step(const S* __restrict__ src, S* __restrict__ dst,
@@ -873,8 +883,9 @@ __global__ void __launch_bounds__(256, LbMinBlocks<R, PAIR>::value) k_lb_step(co
   if (P.pdl & 1) grid_dependency_wait();
   allow_dependent_launch();
   const uint32_t k = launch_step(P, step);
-  const unsigned xt = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  const bool in = (PAIR ? 2 * xt : xt) < P.L && y < P.L;
+  const unsigned ty = div_magic(threadIdx.x, P.mag_row);
+  const unsigned xt = blockIdx.x * P.row + (threadIdx.x - ty * P.row), y = blockIdx.y * P.rows + ty;
+  const bool in = ty < P.rows && (PAIR ? 2 * xt : xt) < P.L && y < P.L;
   const unsigned part = CORR ? __ballot_sync(~0u, in) : 0u;
   if (!in) return;
   if constexpr (PAIR)
@@ -882,14 +893,6 @@ __global__ void __launch_bounds__(256, LbMinBlocks<R, PAIR>::value) k_lb_step(co
   else
     lb_node<S, R, DEV, NOISE, I, CORR>(src, dst, P, Pd, k, xt, y, blockIdx.z, lsm, part);
 }
-
-// n / d for n < 2^24 and 2 <= d <= 256 by one multiply-high with m = ceil(2^32 / d): with
-// e = m d - 2^32 < d, n m / 2^32 = n / d + n e / (d 2^32) and n e < 2^32 keeps the error below
-// the distance of n / d to the next integer (checked exhaustively for every d and n in range).
-__host__ __device__ __forceinline__ unsigned magic_of(unsigned d) {
-  return (unsigned)((0x100000000ull + d - 1) / d);
-}
-__device__ __forceinline__ unsigned div_magic(unsigned n, unsigned m) { return __umulhi(n, m); }
 
 // The same launch over consecutive nodes (4 <= L <= 256), one block of threads after the other, with
 // one more block that waits, for the FP64 kernel.  That kernel is bound by the FP64 pipe (2

@@ -409,7 +409,7 @@ class EngineT final : public Engine {
       cuda_check(cudaFuncSetAttribute(k_adj_prep<S, R, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prep_smem),
                  "adjoint smem");
     dim3 blk, grd;
-    lb_launch_shape(blk, grd, false);  // the adjoint LB kernel: one node per thread
+    lb_launch_shape(blk, grd);
     int cur_lam = 0;
     // 3. reverse sweep over the segments.  The states t0 .. t1 - 1 of a segment sit in the
     //    slots of a pool: slot 0 a copy of its checkpoint, slots 1 .. written by the
@@ -961,6 +961,9 @@ class EngineT final : public Engine {
     const bool chained = ev0 == nullptr;
     P.pdl = chained ? (N_ > 0 ? 2 : 1) : 0;
     const LbLaunch q = lb_launch((P.pdl & 2) != 0);
+    P.row = q.row;
+    P.mag_row = magic_of(q.row);
+    P.rows = q.rows;
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof(lc));
     lc.gridDim = q.grd;
@@ -1076,10 +1079,11 @@ class EngineT final : public Engine {
 
   // How the LB kernel covers the box: in FP64 consecutive nodes (k_lb_linear; its division needs
   // L <= 256), in blocks of 256, halved down to one warp while there are fewer than two blocks per
-  // SM; else rows (lb_launch_shape).
+  // SM; else rows (lb_row_shape).
   struct LbLaunch {
-    bool linear;
+    bool linear = false;
     dim3 blk, grd;
+    unsigned row = 32, rows = 1;  // k_lb_step: threads per row segment and row segments per block
     size_t stage_bytes;  // staged corrections of marked nodes, by warp
   };
   LbLaunch lb_launch(bool waiting) const {
@@ -1091,16 +1095,39 @@ class EngineT final : public Engine {
       q.blk = dim3(t);
       q.grd = dim3((unsigned)((nnodes_ + t - 1) / t) + (waiting ? 1 : 0));
     } else {
-      lb_launch_shape(q.blk, q.grd, pair_nodes());
+      lb_row_shape(q);
       if (waiting) q.grd.z += 1;  // the plane of waiting blocks
     }
-    q.stage_bytes = (size_t)(q.blk.x * q.blk.y / 32) * WarpStage<R>::kBytes;
+    q.stage_bytes = (size_t)(q.blk.x / 32) * WarpStage<R>::kBytes;
     return q;
   }
-  // threads along x cover a row of L nodes (L/2 threads with two nodes each), up to 256 per
-  // block; the rest of the 256 threads take further rows
-  void lb_launch_shape(dim3& blk, dim3& grd, bool pair) const {
-    const unsigned row = pair ? (unsigned)L_ / 2 : (unsigned)L_;
+  // Rows of k_lb_step: a block of `blk` threads takes `rows` rows (segments of `row` threads, which
+  // may begin anywhere in a warp).  Padding the rows to whole warps left up to half of the lanes
+  // idle: us per step, FP32 without a chain, L = 72: 14.2 padded, 9.4 now; 80: 17.0, 11.4; 96: 25.1,
+  // 19.9; 112: 34.1, 33.7; 16: 3.1, 2.6.  Of the blocks of up to 256 threads the ones with the most
+  // lanes in use, with 128 threads or fewer where the difference is below 2 %: they end and begin
+  // more evenly (L = 64: 7.4 and 7.15; BF16 L = 128: 40.2 and 39.5).  A box with a chain that has at
+  // most two padded blocks per SM waits for the bead step, beside which fewer warps are better
+  // (L = 25, N = 16: 6.9 padded, 7.3 with rows of 25 threads).
+  void lb_row_shape(LbLaunch& q) const {
+    const unsigned L = (unsigned)L_, n = pair_nodes() ? L / 2 : L;
+    const unsigned padded = n > 224 ? 256 : (n + 31) / 32 * 32, per = 256 / padded;
+    const bool small = N_ > 0 && (unsigned long long)L * ((L + per - 1) / per) <= 304;
+    q.row = n < 2 || n > 256 || small ? padded : n;
+    q.rows = small ? per : 1;
+    const unsigned segs = (n + q.row - 1) / q.row;
+    auto threads = [&](unsigned k) { return (q.row * k + 31) / 32 * 32; };
+    auto groups = [&](unsigned k) { return (L + k - 1) / k; };
+    auto lanes = [&](unsigned k) { return (double)segs * groups(k) * threads(k); };  // of a plane of nodes
+    for (unsigned k = 2; !small && k <= L && q.row * k <= 256; ++k)
+      if (lanes(k) * (threads(k) <= 128 ? 1.0 : 1.02) <= lanes(q.rows)) q.rows = k;
+    q.blk = dim3(threads(q.rows));
+    q.grd = dim3(segs, groups(q.rows), L);
+  }
+  // the adjoint LB kernel: threads along x cover a row of L nodes, up to 256 per block; the rest of
+  // the 256 threads take further rows
+  void lb_launch_shape(dim3& blk, dim3& grd) const {
+    const unsigned row = (unsigned)L_;
     unsigned bx = (row + 31) / 32 * 32;
     if (bx > 256) bx = 256;
     const unsigned by = 256 / bx;
