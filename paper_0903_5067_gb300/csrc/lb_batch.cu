@@ -171,12 +171,12 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_batch_lb(const 
   grid_dependency_wait();
 }
 
-// One cluster of G 256-thread blocks per replica's chain (a chain that needs the sorted grouping runs
+// One cluster of G blocks of 256 or 384 threads per replica's chain (a chain that needs the sorted grouping runs
 // on its first block): in FP32 at most 80 registers per thread, which leaves room on its SM for
 // four 256-thread LB blocks.  Block 0 also zeroes the tile counters the next step's LB launches
 // will use.
 template <class S, class R, bool DEV>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_batch_bead(const ReplicaK<S, R>* __restrict__ reps, int parity,
+__global__ void __launch_bounds__(sizeof(R) == 4 ? 384 : 256, sizeof(R) == 4 ? 2 : 1) k_batch_bead(const ReplicaK<S, R>* __restrict__ reps, int parity,
                                                      const uint32_t* __restrict__ d_step, uint32_t j,
                                                      unsigned long long* __restrict__ counters, int ngroups, int G) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -315,6 +315,7 @@ class BatchT final : public Batch {
 
   void initialise(cudaStream_t s) override {
     bead_g_ = bead_cluster();
+    bead_threads_ = bead_threads();
     if (!page_) {  // one page for the read-backs of all replicas
       int longest = 0;
       for (auto& e : eng_) longest = std::max(longest, e->chain_length());
@@ -437,6 +438,22 @@ class BatchT final : public Batch {
     return std::max(1, std::min({8, (longest + 3) / 4, 152 / (int)eng_.size()}));
   }
 
+  // Threads of a bead block (FP32): 384 where a block has more than 96 corners to gather, 256 where
+  // the LB kernel sets the step or a block has less to do, so that more LB blocks fit beside it.  us
+  // per step with 256 and 384: 64 replicas of L = 15, N = 32, two substeps (256 corners) 23.3 and
+  // 21.4, 128 of them (512) 39.9 and 33.6, 32 (128) 18.2 and 16.2; 24 of L = 25 (96) 19.6 and 20.6; 64
+  // of L = 15, N = 16, one substep (64) 15.0 and 15.3.  FP64, bound by its pipe: 256.
+  int bead_threads() const {
+    if (sizeof(R) == 8) return 256;
+    unsigned long long nodes = 0;
+    int places = 0;  // beads of a block, each at every substep
+    for (auto& e : eng_) {
+      nodes += e->nodes();
+      places = std::max(places, e->config().substeps * ((e->chain_length() + bead_g_ - 1) / bead_g_));
+    }
+    return nodes <= 2000000ull && 8 * places > 96 ? 384 : 256;
+  }
+
   void ensure_streams() {
     if (cap_) return;
     cuda_check(cudaStreamCreateWithFlags(&cap_, cudaStreamNonBlocking), "capture stream");
@@ -551,7 +568,7 @@ class BatchT final : public Batch {
       cudaLaunchConfig_t lc;
       memset(&lc, 0, sizeof(lc));
       lc.gridDim = dim3((unsigned)(R_ * bead_g_));
-      lc.blockDim = dim3(256);
+      lc.blockDim = dim3((unsigned)bead_threads_);
       lc.dynamicSmemBytes = smem_;
       lc.stream = s;
       cudaLaunchAttribute at[2];
@@ -616,7 +633,7 @@ class BatchT final : public Batch {
   ReplicaK<S, R>* d_reps_ = nullptr;
   uint32_t* d_step_ = nullptr;
   unsigned long long total_tiles_ = 0;
-  int bead_g_ = 1;
+  int bead_g_ = 1, bead_threads_ = 256;
   HostPage* page_ = nullptr;
   // Threads of a tile: small blocks end and begin more evenly (FP32, us per step with 128, 256, 512:
   // 64 replicas of L = 16 ... 64: 123.8, 127.1, 139.8; 16 of L = 32: 17.4, 17.8, 19.9; 64 of L = 15:
