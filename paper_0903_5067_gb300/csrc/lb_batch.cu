@@ -5,11 +5,11 @@
 // L = 10..35 for the finite-size extrapolation, Sec. II E and Sec. III B; the CPU-cost study
 // sums three box sizes per chain length, Sec. III C).  Each replica owns an ordinary engine
 // (its memory, noise keys and chain); the batch drives them in lockstep:
-//   - k_batch_bead: one thread block per replica's chain; it releases the LB kernel of the
+//   - k_batch_bead: a cluster of thread blocks per replica's chain; it releases the LB kernel of the
 //     same step at its start (programmatic dependent launch, one stream),
-//   - k_batch_lb: a tile table over all replicas' nodes, persistent thread blocks walking it;
-//     nodes marked by the previous step's bead kernel add its force corrections to what they
-//     pull, the bead kernel adds them to its gathers,
+//   - k_batch_lb: a tile table over all replicas' nodes, one thread block per tile or persistent
+//     blocks walking it; nodes marked by the previous step's bead kernel add its force corrections
+//     to what they pull, the bead kernel adds them to its gathers,
 //   - k_batch_apply: the last step's force corrections, once at the end of each call.
 // Step indices come from a device counter so that a captured CUDA graph of G steps (G even)
 // can be replayed; the tile size and the number of persistent blocks are chosen by a
