@@ -95,7 +95,9 @@ int lb_set_stream(lb_ctx* ctx, void* stream);
 /* Device workspace: size in bytes (valid after lb_add_chain, if any) and binding of a
  * caller-owned device buffer of at least that size, 256-byte aligned, on the current
  * device, that the caller keeps alive until lb_destroy.  Without a binding the library
- * allocates (cudaMalloc) and frees the workspace itself. */
+ * allocates (cudaMalloc) and frees the workspace itself.  Besides it, double-precision contexts
+ * read constant tables for the fluid noise (16 MiB), file-scope device arrays that a GPU holds from
+ * the first such context's initialisation until the process exits. */
 int lb_workspace_size(lb_ctx* ctx, size_t* bytes);
 int lb_bind_workspace(lb_ctx* ctx, void* device_ptr, size_t bytes);
 

@@ -265,7 +265,7 @@ class BatchT final : public Batch {
   }
 
   BatchT(const std::vector<Config>& cfgs, const std::vector<std::vector<double>>& x0) : x0_(x0) {
-    for (const Config& c : cfgs) eng_.emplace_back(new EngineT<S, R, DEV>(c, /*own_tables=*/false));
+    for (const Config& c : cfgs) eng_.emplace_back(new EngineT<S, R, DEV>(c));
     size_t off = 0;
     for (auto& e : eng_) {
       off = align_up(off, 256);
@@ -281,9 +281,6 @@ class BatchT final : public Batch {
     off = align_up(off, 256);
     counters_off_ = off;
     off += 2 * (cfgs.size() / kBatchGroup + 1) * sizeof(unsigned long long);
-    off = align_up(off, 256);
-    noise_off_ = off;
-    if (sizeof(R) == 8) off += noise_table_bytes();
     off = align_up(off, 256);
     table_off_ = off;
     off += cfgs.size() * sizeof(ReplicaK<S, R>);
@@ -302,10 +299,7 @@ class BatchT final : public Batch {
 
   void bind(void* base) override {
     base_ = static_cast<unsigned char*>(base);
-    for (size_t r = 0; r < eng_.size(); ++r) {
-      eng_[r]->bind(base_ + offs_[r]);
-      if (sizeof(R) == 8) eng_[r]->set_noise_tables(base_ + noise_off_);  // one for all replicas
-    }
+    for (size_t r = 0; r < eng_.size(); ++r) eng_[r]->bind(base_ + offs_[r]);
     d_reps_ = reinterpret_cast<ReplicaK<S, R>*>(base_ + table_off_);
     flags_[0] = reinterpret_cast<unsigned*>(base_ + flags_off_);
     flags_[1] = flags_[0] + max_segs_;
@@ -322,7 +316,10 @@ class BatchT final : public Batch {
       page_ = new_host_page(longest);
       for (auto& e : eng_) e->set_host_page(page_);
     }
-    if (sizeof(R) == 8) launch_fill_noise_tables(base_ + noise_off_, s);
+    if (sizeof(R) == 8) {
+      const NoiseTab tab = noise_tables();
+      for (auto& e : eng_) e->set_noise_tables(tab);
+    }
     for (size_t r = 0; r < eng_.size(); ++r)
       eng_[r]->initialise(x0_[r].empty() ? nullptr : x0_[r].data(), nullptr, s);
     smem_ = 0;
@@ -625,7 +622,7 @@ class BatchT final : public Batch {
   std::vector<BatchLB<S, R>> groups_;
   std::vector<std::vector<double>> x0_;
   std::vector<size_t> offs_;
-  size_t noise_off_ = 0, table_off_ = 0, step_off_ = 0, flags_off_ = 0, counters_off_ = 0, bytes_ = 0, smem_ = 0;
+  size_t table_off_ = 0, step_off_ = 0, flags_off_ = 0, counters_off_ = 0, bytes_ = 0, smem_ = 0;
   unsigned long long* counters_ = nullptr;
   size_t max_segs_ = 0;
   unsigned* flags_[2] = {nullptr, nullptr};  // node marks by slot

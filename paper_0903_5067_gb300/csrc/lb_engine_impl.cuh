@@ -9,22 +9,11 @@
 #include "lb_adjoint.cuh"
 #include "lb_device.cuh"
 #include "lb_engine.h"
+#include "lb_noise.h"
 
 namespace gblb {
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-
-// the noise tables of the FP64 kernels (NoiseTab) in one region: radii, then angles
-inline size_t noise_table_bytes() { return kRadii * sizeof(double) + kAngles * sizeof(double2); }
-inline NoiseTab noise_tables_at(void* base) {
-  double* radius = static_cast<double*>(base);
-  return NoiseTab{radius, reinterpret_cast<const double2*>(radius + kRadii)};
-}
-inline void launch_fill_noise_tables(void* base, cudaStream_t s) {
-  double* radius = static_cast<double*>(base);
-  fill_noise_tables<<<1216, 256, 0, s>>>(radius, reinterpret_cast<double2*>(radius + kRadii));
-  cuda_check(cudaGetLastError(), "noise tables");
-}
 
 // A page of page-locked host memory that the device writes read-backs into
 struct HostPage {
@@ -44,8 +33,7 @@ inline HostPage* new_host_page(int N) {  // null when there is none to be had
 template <class S, class R, bool DEV>
 class EngineT final : public Engine {
  public:
-  // own_tables: the FP64 noise tables are part of this engine's workspace (else set_noise_tables)
-  explicit EngineT(const Config& c, bool own_tables = true) : cfg_(c), own_tables_(own_tables && sizeof(R) == 8) {
+  explicit EngineT(const Config& c) : cfg_(c) {
     L_ = c.L;
     nnodes_ = (unsigned long long)L_ * L_ * L_;
     plane_ = align_up(nnodes_, 64);
@@ -67,7 +55,7 @@ class EngineT final : public Engine {
     drop_graphs();
     cfg_ = c;
   }
-  void set_noise_tables(void* base) { noise_tab_ = base; }
+  void set_noise_tables(const NoiseTab& t) { noise_tab_ = t; }  // of the owner's engines, looked up once
   void set_host_page(HostPage* p) { page_ = p; }  // of the owner's, for at least this many beads
 
   void initialise(const double* x0, const double* v0, cudaStream_t s) override {
@@ -80,7 +68,7 @@ class EngineT final : public Engine {
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q.stage_bytes),
                      "LB kernel shared memory");
     }
-    if (own_tables_) launch_fill_noise_tables(noise_tab_, s);
+    if (sizeof(R) == 8 && !noise_tab_.radius) noise_tab_ = noise_tables();
     if (bead_smem() > 48 * 1024)
       cuda_check(cudaFuncSetAttribute(bead_kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bead_smem()),
                  "bead kernel shared memory");
@@ -1212,7 +1200,7 @@ class EngineT final : public Engine {
     P.body_on = (body[0] != 0 || body[1] != 0 || body[2] != 0) ? 1 : 0;
     for (int q = 0; q < 3; ++q) P.body_dJ[q] = (R)(body[q] * c.h * c.h / c.a);
     P.nonpos = nonpos_;
-    if (noise_tab_) P.tab = noise_tables_at(noise_tab_);
+    P.tab = noise_tab_;
     return P;
   }
 
@@ -1336,7 +1324,6 @@ class EngineT final : public Engine {
     acc_ = reinterpret_cast<double*>(take(4 * sizeof(double)));
     obs_ = reinterpret_cast<double*>(take(kNObs * sizeof(double)));
     parts_ = reinterpret_cast<double*>(take(4 * (size_t)nparts_ * sizeof(double)));
-    if (own_tables_) noise_tab_ = take(noise_table_bytes());
     bytes_ = align_up(off, 256);
   }
 
@@ -1344,8 +1331,7 @@ class EngineT final : public Engine {
   HostPage* page_ = nullptr;
   bool own_page_ = false;
   int bead_reads_ = 0;
-  bool own_tables_ = false;
-  void* noise_tab_ = nullptr;
+  NoiseTab noise_tab_{nullptr, nullptr};  // double precision
   int L_ = 0, N_ = 0, cap_ = 8, nparts_ = 0, nsub_ = 1;
   unsigned long long nnodes_ = 0, plane_ = 0;
   size_t bytes_ = 0;

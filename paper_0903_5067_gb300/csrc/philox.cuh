@@ -183,7 +183,7 @@ __device__ __forceinline__ void fluid_pair(uint32_t w, const NoiseScale<float>& 
   if (SECOND) g1 = r * approx_sin(th);
 }
 // Double precision: every factor of a pair is one of 2^21 radii and one of 2048 angles, so both are
-// read from tables in global memory (fill_noise_tables) instead of computed: the radius table
+// read from tables in global memory (noise_tables) instead of computed: the radius table
 // (16 MiB) stays in the L2 cache, the angle table (32 KiB) in the L1 cache.  A logarithm and a
 // square root cost about 40 FP64 instructions, each of which holds an SM's FP64 pipe for 16
 // clocks; a lookup costs one load.
@@ -192,16 +192,6 @@ struct NoiseTab {
   const double2* angle;  // (cos, sin)(2 pi (u1 - 1/2)), u1 = (k + 1/2) 2^-11, k < 2048
 };
 constexpr unsigned kRadii = 1u << 21, kAngles = 1u << 11;
-static __global__ void fill_noise_tables(double* radius, double2* angle) {
-  for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < kRadii; k += gridDim.x * blockDim.x) {
-    radius[k] = sqrt(-2.0 * log(((double)k + 0.5) * 0x1p-21));
-    if (k < kAngles) {
-      double s, c;
-      sincospi(2.0 * (((double)k + 0.5) * 0x1p-11) - 1.0, &s, &c);
-      angle[k] = make_double2(c, s);
-    }
-  }
-}
 template <bool SECOND>
 __device__ __forceinline__ void fluid_pair(uint32_t w, const NoiseScale<double>& ns, double& g0, double& g1,
                                            const NoiseTab& tab) {
