@@ -33,9 +33,10 @@ L_BENCH, N_BENCH, SEED = 128, 128, 3
 PARAMS = dict(rho=1.0, eta=3.0, eta_b=3.0, kT=1.0, h=0.01, a=1.0)
 CHAIN = dict(m=1.0, zeta=20.8, k_fene=30.0, R0=1.5, eps=1.0, sigma=1.0)
 BYTES_PER_NODE = {"f32": 19 * 4 * 2, "f64": 19 * 8 * 2, "bf16": 19 * 2 * 2}  # algorithmic: 19 reads + 19 writes
-# FP64 operations per node update of the plain FP64 kernel with noise (ncu op counts at L = 128:
-# (DADD + DMUL + 2 DFMA) / nodes = 2.223e9 / 2,097,152); that kernel is bound by FP64 arithmetic
-FP64_FLOPS_PER_NODE = 797
+# FP64 operations per node update of the plain FP64 kernel with noise (ncu op counts at L = 72:
+# (DADD + DMUL + 2 DFMA) / nodes = (48.149e6 + 17.916e6 + 2 x 14.183e6) / 373,248); that kernel is
+# bound by the FP64 pipe, of which an addition takes as much as a multiply-add
+FP64_FLOPS_PER_NODE = 253
 # GB300's dense FP64 rate: 152 SMs x 2 FP64 FMA per SM and clock x 2 flops x 2.07 GHz
 FP64_PEAK_TFLOPS = 1.26
 KERNEL_SOURCES = ["paper_0903_5067_gb300/csrc/lb_device.cuh", "paper_0903_5067_gb300/csrc/d3q19.cuh",
