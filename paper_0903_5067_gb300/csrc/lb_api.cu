@@ -352,7 +352,8 @@ int lb_step(lb_ctx* ctx, int64_t n) {
     for (int64_t t = 0; t < n;) {
       // steps up to the next one that something follows: a sample, a frame, a timing event
       int64_t m = n - t;
-      auto until = [&](int64_t done, int64_t stride) { m = std::min(m, stride - done % stride); };
+      // (a frame's count is negative where a state from before the recording's start was loaded)
+      auto until = [&](int64_t done, int64_t stride) { m = std::min(m, stride - (done % stride + stride) % stride); };
       const bool sample = ctx->obs_stride > 0 && ctx->cfg.N > 0;
       if (sample) until(ctx->step, ctx->obs_stride);
       if (ctx->traj) until(ctx->step - ctx->traj_origin, ctx->traj_stride);

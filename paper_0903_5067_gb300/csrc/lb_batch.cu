@@ -423,7 +423,8 @@ class BatchT final : public Batch {
   // while the bead kernels have the chip to themselves, a block per SM (8 replicas of L = 15,
   // N = 32, two substeps: 27.6, 18.8, 15.5 and 12.9 us per step on 1, 2, 4 and 8 blocks; 64 of them:
   // 32.5, 23.3, 23.8 and 31.2); where the LB kernel sets the step they only take its place (64
-  // replicas, 5.2 M nodes: 131.6, 132.2 and 134.6 us on 1, 2 and 4).
+  // replicas, 5.2 M nodes: 131.6, 132.2 and 134.6 us on 1, 2 and 4).  All with bead blocks and
+  // tiles of 256 threads.
   int bead_cluster() const {
     unsigned long long nodes = 0;
     int longest = 1;

@@ -719,7 +719,7 @@ __device__ __noinline__ void stage_marked_call(const float* __restrict__ corr, u
 // nodes of a row, and a kernel whose blocks are all resident ends with its slowest warp: with
 // every marked thread staging its own nodes one after the other, 19 rounds and one flight each,
 // the step at L = 64, N = 64 (FP32) took 11.4 us, of which 3.2 went with the corrections left out;
-// now 8.6 (7.4 without a chain).
+// then 8.6 (7.4 without a chain); 7.8 with blocks of 128 threads (7.15).
 template <class R, bool PAIR>
 __device__ __forceinline__ void add_corrections(const R* __restrict__ corr, unsigned long long plane, unsigned L,
                                                 unsigned node, unsigned mw, unsigned part, unsigned char* smem,
