@@ -655,7 +655,11 @@ extern "C" {
 
 int lb_analysis_msd(const double* traj, int T, int N, int max_lag, int i0, int i1, double* out, void* stream) {
   if (!traj || !out || T < 1 || N < 1 || max_lag < 0 || i0 < 0 || i1 < 0 || i0 >= N || i1 >= N) return LB_ERR_ARG;
-  if (T <= kMsdFrames) {
+  // Short chains and few lags leave the staged form's exchange of series with nothing to save (us, with the
+  // host's share, staged and plain: T = 200, N = 8, 51 lags 72, 65; T = 1000, N = 8, 61 lags 105, 93;
+  // T = 400, N = 16, 151 lags 86, 80; T = 400, N = 32, 61 lags 78, 101; T = 1000, N = 8, 501 lags 156, 180).
+  const bool plain = (long long)T * (N - 12) <= 4000 && max_lag < 304;
+  if (T <= kMsdFrames && !plain) {
     // as many clusters as fit the chip with one block per SM (15 of 8), no more than the lags need
     int nc = (max_lag + kMsdCluster) / kMsdCluster;
     nc = nc < 15 ? nc : 15;
@@ -682,7 +686,11 @@ int lb_analysis_rouse_modes(const double* traj, int T, int N, int P, double* X, 
 
 int lb_analysis_rouse_correlation(const double* X, int T, int P, int max_lag, double* c, void* stream) {
   if (!X || !c || T < 1 || P < 1 || max_lag < 0 || max_lag > 65535) return LB_ERR_ARG;
-  if (T <= kCorrFrames) {
+  // A block of the staged form takes kCorrLags lags: on less than half of the SMs the form with a block
+  // per lag is as fast or faster (us, with the host's share, staged and plain: T = 1000, P = 7, 61 lags
+  // (7 blocks) 104, 58; T = 531, P = 14, 261 lags (70) 81, 83; T = 300, P = 127, 61 lags (127) 72, 107).
+  const bool few = (long long)P * ((max_lag + kCorrLags) / kCorrLags) < 76;
+  if (T <= kCorrFrames && !few) {
     const size_t smem = 3 * (size_t)T * sizeof(double);
     if (!allow_shared(k_rouse_corr_staged, smem)) return LB_ERR_CUDA;
     k_rouse_corr_staged<<<dim3(P, (max_lag + kCorrLags) / kCorrLags), kThreads, smem, (cudaStream_t)stream>>>(
