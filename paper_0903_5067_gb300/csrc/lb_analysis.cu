@@ -243,9 +243,9 @@ __global__ void __launch_bounds__(kThreads) k_rouse_modes(const double* __restri
     const int f = e / (3 * H), r = e - f * 3 * H, n = r / 3, q = r - 3 * n;
     const double* fr = traj + (size_t)(t0 + f) * N * 3;
     const double lo = fr[r], hi = fr[3 * (N - 1 - n) + q];
-    const bool mid = 2 * n + 1 == N;
-    sd[(2 * f) * 3 * H + r] = mid ? lo : lo + hi;
-    sd[(2 * f + 1) * 3 * H + r] = mid ? 0.0 : lo - hi;
+    // the middle bead is its own partner: its difference is 0, or NaN where it is not finite
+    sd[(2 * f) * 3 * H + r] = 2 * n + 1 == N ? lo : lo + hi;
+    sd[(2 * f + 1) * 3 * H + r] = lo - hi;
   }
   __syncthreads();
   for (int e = threadIdx.x; e < nf * P; e += kThreads) {
