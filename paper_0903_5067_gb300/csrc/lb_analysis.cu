@@ -537,8 +537,9 @@ __global__ void __launch_bounds__(kThreads) k_static_sk(const double* __restrict
 #pragma unroll
     for (int g = 0; g < KG; ++g)
       if (g0 + g < nk) {
-        // the N diagonal terms of every frame and each pair twice, over N T
-        const double pairs = w.k[g] == 0.0 ? 0.25 * (double)N * (N - 1) * T : acc[g] / w.k[g];
+        // the N diagonal terms of every frame and each pair twice, over N T; at k = 0 a sum of 0, or
+        // NaN where a distance is not finite
+        const double pairs = w.k[g] == 0.0 ? 0.25 * (double)N * (N - 1) * T + acc[g] : acc[g] / w.k[g];
         atomicAdd(S + g0 + g, (half ? 0.0 : 1.0) + 2.0 * pairs / ((double)N * T));
       }
   }
@@ -576,7 +577,7 @@ __global__ void __launch_bounds__(kThreads) k_dynamic_sk(const double* __restric
 #pragma unroll
     for (int g = 0; g < KG; ++g)
       if (g0 + g < nk) {
-        const double pairs = w.k[g] == 0.0 ? (double)nn * norig : acc[g] / w.k[g];
+        const double pairs = w.k[g] == 0.0 ? (double)nn * norig + acc[g] : acc[g] / w.k[g];  // (as above)
         S[(size_t)(g0 + g) * nlag + lag] = norig > 0 ? pairs / ((double)N * norig) : 0.0;
       }
   }

@@ -32,3 +32,13 @@ def test_rouse_modes(lblib, N, place):
     n = {"first": 0, "middle": N // 2, "last": N - 1}[place]
     t, traj = _frames(6, N, N, (2, n, 1))
     _same(an.rouse_modes(traj).cpu().numpy(), ob.rouse_modes(t))
+
+
+@pytest.mark.parametrize("ks", [[0.0], [0.0, 0.7, 1.3], [0.9, 1.1]])
+def test_structure_factors(lblib, ks):
+    from paper_0903_5067_gb300 import analysis as an
+
+    t, traj = _frames(4, 5, 11, (3, 1, 2))
+    _same(an.static_sk(traj, ks), ob.static_structure_factor(t, ks))
+    _same(an.dynamic_sk(traj, ks, 3, origin_stride=3), ob.dynamic_structure_factor(t, ks, 3, origin_stride=3))
+    assert np.isnan(an.inverse_radius(traj))
