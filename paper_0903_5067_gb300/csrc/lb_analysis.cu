@@ -13,6 +13,7 @@
 #include <stdint.h>
 
 #include "../../include/lb.h"
+#include "lb_shared.h"
 
 namespace {
 
@@ -608,7 +609,7 @@ constexpr ClusterFit kClusterFit[] = {{16, 7}, {10, 13}, {9, 15}, {6, 23}, {4, 3
 template <class K>
 bool allow_shared(K* kernel, size_t bytes) {
   if (bytes <= 40 * 1024) return true;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess) return true;
+  if (gblb::allow_all_shared((const void*)kernel) == cudaSuccess) return true;
   cudaGetLastError();
   return false;
 }

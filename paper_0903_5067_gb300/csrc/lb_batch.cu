@@ -326,10 +326,8 @@ class BatchT final : public Batch {
     for (auto& e : eng_)
       if (e->chain_length() > 0 && e->bead_smem_bytes(e->sorted_beads() ? 1 : bead_g_) > smem_)
         smem_ = e->bead_smem_bytes(e->sorted_beads() ? 1 : bead_g_);
-    if (smem_ > 48 * 1024)
-      cuda_check(cudaFuncSetAttribute(k_batch_bead<S, R, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem_),
-                 "batch bead shared memory");
+    // (its static part counts towards the 48 KB that need no asking)
+    cuda_check(allow_all_shared((const void*)k_batch_bead<S, R, DEV>), "batch bead shared memory");
     cap_max_ = 8;
     for (auto& e : eng_) cap_max_ = e->pending_capacity() > cap_max_ ? e->pending_capacity() : cap_max_;
     // the engines zeroed their pending counts; no node is marked

@@ -22,6 +22,7 @@
 #include "../../include/lb.h"
 #include "d3q19.cuh"
 #include "lb_engine.h"
+#include "lb_shared.h"
 #include "philox.cuh"
 
 namespace gblb {
@@ -601,8 +602,7 @@ class BDT final : public BDBase {
       else if (P.N <= 64) use_registers<8>();
     }
     if (smem_ > 48 * 1024)
-      cuda_check(cudaFuncSetAttribute(kernel_, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_),
-                 "BD shared memory");
+      cuda_check(allow_all_shared((const void*)kernel_), "BD shared memory");
   }
   ~BDT() override {
     cudaFree(P_.x);

@@ -10,6 +10,7 @@
 #include "lb_device.cuh"
 #include "lb_engine.h"
 #include "lb_noise.h"
+#include "lb_shared.h"
 
 namespace gblb {
 
@@ -70,8 +71,7 @@ class EngineT final : public Engine {
     }
     if (sizeof(R) == 8 && !noise_tab_.radius) noise_tab_ = noise_tables();
     if (bead_smem() > 48 * 1024)
-      cuda_check(cudaFuncSetAttribute(bead_kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bead_smem()),
-                 "bead kernel shared memory");
+      cuda_check(allow_all_shared((const void*)bead_kernel()), "bead kernel shared memory");
     const unsigned long long nb = (nnodes_ + 255) / 256;
     k_init_rest<S, R, DEV><<<(unsigned)nb, 256, 0, s>>>(pop_[0], nnodes_, plane_, (R)cfg_.rho);
     cuda_check(cudaGetLastError(), "init populations");
@@ -391,11 +391,9 @@ class EngineT final : public Engine {
     const ChainK<R> C = chain();
     const size_t smem = scratch_in_smem ? prep_bytes + adj_scratch : 0, prep_smem = adj_prep_smem<R>(N_);
     if (smem > 48 * 1024)
-      cuda_check(cudaFuncSetAttribute(k_adj_bead<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                 "adjoint smem");
+      cuda_check(allow_all_shared((const void*)k_adj_bead<R>), "adjoint smem");
     if (prep_smem > 48 * 1024)
-      cuda_check(cudaFuncSetAttribute(k_adj_prep<S, R, DEV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prep_smem),
-                 "adjoint smem");
+      cuda_check(allow_all_shared((const void*)k_adj_prep<S, R, DEV>), "adjoint smem");
     dim3 blk, grd;
     lb_launch_shape(blk, grd);
     int cur_lam = 0;
