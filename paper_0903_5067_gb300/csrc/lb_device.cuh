@@ -1436,10 +1436,15 @@ __device__ __forceinline__ void bead_step_block(const S* __restrict__ pop, const
       M.cell[poff + t] = c;
       M.fr[t] = over_a(fma(-f, C.a, hi) + lo, C);
     }
-    // every block has started and read the state, once all have arrived: waited for before the
-    // first remote store and the first write of the state (its reads have returned)
-    if (G > 1 && sub == 0) cluster_arrive_relaxed();
     __syncthreads();
+    // every block has started and read the state, once all have arrived: waited for before the
+    // first remote store and the first write of the state.  The last warp's arrival is a release
+    // (with the block's barrier before it for the reads of all its warps); it has the time: 10.05 us
+    // per step at L = 25, N = 32, two substeps, as with none, 10.33 with the first warp's, which gathers.
+    if (G > 1 && sub == 0) {
+      if (warp == nwarp - 1) cluster_arrive();
+      else cluster_arrive_relaxed();
+    }
     // 2. post-stream density and momentum at the corner nodes of the block's beads ...
     const int gw = (nc + 31) >> 5;            // warps that gather
     const int g0 = gw < nwarp ? 32 * gw : 0;  // the other threads (all, when none is left over)
@@ -1520,7 +1525,7 @@ __device__ __forceinline__ void bead_step_block(const S* __restrict__ pop, const
         }
       }
     }
-    if (G > 1) {  // forces sent, old lists cleared
+    if (G > 1) {  // forces sent, old lists cleared (and, before the block's barrier, a substep's start read)
       if (__any_sync(0xffffffffu, wrote)) cluster_arrive();
       else cluster_arrive_relaxed();
     }
