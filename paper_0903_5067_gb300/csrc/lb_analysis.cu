@@ -421,11 +421,12 @@ __device__ __forceinline__ bool rsqrt_range(double x) {  // also false for NaN a
 constexpr int kKGroup = 4;           // most wave numbers of one pass over the pairs
 constexpr double kFastArg = 1.0e6;   // largest k r of the table path
 
-// sin(k r)/(k r) as k times the sum needs it: sin(k r)/r, general arguments
-__device__ __noinline__ double sinc_general(double k, double r2) {
+// sin(k r)/(k r), and k times it (sin(k r)/r) as the sums of the table path need it; general arguments
+__device__ __forceinline__ double sinc(double k, double r2) {
   const double x = k * sqrt(r2);
-  return x == 0.0 ? k : sin(x) / x * k;
+  return x == 0.0 ? 1.0 : sin(x) / x;
 }
+__device__ __noinline__ double sinc_general(double k, double r2) { return sinc(k, r2) * k; }
 
 // Wave numbers g0 .. g0 + KG - 1 (the last group repeats the last one) and the squared distances
 // [2^-100, r2_end) that take the table path for all of them, as a span of high words: compared
@@ -507,32 +508,70 @@ __device__ __forceinline__ double pair_r2(const double* __restrict__ f, int N, u
   return fma(dx, dx, fma(dy, dy, dz * dz));
 }
 
-// Walk the pairs of all frames, thread by thread of the two clusters `half` = 0, 1: f(r2) for each.
-template <class F>
-__device__ __forceinline__ void walk_pairs(const double* __restrict__ traj, int T, int N, unsigned half, F&& f) {
-  const unsigned np = (unsigned)N * (unsigned)(N - 1) / 2;
-  const unsigned nt = 2 * cluster_blocks() * blockDim.x;
-  unsigned q = (half * cluster_blocks() + cluster_rank()) * blockDim.x + threadIdx.x;
-  const double* fr = traj;
-  for (int t = 0; t < T; ++t, fr += 3 * (size_t)N) {
-    for (; q < np; q += nt) f(pair_r2(fr, N, q));
-    q -= np;  // the walk goes on in the next frame where it would have
+// Walk T frames of `per` pairs: the pairs at + m nt, m = 0, 1, ..., of all frames one after the other:
+// f(frame, pair in the frame) for each.  Where a frame has fewer pairs than there are threads, a thread
+// steps over dt whole frames and dq pairs at a time, so that all have a pair in every turn (a loop over
+// the frames with one over a frame's pairs in it runs the threads of a warp one after the other there:
+// S(k) of 16 wave numbers at T = 1000, N = 2 302 us, now 10); else that loop, whose turns cost
+// less (S(k) of 4 at N = 128: 2.92 ms, 3.06 without it).  FEW: the former alone.
+template <bool FEW, class F>
+__device__ __forceinline__ void walk_frames(int T, unsigned per, unsigned nt, unsigned at, F&& f) {
+  if (!FEW && per >= nt) {
+    unsigned q = at;
+    for (int t = 0; t < T; ++t) {
+      for (; q < per; q += nt) f(t, q);
+      q -= per;  // the walk goes on in the next frame where it would have
+    }
+  } else if (per > 0) {
+    const unsigned dt = nt / per, dq = nt % per;
+    unsigned t = at / per, q = at % per;
+    while (t < (unsigned)T) {
+      f((int)t, q);
+      t += dt;
+      q += dq;
+      if (q >= per) {
+        q -= per;
+        ++t;
+      }
+    }
   }
 }
 
-// Two clusters per group of KG wave numbers; S zeroed
+// The pairs i < j of all frames by the nt threads of which this is number `at`: f(r2) for each
+template <bool FEW, class F>
+__device__ __forceinline__ void walk_pairs(const double* __restrict__ traj, int T, int N, unsigned nt, unsigned at, F&& f) {
+  walk_frames<FEW>(T, (unsigned)N * (unsigned)(N - 1) / 2, nt, at,
+                   [&](int t, unsigned q) { f(pair_r2(traj + 3 * (size_t)N * t, N, q)); });
+}
+// The ordered pairs (i, j) at the origins 0, s, 2s, ... of which a later frame exists
+template <bool FEW, class F>
+__device__ __forceinline__ void walk_origins(const double* __restrict__ traj, int norig, int N, int stride, int lag,
+                                             unsigned nt, unsigned at, F&& f) {
+  walk_frames<FEW>(norig, (unsigned)N * (unsigned)N, nt, at, [&](int o, unsigned q) {
+    const double* fa = traj + 3 * (size_t)N * ((size_t)o * (unsigned)stride);
+    const double* fb = fa + 3 * (size_t)N * (unsigned)lag;
+    const unsigned i = q / (unsigned)N, j = q % (unsigned)N;
+    const double dx = fb[3 * i] - fa[3 * j], dy = fb[3 * i + 1] - fa[3 * j + 1], dz = fb[3 * i + 2] - fa[3 * j + 2];
+    f(fma(dx, dx, fma(dy, dy, dz * dz)));
+  });
+}
+__device__ __forceinline__ int origins(int T, int lag, int stride) { return T - lag > 0 ? (T - lag + stride - 1) / stride : 0; }
+
+// `parts` clusters per group of KG wave numbers; two add their sums to S, zeroed
 template <int KG>
 __global__ void __launch_bounds__(kThreads) k_static_sk(const double* __restrict__ traj, int T, int N,
-                                                        const double* __restrict__ ks, int nk, double* __restrict__ S) {
+                                                        const double* __restrict__ ks, int nk, double* __restrict__ S,
+                                                        int parts) {
   __shared__ SinTab tab;
   __shared__ double2 seed[48];
   __shared__ double ws[KG * 32], bs[KG];
   fill_sin_table(&tab, seed);
-  const unsigned half = blockIdx.x / cluster_blocks() & 1;
-  const int g0 = (int)(blockIdx.x / cluster_blocks() / 2) * KG;
+  const unsigned cluster = blockIdx.x / cluster_blocks(), part = cluster % (unsigned)parts;
+  const int g0 = (int)(cluster / (unsigned)parts) * KG;
   const WaveNumbers<KG> w(ks, nk, g0);
   double acc[KG] = {};
-  walk_pairs(traj, T, N, half, [&](double r2) { add_pair<KG>(r2, w, &tab, acc); });
+  walk_pairs<false>(traj, T, N, parts * cluster_blocks() * kThreads, (part * cluster_blocks() + cluster_rank()) * kThreads + threadIdx.x,
+             [&](double r2) { add_pair<KG>(r2, w, &tab, acc); });
   cluster_sum<KG>(acc, ws, bs);
   if (cluster_rank() == 0 && threadIdx.x == 0) {
 #pragma unroll
@@ -540,10 +579,22 @@ __global__ void __launch_bounds__(kThreads) k_static_sk(const double* __restrict
       if (g0 + g < nk) {
         // the N diagonal terms of every frame and each pair twice, over N T; at k = 0 a sum of 0, or
         // NaN where a distance is not finite
-        const double pairs = w.k[g] == 0.0 ? 0.25 * (double)N * (N - 1) * T + acc[g] : acc[g] / w.k[g];
-        atomicAdd(S + g0 + g, (half ? 0.0 : 1.0) + 2.0 * pairs / ((double)N * T));
+        const double pairs = w.k[g] == 0.0 ? 0.5 / parts * (double)N * (N - 1) * T + acc[g] : acc[g] / w.k[g];
+        const double v = (part ? 0.0 : 1.0) + 2.0 * pairs / ((double)N * T);
+        if (parts == 1) S[g0 + g] = v;
+        else atomicAdd(S + g0 + g, v);
       }
   }
+}
+// Few pairs: one block per wave number, without a table
+__global__ void __launch_bounds__(kThreads) k_static_sk_few(const double* __restrict__ traj, int T, int N,
+                                                            const double* __restrict__ ks, double* __restrict__ S) {
+  __shared__ double sh[1][kThreads];
+  const double k = ks[blockIdx.x];
+  double v[1] = {0};
+  walk_pairs<true>(traj, T, N, kThreads, threadIdx.x, [&](double r2) { v[0] += sinc(k, r2); });
+  block_sum<1>(v, sh);
+  if (threadIdx.x == 0) S[blockIdx.x] = ((double)N * T + 2.0 * v[0]) / ((double)N * T);
 }
 
 // One cluster per lag (blockIdx.y) and group of KG wave numbers: all ordered pairs (i, j) at the
@@ -558,41 +609,47 @@ __global__ void __launch_bounds__(kThreads) k_dynamic_sk(const double* __restric
   fill_sin_table(&tab, seed);
   const int g0 = (int)(blockIdx.x / cluster_blocks()) * KG;
   const int lag = blockIdx.y;
-  const int norig = T - lag > 0 ? (T - lag + stride - 1) / stride : 0;
+  const int norig = origins(T, lag, stride);
   const WaveNumbers<KG> w(ks, nk, g0);
   double acc[KG] = {};
-  const unsigned nn = (unsigned)N * (unsigned)N, nt = cluster_blocks() * blockDim.x;
-  unsigned q = cluster_rank() * blockDim.x + threadIdx.x;
-  const double* fa = traj;
-  const double* fb = traj + (size_t)lag * N * 3;
-  for (int o = 0; o < norig; ++o, fa += 3 * (size_t)N * stride, fb += 3 * (size_t)N * stride) {
-    for (; q < nn; q += nt) {
-      const unsigned i = q / (unsigned)N, j = q % (unsigned)N;
-      const double dx = fb[3 * i] - fa[3 * j], dy = fb[3 * i + 1] - fa[3 * j + 1], dz = fb[3 * i + 2] - fa[3 * j + 2];
-      add_pair<KG>(fma(dx, dx, fma(dy, dy, dz * dz)), w, &tab, acc);
-    }
-    q -= nn;
-  }
+  walk_origins<false>(traj, norig, N, stride, lag, cluster_blocks() * kThreads, cluster_rank() * kThreads + threadIdx.x,
+               [&](double r2) { add_pair<KG>(r2, w, &tab, acc); });
   cluster_sum<KG>(acc, ws, bs);
   if (cluster_rank() == 0 && threadIdx.x == 0) {
 #pragma unroll
     for (int g = 0; g < KG; ++g)
       if (g0 + g < nk) {
-        const double pairs = w.k[g] == 0.0 ? (double)nn * norig + acc[g] : acc[g] / w.k[g];  // (as above)
+        const double pairs = w.k[g] == 0.0 ? (double)N * N * norig + acc[g] : acc[g] / w.k[g];  // (as above)
         S[(size_t)(g0 + g) * nlag + lag] = norig > 0 ? pairs / ((double)N * norig) : 0.0;
       }
   }
 }
+// Few pairs: one block per wave number and lag, without a table
+__global__ void __launch_bounds__(kThreads) k_dynamic_sk_few(const double* __restrict__ traj, int T, int N,
+                                                             const double* __restrict__ ks, int stride,
+                                                             double* __restrict__ S, int nlag) {
+  __shared__ double sh[1][kThreads];
+  const double k = ks[blockIdx.x];
+  const int lag = blockIdx.y, norig = origins(T, lag, stride);
+  double v[1] = {0};
+  walk_origins<true>(traj, norig, N, stride, lag, kThreads, threadIdx.x, [&](double r2) { v[0] += sinc(k, r2); });
+  block_sum<1>(v, sh);
+  if (threadIdx.x == 0) S[(size_t)blockIdx.x * nlag + lag] = norig > 0 ? v[0] / ((double)N * norig) : 0.0;
+}
 
-// two clusters: 1/r_ij over the pairs i < j of every frame; out zeroed
+// One block, or two clusters that add to `out`, zeroed: 1/r_ij over the pairs i < j of every frame
 __global__ void __launch_bounds__(2 * kThreads) k_inverse_radius(const double* __restrict__ traj, int T, int N,
                                                                  double* __restrict__ out) {
   __shared__ double ws[32], bs[1];
   double acc[1] = {0.0};
-  walk_pairs(traj, T, N, blockIdx.x / cluster_blocks(),
+  walk_pairs<false>(traj, T, N, gridDim.x * blockDim.x, blockIdx.x * blockDim.x + threadIdx.x,
              [&](double r2) { acc[0] += rsqrt_range(r2) ? rsqrt_pos(r2) : 1.0 / sqrt(r2); });
   cluster_sum<1>(acc, ws, bs);
-  if (cluster_rank() == 0 && threadIdx.x == 0) atomicAdd(out, 2.0 * acc[0] / ((double)N * N * T));
+  if (cluster_rank() == 0 && threadIdx.x == 0) {
+    const double v = 2.0 * acc[0] / ((double)N * N * T);
+    if (gridDim.x == 1) *out = v;
+    else atomicAdd(out, v);
+  }
 }
 
 constexpr size_t kMaxShared = 227 * 1024;  // dynamic and static shared memory of a block
@@ -601,11 +658,27 @@ constexpr size_t kMaxShared = 227 * 1024;  // dynamic and static shared memory o
 // with one block.
 constexpr size_t kOnePerSM = 116 * 1024;
 // Clusters of each size that fit the chip at one block per SM (cudaOccupancyMaxActiveClusters on a
-// GB300: 152 SMs, whose groups do not hold a whole number of larger clusters)
+// GB300: 152 SMs, whose groups do not hold a whole number of larger clusters), and how many of them
+// S(k) puts on a group of wave numbers
 struct ClusterFit {
-  int size, fit;
+  int parts, size, fit;
 };
-constexpr ClusterFit kClusterFit[] = {{16, 7}, {10, 13}, {9, 15}, {6, 23}, {4, 36}};
+constexpr ClusterFit kClusterFit[] = {{2, 16, 7}, {2, 10, 13}, {2, 9, 15}, {2, 6, 23}, {2, 4, 36},
+                                      {1, 8, 15}, {1, 4, 36},  {1, 2, 76}, {1, 1, 152}};
+// What a structure factor takes in us, for the choice between its forms.  A turn, in which each thread of
+// a block takes one pair, is bound by the FP64 pipe of the block's SM: 1 us for the distance and 1.08
+// for each sine by the table, 3.4 with the general sine.  A launch takes 4 us and a block's table and
+// cluster sum 2 to 4.4 (each wave of blocks).  Measured, S(k) of T frames of N beads, by a block per
+// wave number without a table and in groups of 1 and 3 on clusters of 4: T = 1, N = 32 (two turns of
+// a block) 10.5, 10.5, 16.7; T = 100, N = 32 (194) 604, 117, 222.  S(k, t) in groups of 1 on a
+// block, 2 on 2, 4 on 8 at T = 1000, N = 8, 100 lags: 55.6, 51.4, 68.4 (65.1 without a table; by this
+// 61, 52, 67 (69)).
+double us_by_table(double waves, int kg, int cs, double turns) {
+  return 4.0 + 0.25 * cs + waves * (2.0 + 0.6 * kg + (1 + 1.08 * kg) * fmax(1.0, turns));
+}
+double us_without_table(double blocks, double turns) { return 4.0 + 3.4 * ceil(blocks / 152) * fmax(1.0, turns); }
+constexpr double kClear = 0.85;  // a table has to be this much faster by these estimates, which are that rough
+
 template <class K>
 bool allow_shared(K* kernel, size_t bytes) {
   if (bytes <= 40 * 1024) return true;
@@ -705,37 +778,45 @@ int lb_analysis_rouse_correlation(const double* X, int T, int P, int max_lag, do
 
 int lb_analysis_static_sk(const double* traj, int T, int N, const double* k, int nk, double* S, void* stream) {
   if (!traj || !k || !S || T < 1 || N < 1 || nk < 1) return LB_ERR_ARG;
-  // A group of KG wave numbers runs on two clusters and a pair costs 1 + KG units there (its
-  // distance, and each sine): the KG and cluster size with the shortest time, all clusters in one
-  // wave where possible.  16 wave numbers: groups of 3 on 12 clusters of 10 (6.8 ms at T = 1000,
-  // N = 128; groups of 2 on 16 clusters of 8, two waves, 11.5 ms; one block per wave number 144 ms).
-  int kg = 1, cs = 1;
-  double best = 1e30;
+  // The group size and cluster with the shortest time, all clusters in one wave where possible.  16
+  // wave numbers: groups of 3 on 12 clusters of 10 (6.8 ms at T = 1000, N = 128; groups of 2 on 16
+  // clusters of 8, two waves, 11.5 ms; one block per wave number 144 ms).  Few pairs: a block per wave
+  // number without a table (a frame of 8 beads 6.2 us, with a table 10).
+  const double pairs = 0.5 * N * (N - 1.0) * T;
+  const cudaStream_t s = (cudaStream_t)stream;
+  double best = kClear * us_without_table(nk, pairs / kThreads);
+  int kg = 0;
+  ClusterFit c = {};
   for (int g = 1; g <= kKGroup; ++g)
     for (const ClusterFit& f : kClusterFit) {
-      const int clusters = 2 * ((nk + g - 1) / g), waves = (clusters + f.fit - 1) / f.fit;
-      const double t = (double)waves * (1 + g) / f.size;
+      const int clusters = f.parts * ((nk + g - 1) / g), waves = (clusters + f.fit - 1) / f.fit;
+      const double t = us_by_table(waves, g, f.size, ceil(pairs / (f.parts * f.size * kThreads))) + f.parts;
       if (t < best) {
         best = t;
         kg = g;
-        cs = f.size;
+        c = f;
       }
     }
-  cs = cluster_for((unsigned long long)N * (N - 1) / 4 * T, kThreads, cs);
-  const size_t apart = cs > 1 ? kOnePerSM : 0;
-  const dim3 grid((nk + kg - 1) / kg * 2 * cs);
-  const cudaStream_t s = (cudaStream_t)stream;
-  if (cudaMemsetAsync(S, 0, nk * sizeof(double), s) != cudaSuccess) return launch_status();
-  if (kg == 1) return launch_cluster(k_static_sk<1>, grid, kThreads, cs, apart, s, traj, T, N, k, nk, S);
-  if (kg == 2) return launch_cluster(k_static_sk<2>, grid, kThreads, cs, apart, s, traj, T, N, k, nk, S);
-  if (kg == 3) return launch_cluster(k_static_sk<3>, grid, kThreads, cs, apart, s, traj, T, N, k, nk, S);
-  return launch_cluster(k_static_sk<kKGroup>, grid, kThreads, cs, apart, s, traj, T, N, k, nk, S);
+  if (kg == 0) {
+    k_static_sk_few<<<nk, kThreads, 0, s>>>(traj, T, N, k, S);
+    return launch_status();
+  }
+  const size_t apart = c.size > 1 ? kOnePerSM : 0;
+  const dim3 grid((nk + kg - 1) / kg * c.parts * c.size);
+  if (c.parts > 1 && cudaMemsetAsync(S, 0, nk * sizeof(double), s) != cudaSuccess) return launch_status();
+  if (kg == 1) return launch_cluster(k_static_sk<1>, grid, kThreads, c.size, apart, s, traj, T, N, k, nk, S, c.parts);
+  if (kg == 2) return launch_cluster(k_static_sk<2>, grid, kThreads, c.size, apart, s, traj, T, N, k, nk, S, c.parts);
+  if (kg == 3) return launch_cluster(k_static_sk<3>, grid, kThreads, c.size, apart, s, traj, T, N, k, nk, S, c.parts);
+  return launch_cluster(k_static_sk<kKGroup>, grid, kThreads, c.size, apart, s, traj, T, N, k, nk, S, c.parts);
 }
 
 int lb_analysis_inverse_radius(const double* traj, int T, int N, double* out, void* stream) {
   if (!traj || !out || T < 1 || N < 2) return LB_ERR_ARG;
-  const int cs = cluster_for((unsigned long long)N * (N - 1) / 4 * T, 2 * kThreads, 16);
   const cudaStream_t s = (cudaStream_t)stream;
+  const unsigned long long pairs = (unsigned long long)N * (N - 1) / 2 * T;
+  if (pairs <= 2 * 2 * kThreads)  // two pairs of a thread take less than the zeroing
+    return launch_cluster(k_inverse_radius, dim3(1), 2 * kThreads, 1, 0, s, traj, T, N, out);
+  const int cs = cluster_for(pairs / 2, 2 * kThreads, 16);
   if (cudaMemsetAsync(out, 0, sizeof(double), s) != cudaSuccess) return launch_status();
   return launch_cluster(k_inverse_radius, dim3(2 * cs), 2 * kThreads, cs, 0, s, traj, T, N, out);
 }
@@ -744,12 +825,30 @@ int lb_analysis_dynamic_sk(const double* traj, int T, int N, const double* k, in
                            int origin_stride, double* S, void* stream) {
   if (!traj || !k || !S || T < 1 || N < 1 || nk < 1 || max_lag < 0 || max_lag > 65535 || origin_stride < 1)
     return LB_ERR_ARG;
-  const int cs = cluster_for((unsigned long long)N * N * ((T + origin_stride - 1) / origin_stride), kThreads, 8);
-  const dim3 grid((nk + kKGroup - 1) / kKGroup * cs, max_lag + 1);
+  // As for S(k); clusters of up to 8, of which several share an SM: one more wave than blocks fill
+  // (84 blocks take 1.5 to 1.7 times a turn, 404 3.6, 808 5.5)
+  const double pairs = (double)N * N * ((T + origin_stride - 1) / origin_stride), nlag = max_lag + 1.0;
   const cudaStream_t s = (cudaStream_t)stream;
-  if (nk == 1) return launch_cluster(k_dynamic_sk<1>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
-  if (nk == 2) return launch_cluster(k_dynamic_sk<2>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
-  if (nk == 3) return launch_cluster(k_dynamic_sk<3>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
+  double best = kClear * us_without_table(nk * nlag, pairs / kThreads);
+  int kg = 0, cs = 0;
+  for (int g = nk < kKGroup ? nk : kKGroup; g >= 1; --g)
+    for (int c = 8; c >= 1; c -= c > 4 ? 2 : 1) {
+      const double blocks = (nk + g - 1) / g * nlag * c, turns = pairs / (c * kThreads);
+      const double t = us_by_table(1.0 + blocks / 152, g, c, blocks <= 152 ? ceil(turns) : turns);
+      if (t < best) {
+        best = t;
+        kg = g;
+        cs = c;
+      }
+    }
+  if (kg == 0) {
+    k_dynamic_sk_few<<<dim3(nk, max_lag + 1), kThreads, 0, s>>>(traj, T, N, k, origin_stride, S, max_lag + 1);
+    return launch_status();
+  }
+  const dim3 grid((nk + kg - 1) / kg * cs, max_lag + 1);
+  if (kg == 1) return launch_cluster(k_dynamic_sk<1>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
+  if (kg == 2) return launch_cluster(k_dynamic_sk<2>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
+  if (kg == 3) return launch_cluster(k_dynamic_sk<3>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
   return launch_cluster(k_dynamic_sk<kKGroup>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
 }
 
