@@ -422,32 +422,46 @@ class BatchT final : public Batch {
   // N = 32, two substeps: 27.6, 18.8, 15.5 and 12.9 us per step on 1, 2, 4 and 8 blocks; 64 of them:
   // 32.5, 23.3, 23.8 and 31.2); where the LB kernel sets the step they only take its place (64
   // replicas, 5.2 M nodes: 131.6, 132.2 and 134.6 us on 1, 2 and 4).  All with bead blocks and
-  // tiles of 256 threads.
+  // tiles of 256 threads.  But a block with more than 64 places (beads at each substep) takes longer
+  // than the LB kernel does, beside which it slows down (FP32, N = 128, on 1 block of 384 threads and on 2:
+  // 64 replicas of L = 33 142, 96 us, 100 of L = 26 134, 90, 300 of L = 12, N = 64 with two substeps 122,
+  // 110), and a few large boxes have the room for 32 (3 of L = 100, N = 128, on 1, 2 and 4 blocks: 164, 76,
+  // 72; N = 64 on 1 and 2: 80, 71).  In FP64 the LB kernel leaves the time (100 of L = 12, N = 64 with two
+  // substeps on 1 and 2: 241, 274).
   int bead_cluster() const {
-    unsigned long long nodes = 0;
-    int longest = 1;
-    for (auto& e : eng_) {
-      nodes += e->nodes();
-      longest = std::max(longest, e->chain_length());
-    }
-    if (nodes > 2000000ull) return 1;
-    return std::max(1, std::min({8, (longest + 3) / 4, 152 / (int)eng_.size()}));
+    const int R_ = (int)eng_.size(), longest = longest_chain();
+    const int places = sizeof(R) == 4 ? longest * eng_[0]->config().substeps : 0;
+    const int needed = std::max(1, std::min(8, (places + 63) / 64));
+    if (total_nodes() > 2000000ull) return std::max(needed, std::min({8, (places + 31) / 32, 64 / R_}));
+    return std::max(needed, std::min({8, (longest + 3) / 4, 152 / R_}));
   }
 
   // Threads of a bead block (FP32): 384 where a block has more than 96 corners to gather, 256 where
   // the LB kernel sets the step or a block has less to do, so that more LB blocks fit beside it.  us
   // per step with 256 and 384: 64 replicas of L = 15, N = 32, two substeps (256 corners) 23.3 and
   // 21.4, 128 of them (512) 39.9 and 33.6, 32 (128) 18.2 and 16.2; 24 of L = 25 (96) 19.6 and 20.6; 64
-  // of L = 15, N = 16, one substep (64) 15.0 and 15.3.  FP64, bound by its pipe: 256.
+  // of L = 15, N = 16, one substep (64) 15.0 and 15.3.  Beside a long LB kernel only where a chain needs
+  // several blocks with more than 384 corners each and every block has an SM (64 of L = 50, N = 64,
+  // two substeps (512) 206 and 199; 160 of L = 25, N = 110 (440) 133 and 145).  FP64, bound by its
+  // pipe: 256.
   int bead_threads() const {
     if (sizeof(R) == 8) return 256;
-    unsigned long long nodes = 0;
-    int places = 0;  // beads of a block, each at every substep
-    for (auto& e : eng_) {
-      nodes += e->nodes();
-      places = std::max(places, e->config().substeps * ((e->chain_length() + bead_g_ - 1) / bead_g_));
-    }
-    return nodes <= 2000000ull && 8 * places > 96 ? 384 : 256;
+    int corners = 8 * eng_[0]->config().substeps * ((longest_chain() + bead_g_ - 1) / bead_g_);
+    for (auto& e : eng_)
+      if (e->sorted_beads()) corners = std::max(corners, 8 * e->config().substeps * e->chain_length());
+    if (total_nodes() > 2000000ull) return corners > 384 && bead_g_ > 1 && bead_g_ * eng_.size() <= 152 ? 384 : 256;
+    return corners > 96 ? 384 : 256;
+  }
+  unsigned long long total_nodes() const {
+    unsigned long long n = 0;
+    for (auto& e : eng_) n += e->nodes();
+    return n;
+  }
+  int longest_chain() const {  // of those that are not sorted, which take one block
+    int n = 1;
+    for (auto& e : eng_)
+      if (!e->sorted_beads()) n = std::max(n, e->chain_length());
+    return n;
   }
 
   void ensure_streams() {
