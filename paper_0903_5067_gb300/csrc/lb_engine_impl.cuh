@@ -915,7 +915,7 @@ class EngineT final : public Engine {
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof(lc));
     lc.gridDim = dim3((unsigned)G);
-    lc.blockDim = dim3(kBeadThreads);
+    lc.blockDim = dim3(bead_threads());
     lc.dynamicSmemBytes = bead_smem();
     lc.stream = s;
     cudaLaunchAttribute at[2];
@@ -1123,8 +1123,9 @@ class EngineT final : public Engine {
 
   // threads of a bead block: measured 11.0 against 10.6 us per step with 256 at L = 25, N = 32, two
   // substeps (FP32), 17.6 against 16.4 us with 512 at L = 16, N = 8 (FP64, whose pipe the additional
-  // warps do not help)
-  static constexpr int kBeadThreads = sizeof(R) == 8 ? 256 : 512;
+  // warps do not help); the sorted step, whose phases take several turns of the block,
+  // takes 608 us with 512 and 680 with 256 (FP64, L = 24, N = 200)
+  int bead_threads() const { return sizeof(R) == 8 && !bead_sorted() ? 256 : 512; }
   bool bead_sorted() const { return 8 * (size_t)N_ * nsub_ > (size_t)kGroupMax; }
   using BeadKernel = void (*)(const S*, const FluidK<R>, const ChainK<R>, const PendK<R>, const uint32_t);
   BeadKernel bead_kernel() const {

@@ -68,3 +68,8 @@ def yardstick(lblib):
 def test_batch(lblib, yardstick):
     """0.68 ms per step at 2.07 GHz; with the marks of the nodes set in a loop 0.75."""
     assert _ms(_batch(lblib, 1, 200)) / 48 <= 0.110 * yardstick
+
+
+def test_box(lblib, yardstick):
+    """0.61 ms per step at 2.07 GHz on blocks of 512 threads; 0.68 on 256."""
+    assert _ms(_box(lblib, 200)) / 48 <= 0.099 * yardstick
