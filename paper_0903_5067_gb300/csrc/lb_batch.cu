@@ -308,6 +308,7 @@ class BatchT final : public Batch {
   }
 
   void initialise(cudaStream_t s) override {
+    any_sorted_ = std::any_of(eng_.begin(), eng_.end(), [](auto& e) { return e->sorted_beads(); });
     bead_g_ = bead_cluster();
     bead_threads_ = bead_threads();
     if (!page_) {  // one page for the read-backs of all replicas
@@ -571,6 +572,9 @@ class BatchT final : public Batch {
   // a step's LB kernel, not one that writes the counter, which it reads before it waits) waits for
   // the previous step's last LB kernel, then releases the first LB kernel of its step, which runs
   // beside it and completes only after it (see k_batch_lb).  The force corrections stay pending.
+  // The bead kernel of chains that are sorted is an ordinary launch: launched early it finds room on SMs
+  // that still work, and what shares one with a block of hundreds of microseconds then slows it
+  // (FP64, 32 replicas of L = 24, N = 200: 783 us per step chained, 693 not; FP32, 16: 106.9, 107.4).
   void launch_step(cudaStream_t s, uint32_t j, bool chained) {
     const int par = eng_[0]->parity();
     const int R_ = (int)eng_.size();
@@ -589,7 +593,7 @@ class BatchT final : public Batch {
       at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
       at[1].val.programmaticStreamSerializationAllowed = 1;
       lc.attrs = at;
-      lc.numAttrs = chained ? 2 : 1;
+      lc.numAttrs = chained && !any_sorted_ ? 2 : 1;
       cuda_check(cudaLaunchKernelEx(&lc, k_batch_bead<S, R, DEV>, (const ReplicaK<S, R>*)d_reps_, par,
                                     (const uint32_t*)d_step_, j, counters_, (int)groups_.size(), bead_g_),
                  "batch bead");
@@ -644,6 +648,7 @@ class BatchT final : public Batch {
   uint32_t* d_step_ = nullptr;
   unsigned long long total_tiles_ = 0;
   int bead_g_ = 1, bead_threads_ = 256;
+  bool any_sorted_ = false;
   HostPage* page_ = nullptr;
   // Threads of a tile: small blocks end and begin more evenly (FP32, us per step with 128, 256, 512:
   // 64 replicas of L = 16 ... 64: 123.8, 127.1, 139.8; 16 of L = 32: 17.4, 17.8, 19.9; 64 of L = 15:

@@ -73,3 +73,8 @@ def test_batch(lblib, yardstick):
 def test_box(lblib, yardstick):
     """0.61 ms per step at 2.07 GHz on blocks of 512 threads; 0.68 on 256."""
     assert _ms(_box(lblib, 200)) / 48 <= 0.099 * yardstick
+
+
+def test_as_many_chains_as_there_is_room_for(lblib):
+    """A block per chain and many more SMs than chains: 32 take no longer than 2 (5 % are allowed)."""
+    assert _ms(_batch(lblib, 32, 200)) <= 1.05 * _ms(_batch(lblib, 2, 200))
