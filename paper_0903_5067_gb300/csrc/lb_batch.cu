@@ -318,7 +318,7 @@ class BatchT final : public Batch {
       for (auto& e : eng_) e->set_host_page(page_);
     }
     if (sizeof(R) == 8) {
-      const NoiseTab tab = noise_tables();
+      const NoiseTab tab = noise_tables(s);
       for (auto& e : eng_) e->set_noise_tables(tab);
     }
     for (size_t r = 0; r < eng_.size(); ++r)

@@ -69,7 +69,7 @@ class EngineT final : public Engine {
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q.stage_bytes),
                      "LB kernel shared memory");
     }
-    if (sizeof(R) == 8 && !noise_tab_.radius) noise_tab_ = noise_tables();
+    if (sizeof(R) == 8 && !noise_tab_.radius) noise_tab_ = noise_tables(s);
     if (bead_smem() > 48 * 1024)
       cuda_check(allow_all_shared((const void*)bead_kernel()), "bead kernel shared memory");
     const unsigned long long nb = (nnodes_ + 255) / 256;
