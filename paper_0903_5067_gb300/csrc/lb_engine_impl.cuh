@@ -170,14 +170,20 @@ class EngineT final : public Engine {
   // steps are captured once as a CUDA graph, whose kernels add their place in it to a device
   // counter, and replayed: 16 steps leave the buffers and correction slots as they found them, so
   // there is one graph per state of the two.  Capturing and instantiating one costs about as
-  // much as 30 launched steps: only calls of kGraphFirst steps start one.  A stream that is being
-  // captured gets the launches themselves.
+  // much as 30 launched steps: only calls of kGraphFirst steps start one, and where a step takes the GPU
+  // longer than its launches the host, kGraphSteps launched ones keep it busy meanwhile (L = 128, the
+  // first 64 steps: 3540 us without them, 3310 with no graphs at all, 3240 now).  A stream that is
+  // being captured gets the launches themselves.
   void steps_deferred(uint32_t k, int64_t n, cudaStream_t s) override {
     int64_t t = 0;
     if (n > kGraphSteps && graphs_usable(s)) {
       if (N_ > 0 && !open_) step_deferred(k + (uint32_t)t++, s, nullptr, nullptr);  // the first has nothing pending
       cudaGraphExec_t& g = graph_[cur_][pslot_];
-      if (!g && n >= kGraphFirst) g = capture_steps();
+      if (!g && n >= kGraphFirst) {
+        if (longer_than_launches())
+          for (int j = 0; j < kGraphSteps; ++j) step_deferred(k + (uint32_t)t++, s, nullptr, nullptr);
+        g = capture_steps();
+      }
       if (g) {
         for (int j = 0; j < 2; ++j)
           if (snap_pending_[j]) {  // the graph rewrites both snapshot slots
@@ -838,6 +844,11 @@ class EngineT final : public Engine {
 
   static constexpr int kGraphSteps = 16;  // even: buffers and slots alternate
   static constexpr int64_t kGraphFirst = 48;
+
+  // whether a step takes the GPU longer than the 17 us its launches take the host: by the nodes, 22 ps
+  // each in single precision (L = 96 20 us), 20 in 16-bit storage (L = 128 41) and 440 in FP64
+  // (L = 72 163)
+  bool longer_than_launches() const { return (double)nnodes_ * (sizeof(R) == 8 ? 440e-6 : (sizeof(S) == 4 ? 22e-6 : 20e-6)) > 17.0; }
 
   // whether work for s may go through a graph launch: not while s is being captured
   bool graphs_usable(cudaStream_t s) const {
