@@ -410,8 +410,8 @@ __global__ void __launch_bounds__(kBDThreads) k_bd_steps(const BDK<R> P, uint32_
   double* gx = P.x + (size_t)blockIdx.x * n;
   const uint32_t k1 = kTagBD | ((uint32_t)blockIdx.x << 8);
   for (int t = tid; t < n; t += nt) x[t] = (R)gx[t];
-  int lanes = 1;
-  while (lanes < 32 && lanes * 2 * N <= nt) lanes *= 2;
+  int lanes = 1;  // (more than N would add zeros: N = 2, free draining, FP64, 400 chains 21.6 us per step, now 17.7)
+  while (lanes < 32 && lanes < N && lanes * 2 * N <= nt) lanes *= 2;
   __syncthreads();
   for (int it = 0; it < nsteps; ++it) {
     const uint32_t step = step0 + (uint32_t)it;
