@@ -13,6 +13,7 @@
 #include <stdint.h>
 
 #include "../../include/lb.h"
+#include "lb_cluster.h"
 #include "lb_shared.h"
 
 namespace {
@@ -687,28 +688,36 @@ bool allow_shared(K* kernel, size_t bytes) {
   return false;
 }
 
-// a launch of `grid` blocks in clusters of cs along x
+int status_of(cudaError_t e) {
+  return e == cudaSuccess ? LB_OK : (e == cudaErrorMemoryAllocation ? LB_ERR_OOM : LB_ERR_CUDA);
+}
+
+// a launch of grid.x clusters of cs blocks along x (smaller ones where those have no place), grid.y of
+// them along y
 template <class... A, class... B>
 int launch_cluster(void (*kernel)(A...), dim3 grid, int threads, int cs, size_t smem, cudaStream_t s, B... args) {
   if (!allow_shared(kernel, smem)) return LB_ERR_CUDA;
-  if (cs > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-    cudaGetLastError();
-    return LB_ERR_CUDA;
-  }
-  cudaLaunchConfig_t lc = {};
-  lc.gridDim = grid;
-  lc.blockDim = dim3(threads);
-  lc.dynamicSmemBytes = smem;
-  lc.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)cs;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  lc.attrs = at;
-  lc.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&lc, kernel, (A)args...);
-  return e == cudaSuccess ? LB_OK : (e == cudaErrorMemoryAllocation ? LB_ERR_OOM : LB_ERR_CUDA);
+  return status_of(gblb::launch_in_clusters(cs, [&](int size) {
+    cudaError_t e = cudaSuccess;
+    if (size > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) {
+      cudaLaunchConfig_t lc = {};
+      lc.gridDim = dim3(grid.x * size, grid.y);
+      lc.blockDim = dim3(threads);
+      lc.dynamicSmemBytes = smem;
+      lc.stream = s;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)size;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      lc.attrs = at;
+      lc.numAttrs = 1;
+      e = cudaLaunchKernelEx(&lc, kernel, (A)args...);
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+  }));
 }
 
 // Blocks per cluster for `items` pairs per cluster, at most `most`: no more than leave each thread
@@ -719,9 +728,7 @@ int cluster_for(unsigned long long items, int threads, int most) {
 }
 
 int launch_status() {
-  const cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) return LB_OK;
-  return e == cudaErrorMemoryAllocation ? LB_ERR_OOM : LB_ERR_CUDA;
+  return status_of(cudaGetLastError());
 }
 
 }  // namespace
@@ -740,7 +747,7 @@ int lb_analysis_msd(const double* traj, int T, int N, int max_lag, int i0, int i
     nc = nc < 15 ? nc : 15;
     size_t smem = ((size_t)T * 9 + 1) * sizeof(double);
     smem = smem < kOnePerSM ? kOnePerSM : smem;
-    return launch_cluster(k_msd_staged, dim3(nc * kMsdCluster), kMsdThreads, kMsdCluster, smem,
+    return launch_cluster(k_msd_staged, dim3(nc), kMsdThreads, kMsdCluster, smem,
                           (cudaStream_t)stream, traj, T, N, i0, i1, out, max_lag + 1, nc);
   }
   k_msd<<<max_lag + 1, kThreads, 0, (cudaStream_t)stream>>>(traj, T, N, i0, i1, out, max_lag + 1);
@@ -807,7 +814,7 @@ int lb_analysis_static_sk(const double* traj, int T, int N, const double* k, int
     return launch_status();
   }
   const size_t apart = c.size > 1 ? kOnePerSM : 0;
-  const dim3 grid((nk + kg - 1) / kg * c.parts * c.size);
+  const dim3 grid((nk + kg - 1) / kg * c.parts);
   if (c.parts > 1 && cudaMemsetAsync(S, 0, nk * sizeof(double), s) != cudaSuccess) return launch_status();
   if (kg == 1) return launch_cluster(k_static_sk<1>, grid, kThreads, c.size, apart, s, traj, T, N, k, nk, S, c.parts);
   if (kg == 2) return launch_cluster(k_static_sk<2>, grid, kThreads, c.size, apart, s, traj, T, N, k, nk, S, c.parts);
@@ -823,7 +830,7 @@ int lb_analysis_inverse_radius(const double* traj, int T, int N, double* out, vo
     return launch_cluster(k_inverse_radius, dim3(1), 2 * kThreads, 1, 0, s, traj, T, N, out);
   const int cs = cluster_for(pairs / 2, 2 * kThreads, 16);
   if (cudaMemsetAsync(out, 0, sizeof(double), s) != cudaSuccess) return launch_status();
-  return launch_cluster(k_inverse_radius, dim3(2 * cs), 2 * kThreads, cs, 0, s, traj, T, N, out);
+  return launch_cluster(k_inverse_radius, dim3(2), 2 * kThreads, cs, 0, s, traj, T, N, out);
 }
 
 int lb_analysis_dynamic_sk(const double* traj, int T, int N, const double* k, int nk, int max_lag,
@@ -850,7 +857,7 @@ int lb_analysis_dynamic_sk(const double* traj, int T, int N, const double* k, in
     k_dynamic_sk_few<<<dim3(nk, max_lag + 1), kThreads, 0, s>>>(traj, T, N, k, origin_stride, S, max_lag + 1);
     return launch_status();
   }
-  const dim3 grid((nk + kg - 1) / kg * cs, max_lag + 1);
+  const dim3 grid((nk + kg - 1) / kg, max_lag + 1);
   if (kg == 1) return launch_cluster(k_dynamic_sk<1>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
   if (kg == 2) return launch_cluster(k_dynamic_sk<2>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
   if (kg == 3) return launch_cluster(k_dynamic_sk<3>, grid, kThreads, cs, 0, s, traj, T, N, k, nk, origin_stride, S, max_lag + 1);
