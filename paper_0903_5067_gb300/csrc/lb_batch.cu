@@ -521,7 +521,6 @@ class BatchT final : public Batch {
         pd.cur_count = eng_[r]->pending_count(jj);
         pd.cur_mask = flags_[jj];
         pd.mark = 1;
-        pd.cap = eng_[r]->pending_capacity();
         pd.seg0 = (unsigned)segs;
       }
       segs += (q.nnodes + 31) >> kSegShift;

@@ -105,9 +105,9 @@ struct FluidK {
   unsigned long long plane;  // elements between population planes
   R rho0;
   R gs, gb;        // relaxation eigenvalues: shear modes 5..9, bulk mode 4 (kinetic modes: 0)
-  R cnoise[Q];     // sqrt(mu b_k (1 - gamma_k^2)), mode k's noise per sqrt(rho); 0 if silent
   // the same relaxation and noise in terms of the scaled moments a_k = m*_k / b_k used by the
-  // back-transform: a_k = am_k m_k + ae_k m_eq,k + ag_k sqrt(rho) g_k  (k = 4..18)
+  // back-transform: a_k = am_k m_k + ae_k m_eq,k + ag_k sqrt(rho) g_k  (k = 4..18; ag_k b_k = sqrt(mu b_k
+  // (1 - gamma_k^2)), 0 for a silent mode)
   R am[Q], ae[Q], ag[Q];
   // the same times w_2 = 1/36, the weight of the next-nearest velocities, which the forward
   // kernel's back-transform then needs no more multiplications for
@@ -202,7 +202,6 @@ struct PendK {
   R* apply_to;            // null, or FP32/FP64 populations the old list's corrections, not yet applied
                           // to them, are added to where they are cleared
   int mark;               // 1: mark the pulling nodes of this step's list (deferred steps)
-  int cap;
   unsigned long long plane;  // element stride between the 19 planes
   unsigned seg0;             // index of this box's first word in the mask arrays
 };
@@ -1228,12 +1227,8 @@ __device__ __forceinline__ void cluster_store(T* p, int rank, T v) {
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(d), "l"(__double_as_longlong(v)) : "memory");
 }
 
-// Barrier over the thread blocks of a cluster; release/acquire order every memory access
-// before it (shared, distributed shared and global) before every access after it.
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
+// The two halves of a barrier over the thread blocks of a cluster; release and acquire order every memory
+// access before it (shared, distributed shared and global) before every access after it.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 // an arrival that orders no memory access (a release waits for the thread's writes in flight)
 __device__ __forceinline__ void cluster_arrive_relaxed() {

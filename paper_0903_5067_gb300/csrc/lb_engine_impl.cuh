@@ -61,14 +61,6 @@ class EngineT final : public Engine {
 
   void initialise(const double* x0, const double* v0, cudaStream_t s) override {
     snap_valid_ = false;
-    {
-      const LbLaunch q = lb_launch(false);
-      if (q.stage_bytes > 48 * 1024)  // FP64: staged corrections of a 256-thread tile
-        for (int v = 0; v < 8; ++v)
-          cuda_check(cudaFuncSetAttribute(lb_kernel(v & 1, (v >> 1) & 1, v >> 2, pair_nodes()),
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q.stage_bytes),
-                     "LB kernel shared memory");
-    }
     if (sizeof(R) == 8 && !noise_tab_.radius) noise_tab_ = noise_tables(s);
     if (bead_smem() > 48 * 1024)
       cuda_check(allow_all_shared((const void*)bead_kernel()), "bead kernel shared memory");
@@ -1009,7 +1001,6 @@ class EngineT final : public Engine {
     Pd.cur_count = p_count_[c];
     Pd.cur_mask = masks_[c];
     Pd.mark = mark ? 1 : 0;
-    Pd.cap = cap_;
     Pd.seg0 = 0;
     return Pd;
   }
@@ -1095,6 +1086,7 @@ class EngineT final : public Engine {
       lb_row_shape(q);
       if (waiting) q.grd.z += 1;  // the plane of waiting blocks
     }
+    static_assert(256 / 32 * WarpStage<R>::kBytes <= 48 * 1024, "more needs the opt-in to shared memory");
     q.stage_bytes = (size_t)(q.blk.x / 32) * WarpStage<R>::kBytes;
     return q;
   }
@@ -1191,7 +1183,6 @@ class EngineT final : public Engine {
       const double bk = norm36(k) / 36.0;
       const bool on = noise && k >= 4 && (k <= 9 || !c.stress_only);
       const double cn = on ? sqrt(mu * bk * (1.0 - g * g)) : 0.0;
-      P.cnoise[k] = (R)cn;
       P.am[k] = (R)(g / bk);
       P.ae[k] = (R)((1.0 - g) / bk);
       P.ag[k] = (R)(cn / bk);
