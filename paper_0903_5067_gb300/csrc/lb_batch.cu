@@ -79,7 +79,7 @@ struct BatchLB {
 // step's corrections to what it pulls (replicas without a chain have no correction field and
 // are never marked); the pull is issued before the mark is known, and one copy of the
 // collision follows, as in lb_node.  Coordinates come from the slot by two multiply-highs.
-template <class S, class R, bool DEV, bool NOISE>
+template <class S, class R, bool DEV, bool NOISE, bool PERSIST>
 __device__ __forceinline__ void batch_tile(const BatchLB<S, R>& B, const int r, const unsigned long long tile,
                                            const int parity, const uint32_t step, unsigned char* dsm) {
   const unsigned T = blockDim.x;
@@ -101,7 +101,7 @@ __device__ __forceinline__ void batch_tile(const BatchLB<S, R>& B, const int r, 
     const unsigned mw = corr ? B.mask[pslot][rp.seg0 + (node >> kSegShift)] >> (node & 31u) : 0u;
     R n0[Q], n1[Q];
     lb_pull2<S, R, unsigned>(rp.pop[parity], L, pl, x0, y, z, n0, n1);
-    add_corrections<R, true>(rp.p_dense[pslot], rp.plane, L, node, mw, part, dsm, n0, n1);
+    add_corrections<R, true, PERSIST>(rp.p_dense[pslot], rp.plane, L, node, mw, part, dsm, n0, n1);
     lb_collide2_store<S, R, DEV, NOISE, unsigned>(n0, n1, rp.pop[parity ^ 1], B.P, pl, B.rk[r], rp.nonpos, step,
                                                   node);
   } else {
@@ -109,7 +109,7 @@ __device__ __forceinline__ void batch_tile(const BatchLB<S, R>& B, const int r, 
     const unsigned mw = corr ? B.mask[pslot][rp.seg0 + (node >> kSegShift)] >> (node & 31u) : 0u;
     R n[Q];
     lb_pull<S, R, unsigned>(rp.pop[parity], L, pl, xs, y, z, n);
-    add_corrections<R, false>(rp.p_dense[pslot], rp.plane, L, node, mw, part, dsm, n, n);
+    add_corrections<R, false, PERSIST>(rp.p_dense[pslot], rp.plane, L, node, mw, part, dsm, n, n);
     lb_collide_store<S, R, DEV, NOISE, unsigned>(n, rp.pop[parity ^ 1], B.P, pl, B.rk[r], rp.nonpos, step, node);
   }
 }
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_batch_lb(const 
       if (B.rep[mid].tile0 <= tile) lo = mid;
       else hi = mid - 1;
     }
-    batch_tile<S, R, DEV, NOISE>(B, lo, tile, parity, step, dsm);
+    batch_tile<S, R, DEV, NOISE, PERSIST>(B, lo, tile, parity, step, dsm);
     return;
   }
   __shared__ unsigned long long s_next;
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 2 : 1) k_batch_lb(const 
     const unsigned long long t_end = cur + kChunk < B.total_tiles ? cur + kChunk : B.total_tiles;
     for (unsigned long long tile = cur; tile < t_end; ++tile) {
       while (r + 1 < B.nrep && B.rep[r + 1].tile0 <= tile) ++r;  // uniform
-      batch_tile<S, R, DEV, NOISE>(B, r, tile, parity, step, dsm);
+      batch_tile<S, R, DEV, NOISE, PERSIST>(B, r, tile, parity, step, dsm);
       __syncwarp();
     }
     __syncthreads();
@@ -428,7 +428,10 @@ class BatchT final : public Batch {
   // 64 replicas of L = 33 142, 96 us, 100 of L = 26 134, 90, 300 of L = 12, N = 64 with two substeps 122,
   // 110), and a few large boxes have the room for 32 (3 of L = 100, N = 128, on 1, 2 and 4 blocks: 164, 76,
   // 72; N = 64 on 1 and 2: 80, 71).  In FP64 the LB kernel leaves the time (100 of L = 12, N = 64 with two
-  // substeps on 1 and 2: 241, 274).
+  // substeps on 1 and 2: 241, 274).  The LB kernel's shape has no say: the blocks set the order in which a
+  // bead's forces are added, and the results do not depend on the shape.  (Beside persistent LB blocks
+  // one bead block would do better: 16 replicas of L = 24, N = 16 with four of 128 threads per SM 21.4 us on
+  // 4, 17.5 on one; a block per tile takes 13.3.)
   int bead_cluster() const {
     const int R_ = (int)eng_.size(), longest = longest_chain();
     const int places = sizeof(R) == 4 ? longest * eng_[0]->config().substeps : 0;

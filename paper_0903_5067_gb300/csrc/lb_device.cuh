@@ -718,8 +718,10 @@ __device__ __noinline__ void stage_marked_call(const float* __restrict__ corr, u
 // nodes of a row, and a kernel whose blocks are all resident ends with its slowest warp: with
 // every marked thread staging its own nodes one after the other, 19 rounds and one flight each,
 // the step at L = 64, N = 64 (FP32) took 11.4 us, of which 3.2 went with the corrections left out;
-// then 8.6 (7.4 without a chain); 7.8 with blocks of 128 threads (7.15).
-template <class R, bool PAIR>
+// then 8.6 (7.4 without a chain); 7.8 with blocks of 128 threads (7.15).  INLINE: not as a call in
+// single precision either (persistent blocks, in whose loop over tiles the call made the main path
+// spill: 64 replicas of L = 32 on one block of 128 threads per SM 185 us per step, inlined 175).
+template <class R, bool PAIR, bool INLINE = false>
 __device__ __forceinline__ void add_corrections(const R* __restrict__ corr, unsigned long long plane, unsigned L,
                                                 unsigned node, unsigned mw, unsigned part, unsigned char* smem,
                                                 R* n0, R* n1) {
@@ -727,7 +729,7 @@ __device__ __forceinline__ void add_corrections(const R* __restrict__ corr, unsi
   constexpr unsigned kNodes = WarpStage<R>::kNodes;
 #pragma unroll 1
   for (unsigned base = 0;; base += kNodes) {
-    if constexpr (sizeof(R) == 4)
+    if constexpr (sizeof(R) == 4 && !INLINE)
       stage_marked_call<PAIR>(corr, plane, L, node, mw, part, base, smem);
     else
       stage_marked<R, PAIR>(corr, plane, L, node, mw, part, base, smem);
