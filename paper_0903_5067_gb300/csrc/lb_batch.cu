@@ -849,7 +849,7 @@ int lb_batch_get_populations(lb_batch* bt, int r, double* out, size_t cap) {
   if (cap < 19 * L * L * L) return LB_ERR_ARG;
   return bguard([&] {
     bmaterialise(bt);
-    bt->b->replica(r).get_populations(out, bt->stream);
+    bt->b->replica(r).get_populations(out, bt->stream, false);
     return (int)LB_OK;
   });
 }
@@ -868,7 +868,7 @@ int lb_batch_get_observables(lb_batch* bt, int r, double* out, size_t cap) {
   if (!bt || !out || r < 0 || r >= (int)bt->cfgs.size() || cap < LB_NOBS) return LB_ERR_ARG;
   return bguard([&] {
     bmaterialise(bt);
-    bt->b->replica(r).observables(out, bt->step, 0, bt->stream);
+    bt->b->replica(r).observables(out, bt->step, 0, bt->stream, false);
     return (int)LB_OK;
   });
 }

@@ -61,8 +61,9 @@ class Engine {
   // n such steps k .. k + n - 1, as CUDA graphs of several steps where there are enough
   virtual void steps_deferred(uint32_t k, int64_t n, cudaStream_t s) = 0;
   virtual void flush(cudaStream_t s) = 0;
-  // the synchronising read-backs return the device status word as of their synchronisation
-  virtual unsigned get_populations(double* out, cudaStream_t s) = 0;
+  // the synchronising read-backs return the device status word as of their synchronisation (0 where
+  // it is not asked for: reading it takes 7 us)
+  virtual unsigned get_populations(double* out, cudaStream_t s, bool status = true) = 0;
   virtual void set_populations(const double* in, cudaStream_t s) = 0;
   virtual unsigned get_beads(double* x, double* v, cudaStream_t s) = 0;
   // the same read-back enqueued on s without waiting (x, v: host memory that stays valid
@@ -77,7 +78,7 @@ class Engine {
   // wait for read-backs in flight on the engine's own stream
   virtual void drain() = 0;
   // (out null: enqueued only, returns 0)
-  virtual unsigned observables(double* out, int64_t step, int accumulate, cudaStream_t s) = 0;
+  virtual unsigned observables(double* out, int64_t step, int accumulate, cudaStream_t s, bool status = true) = 0;
   virtual void reset_reference(cudaStream_t s) = 0;
   // write the current unwrapped bead positions (3N doubles) to device memory
   virtual void record_frame(double* dst, cudaStream_t s) = 0;

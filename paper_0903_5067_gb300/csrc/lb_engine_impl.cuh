@@ -591,7 +591,7 @@ class EngineT final : public Engine {
   // allocation) is written or read by one conversion kernel over all 19 planes, with no
   // staging copy; other host memory goes through the second population buffer in chunks of
   // as many FP64 planes as it holds, one conversion kernel and one copy per chunk.
-  unsigned get_populations(double* out, cudaStream_t s) override {
+  unsigned get_populations(double* out, cudaStream_t s, bool status = true) override {
     flush(s);
     double* direct = static_cast<double*>(device_view(out, (size_t)Q * nnodes_ * sizeof(double)));
     if (direct) {
@@ -609,7 +609,7 @@ class EngineT final : public Engine {
                    "download planes");
       }
     }
-    return read_status(s);
+    return finish_read(s, status);
   }
 
   void set_populations(const double* in, cudaStream_t s) override {
@@ -720,7 +720,7 @@ class EngineT final : public Engine {
     }
   }
 
-  unsigned observables(double* out, int64_t step, int accumulate, cudaStream_t s) override {
+  unsigned observables(double* out, int64_t step, int accumulate, cudaStream_t s, bool status = true) override {
     flush(s);
     ObsK<R> O = obs(step, accumulate);
     if (!accumulate) {
@@ -732,7 +732,7 @@ class EngineT final : public Engine {
     cuda_check(cudaGetLastError(), "observables");
     if (!out) return 0;
     cuda_check(cudaMemcpyAsync(out, obs_, kNObs * sizeof(double), cudaMemcpyDeviceToHost, s), "dl obs");
-    return read_status(s);
+    return finish_read(s, status);
   }
 
   void reset_reference(cudaStream_t s) override {
@@ -762,6 +762,13 @@ class EngineT final : public Engine {
     cuda_check(cudaStreamSynchronize(s), "sync debug");
     if (x_stored)
       for (size_t t = 0; t < xs.size(); ++t) x_stored[t] = (double)xs[t];
+  }
+
+  // waits for s; the status word if it is asked for
+  unsigned finish_read(cudaStream_t s, bool status) {
+    if (status) return read_status(s);
+    cuda_check(cudaStreamSynchronize(s), "sync read-back");
+    return 0;
   }
 
   // waits for s
