@@ -771,12 +771,13 @@ int lb_analysis_rouse_correlation(const double* X, int T, int P, int max_lag, do
   // What the two forms take, in us.  The staged form walks all origins for 32 lags at a time, however few
   // are asked for, in blocks of kCorrLags lags; the form with a block per lag and mode takes its share
   // of each, more where the modes of a frame lie in few of the cache's sets.  Measured, staged and
-  // plain (and by this): T = 1000, P = 127, 501 lags 282, 642; P = 128, 1 lag 31, 8.5 (29, 8), 12 lags 31, 39
-  // (29, 34); P = 13, 281 lags 54, 47 (54, 50); T = 3100, P = 300, 1 lag 158, 17 (154, 14), 16 lags
-  // 158, 169 (154, 149); T = 100, P = 128, 2 lags 7.8, 6.4 (7, 6.4), 4 lags 7.9, 8.4 (7, 7.7).
+  // plain (and by this): T = 1000, P = 127, 501 lags 282, 642; P = 128, 1 lag 31, 8.5 (30, 8), 12 lags 31, 39
+  // (30, 40); P = 13, 281 lags 54, 47 (55, 50); T = 3100, P = 300, 1 lag 158, 17 (156, 14), 16 lags
+  // 158, 169 (156, 149); T = 100, P = 128, 2 lags 7.8, 6.4 (8, 6.5), P = 32, 11 lags 7.7, 6.2 (8, 7.0).
   const double lags = max_lag + 1.0, blocks = P * ceil(lags / kCorrLags);
-  const double staged = 4.5 + (blocks <= 152 ? 1.0 : fmax(1.4, blocks / 152)) * 0.0246 * T * (lags > 32 ? 2 : 1);
-  const double plain = 5.0 + P * lags * (0.0038 + 8.5e-6 * T * (P % 16 == 0 ? 1.8 : (P % 8 == 0 ? 1.3 : 1.0)));
+  const double waves = blocks <= 152 ? 1.0 : (blocks <= 304 ? fmax(1.4, blocks / 152) : ceil(blocks / 152));
+  const double staged = 5.5 + waves * 0.0246 * T * (lags > 32 ? 2 : 1);
+  const double plain = 5.0 + P * lags * (0.0038 + 8.5e-6 * T * (P % 16 == 0 ? 2.2 : (P % 8 == 0 ? 1.3 : 1.0)));
   if (T <= kCorrFrames && plain > 0.95 * staged) {
     const size_t smem = 3 * (size_t)T * sizeof(double);
     if (!allow_shared(k_rouse_corr_staged, smem)) return LB_ERR_CUDA;
