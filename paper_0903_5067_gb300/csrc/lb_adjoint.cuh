@@ -250,11 +250,6 @@ __host__ __device__ inline size_t adj_prep_smem(int N) {
   return 6 * (size_t)N * sizeof(R) + 32 + M * 8 + 8 * (size_t)N * 4 + 64;
 }
 
-// The forward recomputation of the bead step for the steps step_arg + j, j = blockIdx.x, of a segment,
-// a block per step: it depends on no other step and on no adjoint, so it is off the chain of
-// reverse steps (of whose 15 us per step, N = 16, it took 5 as the first part of k_adj_bead).
-// The state of step j lies j * state_stride bytes behind `state` and the arrays of C, its region
-// j * prep_stride bytes behind `prep`.
 // A checkpoint of the forward pass: the populations (16-byte words) and the bead arrays behind them
 // (4-byte words) to checkpoint (*d_step - k0) / K of those that lie `stride` bytes apart from `to` on
 __global__ static void k_adj_checkpoint(const int4* __restrict__ pops, size_t npops, const int* __restrict__ beads, int nbeads,
@@ -275,6 +270,11 @@ __global__ void k_adj_seed(const double* __restrict__ x0, const double* __restri
     xbar[t] = (R)(2.0 * (x[t] - x0[t]));
 }
 
+// The forward recomputation of the bead step for the steps step_arg + j, j = blockIdx.x, of a segment,
+// a block per step: it depends on no other step and on no adjoint, so it is off the chain of
+// reverse steps (of whose 15 us per step, N = 16, it took 5 as the first part of k_adj_bead).
+// The state of step j lies j * state_stride bytes behind `state` and the arrays of C, its region
+// j * prep_stride bytes behind `prep`.
 template <class S, class R, bool DEV>
 __global__ void __launch_bounds__(512) k_adj_prep(const S* __restrict__ state, const FluidK<R> P, const ChainK<R> C,
                                                    unsigned char* prep, int prep_stride, size_t state_stride,

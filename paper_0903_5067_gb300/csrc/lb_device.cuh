@@ -6,12 +6,12 @@
 // (post-collision populations of the previous step, "pull" storage) and writes B.
 //
 // One step = k_bead_step (one thread block, or a cluster of up to 8: velocity Verlet,
-// FENE/WCA, interpolation, friction + noise, spreading -> sparse list of per-node population
-// corrections), k_lb_step (every node: pull-stream, moments, relaxation + noise,
-// back-transform) and the force corrections, added to B by k_apply_pending or, kept pending,
-// by the next step's kernels where they read.  The bead kernel and the LB kernel read only A,
-// so they are independent; the correction is additive on the post-collision populations
-// because the collision conserves the density and momentum it depends on.
+// FENE/WCA, interpolation, friction + noise, spreading -> population corrections at the nodes around
+// the beads, in a field of the populations' layout, with a list of the nodes), k_lb_step (every
+// node: pull-stream, moments, relaxation + noise, back-transform) and the force corrections, added to
+// B by k_apply_pending or, kept pending, by the next step's kernels where they read.  The bead kernel
+// and the LB kernel read only A, so they are independent; the correction is additive on the
+// post-collision populations because the collision conserves the density and momentum it depends on.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -1354,7 +1354,8 @@ __device__ __forceinline__ R corner_weight(const R* fr, int c) {
 // grouping the corners by a hash table with two scans on block 0 and two cluster barriers.
 // Kernel alone under ncu, before and after: N = 32 with two substeps 25 -> 11 us, N = 64 19 -> 11,
 // N = 16 14 -> 9 (FP32), N = 8 in FP64 50 -> 26.  Inside (clock stamps, N = 16): noise 0.6 us
-// (before the wait), drift 0.6, gathers and forces 1.2, friction 0.4, barrier 0.6, corrections 2.2:
+// (before the wait), drift 0.6, gathers and forces 1.2, friction 0.4, barrier 0.6, corrections 2.2
+// (some 0.3 less since their marks are unrolled):
 // single warps issuing dependent instructions, no longer memory.  (Spreading gathers and
 // corrections over all warps by population, which multiplies their index arithmetic, came out
 // slower: 7.1 against 6.9 us per step at L = 32, N = 16; 31 against 26 for 64 replicas of L = 15.)
