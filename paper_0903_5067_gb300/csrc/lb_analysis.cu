@@ -206,8 +206,8 @@ __global__ void __launch_bounds__(kMsdThreads) k_msd_staged(const double* __rest
   }
 }
 
-// Longer runs: one block per lag, origins t0 strided over the threads, the centres of both frames
-// formed by each thread
+// Longer runs, and short chains with few lags: one block per lag, origins t0 strided over the threads,
+// the centres of both frames formed by each thread
 __global__ void __launch_bounds__(kThreads) k_msd(const double* __restrict__ traj, int T, int N, int i0, int i1,
                                                   double* __restrict__ out, int nlag) {
   __shared__ double sh[3][kThreads];
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kThreads) k_rouse_corr_staged(const double* __
   }
 }
 
-// Longer runs: one block per (p, lag)
+// Longer runs, few lags or few modes: one block per (p, lag)
 __global__ void __launch_bounds__(kThreads) k_rouse_corr(const double* __restrict__ X, int T, int P,
                                                          double* __restrict__ c, int nlag) {
   __shared__ double sh[1][kThreads];
